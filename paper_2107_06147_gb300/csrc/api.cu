@@ -14,6 +14,7 @@
 #include "api_internal.h"
 #include "eigen.h"
 #include "fused_launch.cuh"
+#include "fused_plan.h"
 #include "plain.cuh"
 #include "qtraj.h"
 
@@ -101,7 +102,8 @@ struct qtraj_ctx {
     qtraj_params p{};
     int device = 0, sm_count = 0;
     // read-only tables
-    void *W = nullptr, *WL = nullptr, *KT = nullptr, *sinpre = nullptr, *statV = nullptr, *statV2 = nullptr;
+    void *W = nullptr, *WL = nullptr, *KT = nullptr, *sinpre = nullptr, *statP = nullptr;   // plain, FP32 KSU
+    void *KF = nullptr, *TA = nullptr, *TM = nullptr, *TI = nullptr, *TS = nullptr, *statV = nullptr, *statV2 = nullptr;   // fused
     double *eig = nullptr;
     double *ic = nullptr, *ov0 = nullptr;
     int *ov0_zero = nullptr, *spec_l = nullptr, *spec_color = nullptr;
@@ -218,27 +220,38 @@ Layout layout(const qtraj_ctx *c, int n)
 }
 
 // the static part of the space kernel for every (colour, l < LTAB, j), rows [colour][l][j]:
-// exp(-i V dt/2) (s1) and exp(-i V dt) (s2), V = coul_c / r + l(l+1) / (M r^2) at r = j dr, in FP64
-// (entry j = 0 is zero: u(0) = 0).  Built on the device: 2 x 2 x LTAB x N phases.
+// exp(-i V span dt/2), V = coul_c / r + l(l+1) / (M r^2) at r = j dr, in FP64 (entry j = 0 is zero:
+// u(0) = 0).  span 1 (half step) or 2.  R > 0: the entries of a row in the fused kernel's order
+// (fused_plan.h), else in natural order.  Built on the device: 2 x LTAB x N phases.
 template <typename T>
-__global__ void stat_rows(typename Prec<T>::S *s1, typename Prec<T>::S *s2, int N, double dr, double M, double dt,
-                          double coul0, double coul1)
+__global__ void stat_rows(typename Prec<T>::S *out, int N, double dr, double M, double dt, double coul0, double coul1,
+                          double span, int R, int PM, int G)
 {
     const size_t n = (size_t)2 * LTAB * N;
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        const int j = (int)(i % (size_t)N), row = (int)(i / (size_t)N);
+        int j = (int)(i % (size_t)N), row = (int)(i / (size_t)N);
+        if (R > 0) {
+            int g, e;
+            plan_entry(j, sizeof(T) == 4, R, G, g, e);
+            j = plan_j(g, e, R, PM, G);
+        }
         const int col = row / LTAB, l = row % LTAB;
-        double c1 = 0.0, sn1 = 0.0, c2 = 0.0, sn2 = 0.0;
+        double co = 0.0, sn = 0.0;
         if (j > 0) {
             const double r = j * dr;
             const double V = (col ? coul1 : coul0) / r + (double)l * (l + 1) / (M * r * r);
-            const double ph = -V * dt * 0.5;
-            sincos(ph, &sn1, &c1);
-            sincos(2.0 * ph, &sn2, &c2);
+            sincos(span * (-V * dt * 0.5), &sn, &co);
         }
-        s1[i] = Prec<T>::make_s(c1, sn1);
-        s2[i] = Prec<T>::make_s(c2, sn2);
+        out[i] = Prec<T>::make_s(co, sn);
     }
+}
+
+// host array -> new device array
+template <typename V> qtraj_status upload(void **out, const std::vector<V> &v)
+{
+    CK(cudaMalloc(out, sizeof(V) * v.size()));
+    CK(cudaMemcpy(*out, v.data(), sizeof(V) * v.size(), cudaMemcpyHostToDevice));
+    return QTRAJ_OK;
 }
 
 template <typename T> qtraj_status build_tables(qtraj_ctx *c)
@@ -246,19 +259,13 @@ template <typename T> qtraj_status build_tables(qtraj_ctx *c)
     using PC = typename Prec<T>::C;
     using PR = typename Prec<T>::Rl;
     const int N = c->N;
-    std::vector<PC> W(N), KT(N);
-    std::vector<PR> sp(N);
-    for (int t = 0; t < N; ++t) {
-        const double a = -2.0 * PI * (double)t / N;
-        W[t] = Prec<T>::make(std::cos(a), std::sin(a));
-        sp[t] = Prec<T>::make_r(std::sin(PI * (double)t / N));
-    }
+    std::vector<std::pair<double, double>> kt(N);   // exp(-i T_kin(p_k) dt)
     for (int k = 0; k < N; ++k) {
         const double pk = PI * k / c->L;
         double Tk = pk * pk / c->M;
         if (c->p.deriv_type == 1) Tk = 2.0 * (1.0 - std::cos(pk * c->dr)) / (c->M * c->dr * c->dr);
         const double ph = -Tk * c->dt;
-        KT[k] = Prec<T>::make(std::cos(ph) * 2.0 / N, std::sin(ph) * 2.0 / N);
+        kt[k] = {std::cos(ph), std::sin(ph)};
     }
     const double Nc = c->p.Nc, CF = (Nc * Nc - 1.0) / (2.0 * Nc);
     double coul[2] = {-CF * c->p.alpha_s, c->p.alpha_s / (2.0 * Nc)};
@@ -325,35 +332,84 @@ template <typename T> qtraj_status build_tables(qtraj_ctx *c)
         CK(cudaMalloc(&c->phi_tab, sizeof(T) * tab.size()));
         CK(cudaMemcpy(c->phi_tab, tab.data(), sizeof(T) * tab.size(), cudaMemcpyHostToDevice));
     }
-    // last-pass twiddles of the fused kernel, W^(m g) for m < R, g < G = N/(2R), one compact section
-    // [R][G] (N/2 entries) per radix R = 16, 8, 4 at offsets 0, N/2, N: a kernel reads the section of
-    // its own radix, and the threads of a warp read consecutive entries
-    std::vector<PC> WL((size_t)3 * (N / 2));
-    for (int sec = 0; sec < 3; ++sec) {
-        const int R = 16 >> sec, G = N / (2 * R);
-        for (int m = 0; m < R; ++m)
-            for (int g = 0; g < G; ++g) WL[(size_t)sec * (N / 2) + (size_t)m * G + g] = W[(size_t)m * g];
-    }
-    CK(cudaMalloc(&c->WL, sizeof(PC) * WL.size()));
-    CK(cudaMemcpy(c->WL, WL.data(), sizeof(PC) * WL.size(), cudaMemcpyHostToDevice));
-    CK(cudaMalloc(&c->W, sizeof(PC) * N));
-    CK(cudaMalloc(&c->KT, sizeof(PC) * N));
-    CK(cudaMalloc(&c->sinpre, sizeof(PR) * N));
+    // the forms' own tables: the plain form's in natural order, the fused kernel's in its threads' order
+    // (a plain context needs the latter for the vacuum evolution of its initial states)
     using PS = typename Prec<T>::S;
     const size_t nstat = (size_t)2 * LTAB * N;
-    if (cudaMalloc(&c->statV, sizeof(PS) * nstat) != cudaSuccess ||
-        cudaMalloc(&c->statV2, sizeof(PS) * nstat) != cudaSuccess) {
-        cudaGetLastError();
-        return fail(QTRAJ_ENOMEM, "cudaMalloc of the static space-kernel tables (%zu bytes)", 2 * sizeof(PS) * nstat);
+    const bool plain = c->p.form == QTRAJ_PLAIN, fused = !plain || c->p.t_vacuum > 0;
+    const bool ksu32 = c->p.potential == 1 && sizeof(T) == 4;   // its own kernel (fused_ksu32.cuh)
+    const Plan p = make_plan(N, sizeof(T) == 8, c->p.potential == 1 ? 0 : c->p.variant);
+    qtraj_status st = QTRAJ_OK;
+    if (plain || ksu32) {
+        std::vector<PC> W(N), KT(N);
+        std::vector<PR> sp(N);
+        for (int t = 0; t < N; ++t) {
+            const double a = -2.0 * PI * (double)t / N;
+            W[t] = Prec<T>::make(std::cos(a), std::sin(a));
+            sp[t] = Prec<T>::make_r(std::sin(PI * (double)t / N));
+            KT[t] = Prec<T>::make(kt[t].first * 2.0 / N, kt[t].second * 2.0 / N);
+        }
+        if ((st = upload(&c->W, W)) != QTRAJ_OK || (st = upload(&c->KT, KT)) != QTRAJ_OK ||
+            (st = upload(&c->sinpre, sp)) != QTRAJ_OK)
+            return st;
+        if (ksu32) {
+            // last-pass twiddles W^(m g) for m < R, g < G = N/(2R), one compact section [R][G] (N/2 entries)
+            // per radix R = 16, 8, 4: the threads of a warp read consecutive entries
+            std::vector<PC> WL((size_t)3 * (N / 2));
+            for (int sec = 0; sec < 3; ++sec) {
+                const int R = 16 >> sec, G = N / (2 * R);
+                for (int m = 0; m < R; ++m)
+                    for (int g = 0; g < G; ++g) WL[(size_t)sec * (N / 2) + (size_t)m * G + g] = W[(size_t)m * g];
+            }
+            if ((st = upload(&c->WL, WL)) != QTRAJ_OK) return st;
+        }
     }
-    CK(cudaMemcpy(c->W, W.data(), sizeof(PC) * N, cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(c->KT, KT.data(), sizeof(PC) * N, cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(c->sinpre, sp.data(), sizeof(PR) * N, cudaMemcpyHostToDevice));
+    if (fused && !ksu32) {
+        auto root = [&](long k, long n) {   // exp(-2 pi i k / n)
+            const double a = -2.0 * PI * (double)(k % n) / (double)n;
+            return Prec<T>::make(std::cos(a), std::sin(a));
+        };
+        std::vector<PC> KF(N), TA((size_t)p.R / 2 * p.NS), TM(p.S), TI((size_t)p.M1 * p.M2), TS(p.R / 2);
+        for (int i = 0; i < N; ++i) {
+            int g, e;
+            plan_entry(i, false, p.R, p.G, g, e);
+            const int j = plan_j(g, e, p.R, p.M, p.G);
+            const double f = j == 0 ? 0.0 : -0.5 / N;   // two transforms X = -2i S, and the inverse's 2/N
+            KF[i] = Prec<T>::make(kt[j].first * f, kt[j].second * f);
+        }
+        for (int s = 0; s < p.NS; ++s) {
+            int lo, hi;
+            slot_points(s, p.R, p.M, lo, hi);
+            for (int k = 1; k <= p.R / 2; ++k) TA[(size_t)(k - 1) * p.NS + s] = root((long)lo * k, 2L * N);
+        }
+        for (int b1 = 0; b1 < p.R; ++b1)
+            for (int q1 = 0; q1 < p.M; ++q1) TM[p.tw_last ? b1 * p.M + q1 : q1 * p.R + b1] = root((long)b1 * q1, p.S);
+        for (int k1 = 0; k1 < p.M1; ++k1)
+            for (int m2 = 0; m2 < p.M2; ++m2) TI[(size_t)k1 * p.M2 + m2] = root((long)m2 * k1, p.M);
+        for (int k = 1; k < p.R / 2; ++k) TS[k] = Prec<T>::make(0.5 / std::sin(PI * k / p.R), 0.5 / std::tan(PI * k / p.R));
+        if ((st = upload(&c->KF, KF)) != QTRAJ_OK || (st = upload(&c->TA, TA)) != QTRAJ_OK ||
+            (st = upload(&c->TM, TM)) != QTRAJ_OK || (st = upload(&c->TI, TI)) != QTRAJ_OK ||
+            (st = upload(&c->TS, TS)) != QTRAJ_OK)
+            return st;
+    }
+    const int ntab = (plain ? 1 : 0) + (fused ? 2 : 0);
+    if ((plain && cudaMalloc(&c->statP, sizeof(PS) * nstat) != cudaSuccess) ||
+        (fused && (cudaMalloc(&c->statV, sizeof(PS) * nstat) != cudaSuccess ||
+                   cudaMalloc(&c->statV2, sizeof(PS) * nstat) != cudaSuccess))) {
+        cudaGetLastError();
+        return fail(QTRAJ_ENOMEM, "cudaMalloc of the static space-kernel tables (%zu bytes)", ntab * sizeof(PS) * nstat);
+    }
     // a private non-blocking stream: building a context waits for nothing else on the device
     cudaStream_t s = nullptr;
     CK(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
     const int blocks = (int)std::min<size_t>((nstat + 255) / 256, 4096);
-    stat_rows<T><<<blocks, 256, 0, s>>>((PS *)c->statV, (PS *)c->statV2, N, c->dr, c->M, c->dt, coul[0], coul[1]);
+    auto rows = [&](void *out, double span, int R) {
+        if (out)
+            stat_rows<T><<<blocks, 256, 0, s>>>((PS *)out, N, c->dr, c->M, c->dt, coul[0], coul[1], span, R, p.M, p.G);
+    };
+    rows(c->statP, 1.0, 0);
+    rows(c->statV, 1.0, ksu32 ? 0 : p.R);
+    rows(c->statV2, 2.0, ksu32 ? 0 : p.R);
     cudaError_t e = cudaGetLastError();
     const cudaError_t e2 = cudaStreamSynchronize(s);
     if (e == cudaSuccess) e = e2;
@@ -370,6 +426,12 @@ template <typename T> Tables<T> tables(const qtraj_ctx *c)
     t.WL = (const PC *)c->WL;
     t.KT = (const PC *)c->KT;
     t.sinpre = (const typename Prec<T>::Rl *)c->sinpre;
+    t.statP = (const typename Prec<T>::S *)c->statP;
+    t.KF = (const PC *)c->KF;
+    t.TA = (const PC *)c->TA;
+    t.TM = (const PC *)c->TM;
+    t.TI = (const PC *)c->TI;
+    t.TS = (const PC *)c->TS;
     t.statV = (const typename Prec<T>::S *)c->statV;
     t.statV2 = (const typename Prec<T>::S *)c->statV2;
     t.eig = c->eig;
@@ -713,6 +775,12 @@ void qtraj_destroy(qtraj_ctx *c)
     free_ptr(c->WL);
     free_ptr(c->KT);
     free_ptr(c->sinpre);
+    free_ptr(c->statP);
+    free_ptr(c->KF);
+    free_ptr(c->TA);
+    free_ptr(c->TM);
+    free_ptr(c->TI);
+    free_ptr(c->TS);
     free_ptr(c->statV);
     free_ptr(c->statV2);
     free_ptr(c->phi_tab);

@@ -1,9 +1,9 @@
 // fused.cuh -- the fused persistent trajectory kernel.
 //
 // One CTA evolves one trajectory at a time, through every step of its medium, and then fetches the
-// next trajectory from a global work counter.  The wave function never leaves the SM: between the
-// sine transforms it lives in one shared-memory buffer of N + N/R complex values; during a transform
-// each thread holds 2R values in registers.
+// next trajectory from a global work counter.  The wave function never leaves the SM: between the sine
+// transforms it lives in registers (N/G values a thread), and shared memory only exchanges values
+// between the threads inside a transform.
 //
 // One step (Sec. 3.3, steps 1-5) with T = T(tau_n) (Sec. 3.4, Bjorken):
 //   x <- K_V(n) x        K_V = exp(-i V_eff dt/2) = static(c, l, r) * exp((er + i ei) T^3 r^2)
@@ -17,48 +17,58 @@
 // jump, the start half-step is turned into the new colour's and l's afterwards (all these factors are
 // diagonal in r and commute with the jump's multiplication by r).
 //
-// The DST-I of the N-point complex vector f (f_0 = f_N = 0) is computed with one N-point complex FFT:
-//   y_j = sin(pi j/N)(f_j + f_{N-j}) + (f_j - f_{N-j})/2,   Y = FFT_N(y),
-//   S_{2k}   = (i/2)(Y_k - Y_{N-k}),
-//   S_{2k+1} = S_{2k-1} + (Y_k + Y_{N-k})/2,  S_{-1} = -S_1    (a prefix sum over k < N/2).
-// This equals the length-2N FFT of the odd extension (the paper's sine series with the wall at
-// r = L) at half its arithmetic and memory.  In shared memory S is kept as S_{2k} at [k] and S_{2k+1}
-// at [N/2 + k + k/R] (the padded "odd area").
-//
-// FFT: Stockham autosort with radices R (first pass), MID = N/R^2 in passes of <= 16, R (last).
-// Thread g of G = N/(2R) owns butterflies b1 = g, b2 = N/R - g (g = 0: 0 and N/(2R)) of the first
-// and last passes, i.e. the indices b + m N/R, m < R.  Those index sets are closed under j -> N - j,
-// so the pre- and post-processing, which pair j with N - j, stay inside a thread's registers.
-// Shared-memory addresses of the FFT passes are padded by one element every R.
+// The sine transform.  With X the length-2N FFT of the odd extension of x, X_k = -2i S_k, and both x and X
+// are odd: only half of every pass is independent, and only that half is computed and stored.  Indices
+// n = b + S m (m < R, S = 2N/R), k = kk + R q (kk < R):
+//   first pass   Z_b[kk] = DFT_R of x_{b + S m} over m, for one b of every pair +-b (mod S);
+//                A_kk[b] = W_2N^(b kk) Z_b[kk], and by the oddness A_{R-kk}[b] = -conj(W^(b kk))..., i.e.
+//                A_kk[-b] = -W_2N^(-b kk) Z_b[R-kk]: one b fills the sequences kk = 1 .. R/2-1 at b and -b;
+//   middle       FFT_S of each sequence over b = b1 + R m: DFT_M over m (in place), twiddle W_S^(b1 q1),
+//   last pass    DFT_R over b1 -> X_{kk + R q1 + S q2}, q2 < R.
+// The last pass leaves a thread with the points b + S q2, b = kk + R q1 -- the inputs of one first-pass
+// butterfly of the next transform.  So the kinetic and potential factors and the norm act on registers
+// between a last and a first pass, and a transform exchanges values through shared memory twice.
+// (A transform through one N-point FFT with sine pre- and post-processing, which this replaced, needed
+// four to five exchanges, a compensated prefix sum over the N/2 odd coefficients, and about 1.9 times the
+// instructions; its running sum also carried the FFT's rounding errors along k.)
+// The sequences kk = 0 (U, odd: U_{-q} = -U_q) and kk = R/2 (V, V_{-1-q} = -V_q) are half as long; they
+// share one FFT_S of their sum P, and P_q + P_{-q} = V_q - V_{q-1} gives V by a prefix sum of S/2 values
+// and U = P - V (split()).  The two sequences b = 0 and b = S/2 of the first pass (odd and half-odd in m)
+// share the butterfly of slot 0 the same way, separated in closed form (special_in, special_mid).
+// Which points a thread holds: fused_plan.h.
 #pragma once
 #include "fused_launch.cuh"
+#include "fused_plan.h"
 #include "qtraj_device.cuh"
 
 namespace qt {
 
-// V selects the launch variant (fused_launch.cuh); variants 2 and 3 use radix 8 for N >= 1024:
-// twice the threads per trajectory, half the registers per thread, one more FFT pass.
-
-template <int N, int V = 0> struct FusedPlan {
-    // radix 8 up to N = 2048 (passes 8, 16, 8 at N = 1024 and 8, 16, 2, 8 at 2048: +9% each over
-    // radix 16's 16, 4, 16 and 16, 8, 16, whose short middle passes and small CTAs cost more
-    // instructions per point), 16 above
-    static constexpr int R = (N <= 32) ? 4 : (N <= 2048) ? 8 : (V == 2 || V == 3 ? 8 : 16);
-    static constexpr int G = N / (2 * R);        // threads per trajectory
-    static constexpr int NR = N / R;             // stride of a first/last-pass butterfly
-    static constexpr int MID = N / (R * R);      // product of the middle radices
-    static constexpr int M1 = MID >= 16 ? 16 : MID;
-    static constexpr int M2 = MID / M1;          // 1, 2, 4, 8 or 16
-    static constexpr int BUF = N + N / R + 8;    // padded FFT extent; also holds the E/odd layout
-    // middle-pass twiddle tables in shared memory, row m holding W^(m k) for the k of every thread
-    // (tw1: [M1][R] of W_{R M1}; tw2: [M2][R M1] of W_{R M1 M2}), so that a warp reads consecutive
-    // entries.  (A flat table W^t read at t = m k with one pad entry every 8 met up to 7-way bank
-    // conflicts at odd m -- 44% of the step's shared-memory conflicts at N = 4096.)
-    static constexpr int TW1 = R * M1;
-    static constexpr int TW2 = M2 > 1 ? R * M1 * M2 : 0;
-    static_assert(N == R * M1 * M2 * R, "plan");
+// V selects the launch variant (fused_launch.cuh): 0, 1 the plan of the grid size with 512 or 640 resident
+// threads per SM, 2 and 3 the radix-8 plans with 768 and 1024; 4 and 6 the traced twins of 0 and 2, 5 the
+// KSU twin of 0.
+template <typename T, int N, int V = 0> struct FusedPlan {
+    static constexpr PlanDims D = plan_dims(N, sizeof(T) == 8, V == 2 || V == 3 || V == 6);
+    static constexpr int R = D.R, E = D.E, M1 = D.M1, M2 = D.M2;
+    static constexpr int H = R / 2;              // sequences
+    static constexpr int M = M1 * M2;            // length of the middle transform
+    static constexpr int S = R * M;              // length of a sequence
+    static constexpr int G = N / E;              // threads per trajectory
+    static constexpr int NS = E / R;             // slots per thread
+    static constexpr int NSLOT = N / R;
+    static constexpr bool TWL = plan_tw_last(D);
+    // Shared-memory address of position b of a sequence: b + b/R (one pad element every R), so that the
+    // stride-R accesses of the first and last passes are stride R+1 and conflict-free; the sequences are
+    // SEQ apart, with SEQ = M (mod 16) where several sequences share a half-warp (M < 16), so that their
+    // M-lane runs are adjacent modulo the banks.
+    static constexpr int SEQ0 = S + S / R;
+    static constexpr int SEQ = M < 16 ? SEQ0 + ((M - SEQ0) % 16 + 16) % 16 : SEQ0;
+    static constexpr int BUF = H * SEQ;
+    // butterflies a thread does in a middle pass, and the registers these take
+    static constexpr int PER1 = (N / M1 + G - 1) / G, PER2 = (N / M2 + G - 1) / G;
+    static constexpr int X0 = PER1 * M1 > E ? PER1 * M1 : E;
+    static constexpr int XN = M2 > 1 && PER2 * M2 > X0 ? PER2 * M2 : X0;
+    static_assert(N * 2 == R * R * M && G % R == 0 && M <= G && E % R == 0, "plan");
 };
-
 
 // ------------------------------------------------------------------------------------------------
 // accumulators: FP32 forms accumulate sums of squares with compensated (cascaded) summation and
@@ -105,48 +115,6 @@ template <> struct SqAcc<double> {
     __device__ __forceinline__ void add_w(cpx<double> a, double w) { v = fma(w, fma(a.x, a.x, a.y * a.y), v); }
     __device__ __forceinline__ void shfl_add(unsigned mask, int off, int w) { v += __shfl_xor_sync(mask, v, off, w); }
     __device__ __forceinline__ double value() const { return v; }
-};
-
-// compensated complex value for the scan's carries between threads.  Chunk totals use cascaded
-// summation (the TwoSum error terms are collected separately); carries between threads are
-// double-float additions.  The rounding of a chunk total is added to every later odd coefficient
-// (a step in k, energy growing with the number of coefficients after it): with plain FP32 chunk
-// totals the no-jump FP32 norm drifted by +7e-9 per step at N = 1024 (against < 5e-9 compensated),
-// so the 3% they would save at N = 4096 is not taken.
-template <typename T> struct Carry;
-template <> struct Carry<float> {
-    DF re{0.f, 0.f}, im{0.f, 0.f};
-    __device__ __forceinline__ void add(cpx<float> a)
-    {
-        const DF r = two_sum(re.hi, a.x), i = two_sum(im.hi, a.y);
-        re = DF{r.hi, re.lo + r.lo};
-        im = DF{i.hi, im.lo + i.lo};
-    }
-    __device__ __forceinline__ void add(const Carry &o) { re = df_add(re, o.re); im = df_add(im, o.im); }
-    __device__ __forceinline__ cpx<float> plus(cpx<float> a) const   // this + a, one rounding of the sum
-    {
-        return mk((re.hi + a.x) + re.lo, (im.hi + a.y) + im.lo);
-    }
-    __device__ __forceinline__ Carry shfl_up(unsigned mask, int off, int w) const
-    {
-        Carry o;
-        o.re = DF{__shfl_up_sync(mask, re.hi, off, w), __shfl_up_sync(mask, re.lo, off, w)};
-        o.im = DF{__shfl_up_sync(mask, im.hi, off, w), __shfl_up_sync(mask, im.lo, off, w)};
-        return o;
-    }
-};
-template <> struct Carry<double> {
-    double re = 0.0, im = 0.0;
-    __device__ __forceinline__ void add(cpx<double> a) { re += a.x; im += a.y; }
-    __device__ __forceinline__ void add(const Carry &o) { re += o.re; im += o.im; }
-    __device__ __forceinline__ cpx<double> plus(cpx<double> a) const { return mk(re + a.x, im + a.y); }
-    __device__ __forceinline__ Carry shfl_up(unsigned mask, int off, int w) const
-    {
-        Carry o;
-        o.re = __shfl_up_sync(mask, re, off, w);
-        o.im = __shfl_up_sync(mask, im, off, w);
-        return o;
-    }
 };
 
 template <int G> __device__ __forceinline__ unsigned lane_mask()
@@ -243,6 +211,31 @@ template <typename T, int G> __device__ __forceinline__ typename NormSum<T>::typ
     }
 }
 
+// the step loop's norm sum: as slot_norm_sum, with one barrier, which also tells that every thread has read
+// the transform's output (redh is written again only several barriers later)
+template <typename T, int G> __device__ __forceinline__ typename NormSum<T>::type step_norm(SqAcc<T> acc, typename NormSum<T>::type *redh)
+{
+    if constexpr (G <= 32) {
+        const typename NormSum<T>::type v = slot_norm_sum<T, G>(acc, nullptr);
+        __syncwarp(lane_mask<G>());
+        return v;
+    } else {
+        const unsigned mask = lane_mask<G>();
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) acc.shfl_add(mask, off, 32);
+        if ((threadIdx.x & 31) == 0) redh[threadIdx.x >> 5] = acc.v;
+        __syncthreads();
+        acc.v = redh[0];
+#pragma unroll
+        for (int w = 1; w < G / 32; ++w) {
+            SqAcc<T> o;
+            o.v = redh[w];
+            acc.merge(o);
+        }
+        return acc.v;
+    }
+}
+
 // The waiting-time threshold in the form of the norm sum it is compared with: r / dr (the norm is
 // dr times the sum), as a normalised double-float in FP32 forms, computed in FP64 once per waiting
 // period.  The comparisons are then exact on the double-float values.
@@ -272,8 +265,6 @@ template <> struct Threshold<float> {
 // exp(x) and (cos, sin)(pi y): the pi-scaled form has no large-argument reduction path
 __device__ __forceinline__ float k_exp(float x) { return expf(x); }
 __device__ __forceinline__ double k_exp(double x) { return exp(x); }
-__device__ __forceinline__ float k_expm1(float x) { return expm1f(x); }
-__device__ __forceinline__ double k_expm1(double x) { return expm1(x); }
 
 template <typename T> __device__ __noinline__ T table_T3_far(const double *p, int len, T tau, int *seg)
 {
@@ -360,51 +351,71 @@ template <> struct Dyn<float> {
         *e = em1;
     }
     // both points of a pair at once in packed FP32x2 instructions, the same operations per component
-    // as f1t / em1 (bit-identical); a pair with a point outside the series' range takes f1t per point
-    static __device__ __forceinline__ void f1t2(float2 a, float2 t, float2 *fr, float2 *fi, float2 *e)
-    {
-        if (a.x >= -0.5f && a.y >= -0.5f && fabsf(t.x) <= 1.0f && fabsf(t.y) <= 1.0f) {
-            float2 p = __ffma2_rn(make_float2(1.0f / 40320.0f, 1.0f / 40320.0f), a, make_float2(1.0f / 5040.0f, 1.0f / 5040.0f));
-            p = __ffma2_rn(p, a, make_float2(1.0f / 720.0f, 1.0f / 720.0f));
-            p = __ffma2_rn(p, a, make_float2(1.0f / 120.0f, 1.0f / 120.0f));
-            p = __ffma2_rn(p, a, make_float2(1.0f / 24.0f, 1.0f / 24.0f));
-            p = __ffma2_rn(p, a, make_float2(1.0f / 6.0f, 1.0f / 6.0f));
-            p = __ffma2_rn(p, a, make_float2(0.5f, 0.5f));
-            p = __ffma2_rn(p, a, make_float2(1.0f, 1.0f));
-            const float2 em1 = __fmul2_rn(a, p);
-            const float2 u = __fmul2_rn(t, t);
-            float2 ps = __ffma2_rn(make_float2(1.0f / 362880.0f, 1.0f / 362880.0f), u, make_float2(-1.0f / 5040.0f, -1.0f / 5040.0f));
-            ps = __ffma2_rn(ps, u, make_float2(1.0f / 120.0f, 1.0f / 120.0f));
-            ps = __ffma2_rn(ps, u, make_float2(-1.0f / 6.0f, -1.0f / 6.0f));
-            ps = __ffma2_rn(ps, u, make_float2(1.0f, 1.0f));
-            const float2 s = __fmul2_rn(t, ps);
-            float2 pc = __ffma2_rn(make_float2(-1.0f / 3628800.0f, -1.0f / 3628800.0f), u, make_float2(1.0f / 40320.0f, 1.0f / 40320.0f));
-            pc = __ffma2_rn(pc, u, make_float2(-1.0f / 720.0f, -1.0f / 720.0f));
-            pc = __ffma2_rn(pc, u, make_float2(1.0f / 24.0f, 1.0f / 24.0f));
-            pc = __ffma2_rn(pc, u, make_float2(-0.5f, -0.5f));
-            const float2 cm1 = __fmul2_rn(u, pc);
-            const float2 mag = __fadd2_rn(make_float2(1.0f, 1.0f), em1);
-            *fr = __ffma2_rn(cm1, mag, em1);
-            *fi = __fmul2_rn(s, mag);
-            *e = em1;
-        } else {
-            f1t(a.x, t.x, &fr->x, &fi->x, &e->x);
-            f1t(a.y, t.y, &fr->y, &fi->y, &e->y);
-        }
-    }
+    // as f1t / em1 (bit-identical), for arguments in the series' range
+    static __device__ __forceinline__ float2 rep(float v) { return make_float2(v, v); }
     static __device__ __forceinline__ float2 em1_2(float2 a)
     {
-        if (a.x >= -0.5f && a.y >= -0.5f) {
-            float2 p = __ffma2_rn(make_float2(1.0f / 40320.0f, 1.0f / 40320.0f), a, make_float2(1.0f / 5040.0f, 1.0f / 5040.0f));
-            p = __ffma2_rn(p, a, make_float2(1.0f / 720.0f, 1.0f / 720.0f));
-            p = __ffma2_rn(p, a, make_float2(1.0f / 120.0f, 1.0f / 120.0f));
-            p = __ffma2_rn(p, a, make_float2(1.0f / 24.0f, 1.0f / 24.0f));
-            p = __ffma2_rn(p, a, make_float2(1.0f / 6.0f, 1.0f / 6.0f));
-            p = __ffma2_rn(p, a, make_float2(0.5f, 0.5f));
-            p = __ffma2_rn(p, a, make_float2(1.0f, 1.0f));
-            return __fmul2_rn(a, p);
-        }
-        return make_float2(em1(a.x), em1(a.y));
+        float2 p = __ffma2_rn(rep(1.0f / 40320.0f), a, rep(1.0f / 5040.0f));
+        p = __ffma2_rn(p, a, rep(1.0f / 720.0f));
+        p = __ffma2_rn(p, a, rep(1.0f / 120.0f));
+        p = __ffma2_rn(p, a, rep(1.0f / 24.0f));
+        p = __ffma2_rn(p, a, rep(1.0f / 6.0f));
+        p = __ffma2_rn(p, a, rep(0.5f));
+        p = __ffma2_rn(p, a, rep(1.0f));
+        return __fmul2_rn(a, p);
+    }
+    static __device__ __forceinline__ void sc2(float2 t, float2 *s, float2 *cm1)   // sin(t), cos(t) - 1
+    {
+        const float2 u = __fmul2_rn(t, t);
+        float2 ps = __ffma2_rn(rep(1.0f / 362880.0f), u, rep(-1.0f / 5040.0f));
+        ps = __ffma2_rn(ps, u, rep(1.0f / 120.0f));
+        ps = __ffma2_rn(ps, u, rep(-1.0f / 6.0f));
+        ps = __ffma2_rn(ps, u, rep(1.0f));
+        *s = __fmul2_rn(t, ps);
+        float2 pc = __ffma2_rn(rep(-1.0f / 3628800.0f), u, rep(1.0f / 40320.0f));
+        pc = __ffma2_rn(pc, u, rep(-1.0f / 720.0f));
+        pc = __ffma2_rn(pc, u, rep(1.0f / 24.0f));
+        pc = __ffma2_rn(pc, u, rep(-0.5f));
+        *cm1 = __fmul2_rn(u, pc);
+    }
+    static __device__ __forceinline__ void f1t2(float2 a, float2 t, float2 *fr, float2 *fi, float2 *e)
+    {
+        const float2 em1 = em1_2(a);
+        float2 s, cm1;
+        sc2(t, &s, &cm1);
+        const float2 mag = __fadd2_rn(rep(1.0f), em1);
+        *fr = __ffma2_rn(cm1, mag, em1);
+        *fi = __fmul2_rn(s, mag);
+        *e = em1;
+    }
+    // the same beyond the series' range, reduced to it by Cody and Waite's two-part constants: exp(a) = 2^n exp(a - n ln 2), and t - 2 pi k quartered
+    // and doubled back twice (cos 2x - 1 = -2 sin^2 x, sin 2x = 2 sin x (1 + (cos x - 1))); a < -87 counts as
+    // -87, |t| <= 1e5
+    static __device__ __forceinline__ void far2(float2 a, float2 t, float2 *fr, float2 *fi, float2 *e)
+    {
+        const float2 magic = rep(12582912.0f);   // 1.5 x 2^23: adding it rounds to the nearest integer
+        a = make_float2(fmaxf(a.x, -87.0f), fmaxf(a.y, -87.0f));
+        const float2 nm = __ffma2_rn(a, rep(1.44269504088896341f), magic);
+        const float2 n = __fadd2_rn(nm, rep(-12582912.0f));
+        float2 r = __ffma2_rn(n, rep(-0.693147182464599609f), a);
+        r = __ffma2_rn(n, rep(1.90465429995776804e-9f), r);
+        const float2 sc = make_float2(__int_as_float((__float_as_int(nm.x) << 23) + 0x3f800000),
+                                      __int_as_float((__float_as_int(nm.y) << 23) + 0x3f800000));   // 2^n
+        const float2 em1 = __ffma2_rn(sc, em1_2(r), __fadd2_rn(sc, rep(-1.0f)));
+        const float2 k = __fadd2_rn(__ffma2_rn(t, rep(0.159154943091895336f), magic), rep(-12582912.0f));
+        t = __ffma2_rn(k, rep(-6.28318548202514648f), t);
+        t = __ffma2_rn(k, rep(1.74845560e-7f), t);
+        float2 s, c;
+        sc2(__fmul2_rn(t, rep(0.25f)), &s, &c);
+        float2 s2 = __fmul2_rn(s, rep(2.0f)), c2 = __fmul2_rn(s2, make_float2(-s.x, -s.y));
+        s2 = __ffma2_rn(s2, c, s2);
+        s = __fmul2_rn(s2, rep(2.0f));
+        c = __fmul2_rn(s, make_float2(-s2.x, -s2.y));
+        s = __ffma2_rn(s, c2, s);
+        const float2 mag = __fadd2_rn(rep(1.0f), em1);
+        *fr = __ffma2_rn(c, mag, em1);
+        *fi = __fmul2_rn(s, mag);
+        *e = em1;
     }
 };
 template <> struct Dyn<double> {
@@ -518,23 +529,34 @@ template <typename T> __device__ __forceinline__ void ksu_point(const Tables<T> 
     vi = -k.gI * ksu_phi(tb, x);
 }
 
-// in-place DFT of RR values (natural order in); output k lands in slot operm(k); PK: packed products
-template <typename T, int RR, bool PK = false> struct DFTI {
+// in-place DFT of RR values (natural order in); output k lands in slot operm(k)
+template <typename T, int RR> struct DFTI {
     static __device__ __forceinline__ constexpr int operm(int k)
     {
-        if constexpr (RR == 16) return (k % 4) * 4 + k / 4;
+        if constexpr (RR == 32) return (k % 4) * 8 + DFTI<T, 8>::operm(k / 4);
+        else if constexpr (RR == 16) return (k % 4) * 4 + k / 4;
         else if constexpr (RR == 8) return (k % 4) * 2 + k / 4;
         else return k;
     }
     static __device__ __forceinline__ void run(cpx<T> *x)
     {
-        if constexpr (RR == 16) {
+        if constexpr (RR == 32) {
+#pragma unroll
+            for (int n2 = 0; n2 < 8; ++n2) {
+                dft4(x[n2], x[8 + n2], x[16 + n2], x[24 + n2]);      // k1 of column n2 at slot n2 + 8 k1
+                x[8 + n2] = tw32<T>(x[8 + n2], n2 * 1);
+                x[16 + n2] = tw32<T>(x[16 + n2], n2 * 2);
+                x[24 + n2] = tw32<T>(x[24 + n2], n2 * 3);
+            }
+#pragma unroll
+            for (int k1 = 0; k1 < 4; ++k1) DFTI<T, 8>::run(x + 8 * k1);
+        } else if constexpr (RR == 16) {
 #pragma unroll
             for (int n2 = 0; n2 < 4; ++n2) {
                 dft4(x[n2], x[4 + n2], x[8 + n2], x[12 + n2]);       // k1 of column n2 at slot n2 + 4 k1
-                x[4 + n2] = tw16<T, PK>(x[4 + n2], n2 * 1);
-                x[8 + n2] = tw16<T, PK>(x[8 + n2], n2 * 2);
-                x[12 + n2] = tw16<T, PK>(x[12 + n2], n2 * 3);
+                x[4 + n2] = tw16<T>(x[4 + n2], n2 * 1);
+                x[8 + n2] = tw16<T>(x[8 + n2], n2 * 2);
+                x[12 + n2] = tw16<T>(x[12 + n2], n2 * 3);
             }
 #pragma unroll
             for (int k1 = 0; k1 < 4; ++k1) dft4(x[4 * k1], x[4 * k1 + 1], x[4 * k1 + 2], x[4 * k1 + 3]);
@@ -542,9 +564,9 @@ template <typename T, int RR, bool PK = false> struct DFTI {
 #pragma unroll
             for (int n2 = 0; n2 < 2; ++n2) {
                 dft4(x[n2], x[2 + n2], x[4 + n2], x[6 + n2]);        // k1 of column n2 at slot n2 + 2 k1
-                x[2 + n2] = tw16<T, PK>(x[2 + n2], 2 * n2 * 1);
-                x[4 + n2] = tw16<T, PK>(x[4 + n2], 2 * n2 * 2);
-                x[6 + n2] = tw16<T, PK>(x[6 + n2], 2 * n2 * 3);
+                x[2 + n2] = tw16<T>(x[2 + n2], 2 * n2 * 1);
+                x[4 + n2] = tw16<T>(x[4 + n2], 2 * n2 * 2);
+                x[6 + n2] = tw16<T>(x[6 + n2], 2 * n2 * 3);
             }
 #pragma unroll
             for (int k1 = 0; k1 < 4; ++k1) dft2(x[2 * k1], x[2 * k1 + 1]);
@@ -559,260 +581,397 @@ template <typename T, int RR, bool PK = false> struct DFTI {
 // ------------------------------------------------------------------------------------------------
 // the sine transform
 // ------------------------------------------------------------------------------------------------
-template <typename T, int N, int V> struct Fused {
-    using P = FusedPlan<N, V>;
+template <int G> __device__ __forceinline__ void traj_sync()
+{
+    if constexpr (G > 32) __syncthreads();
+    else __syncwarp(lane_mask<G>());
+}
+
+template <typename T, int N, int V> struct Sine {
+    using P = FusedPlan<T, N, V>;
     using PR = Prec<T>;
     using C = typename Prec<T>::C;
-    using RL = typename Prec<T>::Rl;
-    static constexpr int R = P::R, G = P::G, NR = P::NR, E = 2 * R;
-    // FP32 at N >= 8192: the hi+lo complex products (pass twiddles, kinetic factors, DFT constants) as
-    // packed FP32x2 instructions -- +9% at N = 8192 and +12% at 16384 over the scalar products, which
-    // stay faster at N <= 4096 (-6% at 4096 with the packed form); the results are bit-identical
-    static constexpr bool PK = sizeof(T) == 4 && N >= 8192;
-    using DR = DFTI<T, R, PK>;
-    static __device__ __forceinline__ cpx<T> cmul(cpx<T> x, C w) { return PK ? PR::mul2(x, w) : PR::mul(x, w); }
+    static constexpr int R = P::R, H = P::H, G = P::G, M = P::M, S = P::S, NS = P::NS, SEQ = P::SEQ;
+    // (the hi+lo products stay scalar: as packed FP32x2 instructions, with their operands regrouped, they ran 8%
+    // slower at N = 8192 and 4% at 16384)
+    using DR = DFTI<T, R>;
+    static __device__ __forceinline__ cpx<T> cmul(cpx<T> x, C w) { return PR::mul(x, w); }
+    static __device__ __forceinline__ cpx<T> neg(cpx<T> a) { return mk(-a.x, -a.y); }
 
-    static __device__ __forceinline__ int pad(int j) { return j + j / R; }
-    // E/odd layout of the transform's output (and of the state between transforms): S_{2k} at
-    // even_pos(k), S_{2k+1} at odd_pos(k).  (An XOR swizzle of both areas, meant to spread the
-    // even/odd lanes of the transform's load over all banks, measured 0.4-4.6% slower.)
-    static __device__ __forceinline__ int even_pos(int k) { return k; }
-    static __device__ __forceinline__ int odd_pos(int k) { return N / 2 + k + k / R; }
-    static __device__ __forceinline__ int b_of(int g, int t) { return t == 0 ? (g == 0 ? 0 : g) : (g == 0 ? NR / 2 : NR - g); }
-    // global index of register element e (first/last-pass layout)
-    static __device__ __forceinline__ int idx(int g, int e) { return b_of(g, e / R) + (e % R) * NR; }
-    // shared-memory position of S_j in the E/odd layout
-    static __device__ __forceinline__ int s_pos(int j) { return (j & 1) ? odd_pos(j >> 1) : even_pos(j >> 1); }
+    // addresses of position b of a sequence and of its mirror S - b
+    static __device__ __forceinline__ int pos(int b) { return b + b / R; }
 
-    // y_j = s (f_j + f_{N-j}) + (f_j - f_{N-j})/2 for the pair (ea, eb) = (j, N-j)
-    static __device__ __forceinline__ void pre_pair(cpx<T> *x, int ea, int eb, RL s)
+    // Slot 0 holds y_m = x_{S m} (m < R/2) and w_m = x_{S/2 + S m} (m >= R/2), the independent halves of the
+    // odd sequence y (y_0 = y_{R/2} = 0, y_{R-m} = -y_m) and of w (w_{R-1-m} = -w_m): y + w, in place
+    static __device__ __forceinline__ void special_in(cpx<T> *r)
     {
-        const cpx<T> a = x[ea], b = x[eb];
-        const cpx<T> sum = PR::mulr(a + b, s), dif = scale(a - b, (T)0.5);
-        x[ea] = sum + dif;
-        x[eb] = sum - dif;
-    }
-
-    static __device__ __forceinline__ void pre(cpx<T> *x, int g, const RL *sinpre)
-    {
-        if (g != 0) {
+        r[0] = neg(r[R - 1]);
 #pragma unroll
-            for (int m = 0; m < R; ++m) pre_pair(x, m, R + (R - 1 - m), PR::ldr(&sinpre[g + m * NR]));
-        } else {
-            x[0] = mk<T>(0, 0);                                // j = 0
-            x[R / 2] = scale(x[R / 2], (T)2);                  // j = N/2 pairs with itself, sin = 1
-#pragma unroll
-            for (int m = 1; m < R / 2; ++m) pre_pair(x, m, R - m, PR::ldr(&sinpre[m * NR]));
-#pragma unroll
-            for (int m = 0; m < R / 2; ++m) pre_pair(x, R + m, R + (R - 1 - m), PR::ldr(&sinpre[NR / 2 + m * NR]));
+        for (int m = 1; m < H; ++m) {
+            r[R - m] = r[R - m] - r[m];
+            r[m] = r[m] - r[R - 1 - m];
         }
     }
 
-    // E_k = (i/2)(Y_k - Y_{N-k}) -> [k];  C_k = (Y_k + Y_{N-k})/2 (C_0 halved) -> odd area
-    static __device__ __forceinline__ void post_pair(cpx<T> *buf, int k, cpx<T> A, cpx<T> B)
+    // The DFT Z of y + w is left at the positions 0 (Z[k]) and S/2 (Z[R-k]) of sequence k, and the threads of
+    // the middle pass that read both separate them: y's part is odd in k and w's obeys Z_w[-k] = -W_R^k
+    // Z_w[k], so Z_w[k] = (Z[k] + Z[-k]) / (1 - W_R^k) (at most 1/(2 sin(pi/R)) times the sum), and with w's
+    // first-pass twiddle W_2R^k and q = Z[k] + Z[-k], d = Z[k] - Z[-k]:
+    // A_k[S/2] = -i q / (2 sin(pi k/R)), A_k[0] = d/2 + (i/2) cot(pi k/R) q.
+    static __device__ __forceinline__ void special_out(const cpx<T> *x, cpx<T> *buf)
     {
-        buf[even_pos(k)] = mul_i(scale(A - B, (T)0.5));
-        buf[odd_pos(k)] = scale(A + B, (T)0.5);
+        constexpr int p2 = S / 2 + S / 2 / R;
+#pragma unroll
+        for (int k = 1; k < H; ++k) {
+            buf[k * SEQ] = x[DR::operm(k)];
+            buf[k * SEQ + p2] = x[DR::operm(R - k)];
+        }
+        buf[0] = mk<T>(0, 0);
+        buf[p2] = mul_mi(x[DR::operm(H)]);
+    }
+    static __device__ __forceinline__ void special_mid(cpx<T> &a, cpx<T> &b, const C *ts, int k)
+    {
+        const C w = PR::ld(ts + k);   // (1 / (2 sin), cot / 2)
+        const cpx<T> q = a + b, d = scale(a - b, (T)0.5), al = PR::mulr(q, PR::re(w)), be = PR::mulr(q, PR::im(w));
+        a = d + mul_i(be);
+        b = mul_mi(al);
     }
 
-    // Y at index b_t + m NR is in register slot t R + operm(m) after the last pass
-    static __device__ __forceinline__ cpx<T> Y(const cpx<T> *x, int t, int m) { return x[t * R + DR::operm(m)]; }
-
-    static __device__ __forceinline__ void post(const cpx<T> *x, int g, cpx<T> *buf)
+    // First pass: the slots' DFTs, twiddles, and the writes of every sequence at b and -b.  pb, pm: the
+    // addresses of b and S - b of the thread's slots.
+    static __device__ __forceinline__ void first(cpx<T> *x, cpx<T> *buf, const C *ta, int g, const int *pb, const int *pm)
     {
-        if (g != 0) {
+        if (g == 0) special_in(x);
 #pragma unroll
-            for (int m = 0; m < R; ++m) {
-                if (m < R / 2) post_pair(buf, g + m * NR, Y(x, 0, m), Y(x, 1, R - 1 - m));
-                else post_pair(buf, (NR - g) + (R - 1 - m) * NR, Y(x, 1, R - 1 - m), Y(x, 0, m));
-            }
-        } else {
-            buf[even_pos(0)] = mk<T>(0, 0);
-            buf[odd_pos(0)] = scale(Y(x, 0, 0), (T)0.5);      // S_1 = C_0 / 2 = Y_0 / 2
+        for (int t = 0; t < NS; ++t) {
+            cpx<T> *v = x + t * R;
+            DR::run(v);
+            if (t == 0 && g == 0) {
+                special_out(v, buf);
+            } else {
+                const C *w = ta + g + t * G;
+                cpx<T> *ob = buf + pb[t], *om = buf + pm[t];
 #pragma unroll
-            for (int m = 1; m < R / 2; ++m) post_pair(buf, m * NR, Y(x, 0, m), Y(x, 0, R - m));
-#pragma unroll
-            for (int m = 0; m < R / 2; ++m) post_pair(buf, NR / 2 + m * NR, Y(x, 1, m), Y(x, 1, R - 1 - m));
-        }
-    }
-
-    // inclusive prefix sum of the N/2 odd-area values: thread g owns the chunk k in [gR, gR + R).
-    // Chunk totals and the carries between chunks are compensated (a rounding error there would reach
-    // every later coefficient); the running sum inside a chunk is plain and only reaches its chunk.
-    static __device__ __forceinline__ void scan(cpx<T> *buf, int g, Carry<T> *wtot)
-    {
-        constexpr int W = G < 32 ? G : 32;
-        const unsigned mask = lane_mask<G>();
-        cpx<T> v[R];
-#pragma unroll
-        for (int q = 0; q < R; ++q) v[q] = buf[odd_pos(g * R + q)];
-        Carry<T> tot;
-#pragma unroll
-        for (int q = 0; q < R; ++q) tot.add(v[q]);
-        const int lane = threadIdx.x & (W - 1);
-        Carry<T> inc = tot;
-#pragma unroll
-        for (int off = 1; off < W; off <<= 1) {
-            Carry<T> y = inc.shfl_up(mask, off, W);
-            if (lane >= off) inc.add(y);
-        }
-        Carry<T> excl = inc.shfl_up(mask, 1, W);
-        if (lane == 0) excl = Carry<T>();
-        if constexpr (G > 32) {
-            const int warp = threadIdx.x >> 5;
-            if (lane == 31) wtot[warp] = inc;
-            __syncthreads();
-#pragma unroll 1
-            for (int w = 0; w < warp; ++w) excl.add(wtot[w]);
-        }
-        cpx<T> run = mk<T>(0, 0);
-#pragma unroll
-        for (int q = 0; q < R; ++q) {
-            run = run + v[q];
-            buf[odd_pos(g * R + q)] = excl.plus(run);
-        }
-    }
-
-    // One middle pass (radix RM after PP points): butterfly i reads [i + m N/RM], multiplies by
-    // W_{PP RM}^{m k} (k = i mod PP) and writes [(i - k) RM + k + m PP].  A thread's butterflies are
-    // g + q G; when PP <= G they share k = g mod PP and so their twiddles, which are loaded once per m
-    // (from tw, the table [RM][PP] of W_{PP RM}^{m k}).
-    template <int RM, int PP>
-    static __device__ __forceinline__ void mid_pass(cpx<T> *x, cpx<T> *buf, const C *tw, int g)
-    {
-        if constexpr (RM > 1) {
-            constexpr int NB = N / RM, PER = E / RM;
-            static_assert(PP <= G, "mid-pass twiddle sharing needs PP <= G");
-            const int k = g & (PP - 1);
-#pragma unroll
-            for (int m = 0; m < RM; ++m) {
-                C w{};
-                if (m) w = tw_at(tw, m * PP + k);
-#pragma unroll
-                for (int q = 0; q < PER; ++q) {
-                    cpx<T> v = buf[pad(g + q * G + m * NB)];
-                    if (m) v = cmul(v, w);
-                    x[q * RM + m] = v;
+                for (int k = 1; k < H; ++k) {
+                    const C wk = PR::ld(w + (k - 1) * P::NSLOT);
+                    ob[k * SEQ] = cmul(v[DR::operm(k)], wk);
+                    om[k * SEQ] = cmul(v[DR::operm(R - k)], PR::nconj(wk));
                 }
+                // the sequence P = U + V at b: u + th z, at -b: -u - conj(th) z, th = e^(-i pi b/S)
+                const C th = PR::ld(w + (H - 1) * P::NSLOT);
+                const cpx<T> u = v[0], z = v[DR::operm(H)];
+                const cpx<T> s = PR::mulr(z, PR::re(th)), d = PR::mulr(z, PR::im(th));
+                const cpx<T> a = u + s, b = mul_i(d);
+                ob[0] = a + b;
+                om[0] = b - a;
             }
-            __syncthreads();
+        }
+    }
+
+    // One middle pass of radix RM in place: butterfly i = (kk RO + o) R + b1 of the values at
+    // b1 + R (LO o + LM m), m < RM.  TW 0: none, 1: the last pass's twiddle W_S^(b1 q1) from tm [q1][b1]
+    // (M2 = 1), 2: the inner twiddle W_M^(m2 k1) from ti [k1][m2] (o = m2).
+    template <int RM, int RO, int LO, int LM, int TW, bool FIRST>
+    static __device__ __forceinline__ void mid_pass(cpx<T> *x, cpx<T> *buf, const C *tw, const C *ts, int g)
+    {
+        constexpr int NB = N / RM, PER = (NB + G - 1) / G;
+        const int b1 = g % R;   // the same for all of a thread's butterflies (R divides G)
+#pragma unroll
+        for (int q = 0; q < PER; ++q) {
+            const int i = g + q * G;
+            if (NB % G == 0 || i < NB) {
+                const int o = i / R % RO, kk = i / (R * RO);
+                const cpx<T> *p = buf + kk * SEQ + b1 + (R + 1) * LO * o;
+#pragma unroll
+                for (int m = 0; m < RM; ++m) x[q * RM + m] = p[(R + 1) * LM * m];
+                // the positions 0 and S/2 (both at o = 0: M1 is even)
+                if (FIRST && b1 == 0 && o == 0 && kk > 0) special_mid(x[q * RM], x[q * RM + RM / 2], ts, kk);
+                DFTI<T, RM>::run(x + q * RM);
+            }
+        }
+#pragma unroll
+        for (int m = 0; m < RM; ++m) {
+            C w{};
+            if (m && TW == 1) w = PR::ld(tw + m * R + b1);
 #pragma unroll
             for (int q = 0; q < PER; ++q) {
                 const int i = g + q * G;
-                DFTI<T, RM, PK>::run(x + q * RM);
-                const int base = (i - k) * RM + k;
-#pragma unroll
-                for (int m = 0; m < RM; ++m) buf[pad(base + m * PP)] = x[q * RM + DFTI<T, RM, PK>::operm(m)];
-            }
-            __syncthreads();
-        }
-    }
-
-    // twiddle tables of the middle passes live in shared memory (FusedPlan: TW1, TW2); an FP32 entry
-    // (hi+lo, 16 bytes) is one 16-byte load
-    static __device__ __forceinline__ C tw_at(const C *tw, int i)
-    {
-        if constexpr (sizeof(T) == 4) {
-            const float4 v = *reinterpret_cast<const float4 *>(tw + i);
-            return C{v.x, v.y, v.z, v.w};
-        } else {
-            return tw[i];
-        }
-    }
-
-    // S (E/odd layout in buf), optionally times K_T, at the first-pass indices -> DST -> E/odd layout
-    static __device__ __forceinline__ void dst(cpx<T> *x, cpx<T> *buf, const Tables<T> &tb, int g, Carry<T> *wtot,
-                                               const C *tw1, const C *tw2, bool kinetic)
-    {
-#pragma unroll
-        for (int e = 0; e < E; ++e) {
-            const int j = idx(g, e);
-            cpx<T> v = buf[s_pos(j)];
-            if (kinetic) v = cmul(v, PR::ld(&tb.KT[j]));
-            x[e] = v;
-        }
-        __syncthreads();
-        pre(x, g, tb.sinpre);
-        // first pass (radix R, no twiddles): butterfly b -> [b R + k]
-#pragma unroll
-        for (int t = 0; t < 2; ++t) {
-            DR::run(x + t * R);
-            const int b = b_of(g, t);
-#pragma unroll
-            for (int k = 0; k < R; ++k) buf[pad(b * R + k)] = x[t * R + DR::operm(k)];
-        }
-        __syncthreads();
-        mid_pass<P::M1, R>(x, buf, tw1, g);
-        mid_pass<P::M2, R * P::M1>(x, buf, tw2, g);
-        // last pass (radix R, stride N/R): inputs [b + m NR], twiddle W^(m b).  For the mirror butterfly
-        // b2 = NR - g, W^(m b2) = W_R^m conj(W^(m g)): one table load serves both (g = 0 pairs
-        // 0 with NR/2, whose twiddles are loaded directly).
-#pragma unroll
-        for (int m = 0; m < R; ++m) {
-            cpx<T> v1 = buf[pad(b_of(g, 0) + m * NR)];
-            cpx<T> v2 = buf[pad(b_of(g, 1) + m * NR)];
-            if (m) {
-                // W^(m g): up to N = 2048 from the radix's compact [m][g] section (a warp reads
-                // consecutive entries; measured +3% at N = 1024, +6.5% at 2048), above from the
-                // strided W[m g] (the compact table measured 9% slower at N = 4096, 1% at 16384)
-                const C w = N <= 2048 ? PR::ld(&tb.WL[(R == 16 ? 0 : R == 8 ? N / 2 : N) + m * G + g])
-                                      : PR::ld(&tb.W[m * g]);
-                v1 = cmul(v1, w);
-                if (g != 0) {
-                    v2 = tw16<T, PK>(cmul(v2, PR::conj(w)), m * (16 / R));
-                } else {
-                    v2 = cmul(v2, PR::ld(&tb.W[m * (NR / 2)]));
+                if (NB % G == 0 || i < NB) {
+                    const int o = i / R % RO, kk = i / (R * RO);
+                    if (m && TW == 2) w = PR::ld(tw + m * RO + o);
+                    cpx<T> v = x[q * RM + DFTI<T, RM>::operm(m)];
+                    if (m && TW) v = cmul(v, w);
+                    buf[kk * SEQ + b1 + (R + 1) * (LO * o + LM * m)] = v;
                 }
             }
-            x[m] = v1;
-            x[R + m] = v2;
         }
-        __syncthreads();
+    }
+
+    static __device__ __forceinline__ void mid(cpx<T> *x, cpx<T> *buf, const C *tm, const C *ti, const C *ts, int g)
+    {
+        if constexpr (P::M2 == 1) {
+            mid_pass<P::M1, 1, 0, 1, P::TWL ? 0 : 1, true>(x, buf, tm, ts, g);
+        } else {
+            // m = m2 + M2 m1: DFT over m1 -> k1, twiddle, DFT over m2 -> k2; q1 = k1 + M1 k2 at M2 k1 + k2
+            mid_pass<P::M1, P::M2, 1, P::M2, 2, true>(x, buf, ti, ts, g);
+            traj_sync<G>();
+            mid_pass<P::M2, P::M1, P::M2, 1, 0, false>(x, buf, nullptr, nullptr, g);
+        }
+    }
+
+    // Last pass: X_{b + S q2} into value q2 of every slot (natural order)
+    static __device__ __forceinline__ void last(cpx<T> *x, cpx<T> *buf, const C *tm, int g)
+    {
+        constexpr bool SAME = G % M == 0;   // a thread's slots share q1
+        cpx<T> y[NS * R];
 #pragma unroll
-        for (int t = 0; t < 2; ++t) DR::run(x + t * R);
-        post(x, g, buf);
-        __syncthreads();
-        scan(buf, g, wtot);
-        __syncthreads();
+        for (int b1 = 0; b1 < R; ++b1) {
+            C w{};
+            if (P::TWL && SAME && b1) w = PR::ld(tm + b1 * M + g % M);
+#pragma unroll
+            for (int t = 0; t < NS; ++t) {
+                const int s = g + t * G, q1 = s % M;
+                const int loc = P::M2 == 1 ? q1 : q1 / P::M1 + P::M2 * (q1 % P::M1);
+                cpx<T> v = buf[s / M * SEQ + (R + 1) * loc + b1];
+                if (P::TWL && b1) {
+                    if (!SAME) w = PR::ld(tm + b1 * M + q1);
+                    v = cmul(v, w);
+                }
+                y[t * R + b1] = v;
+            }
+        }
+#pragma unroll
+        for (int t = 0; t < NS; ++t) {
+            DR::run(y + t * R);
+#pragma unroll
+            for (int m = 0; m < R; ++m) x[t * R + m] = y[t * R + DR::operm(m)];
+        }
+        if constexpr (M > 32) traj_sync<G>();
+        if (M > 32 || g < 32) split(x, buf, g);   // (warp 0)
+    }
+
+    // The kk = 0 slots (threads g < M) hold P_q = U_q + V_q, q = g + M m; leaves V_q in the slots g >= M/2,
+    // U_q in those below, and slot 0's two half sequences (special_in).  V_q = P_0 + sum_{i=1..q} (P_i +
+    // P_{-i}) for q < S/2, through the kk = 0 sequence's own shared memory: each of LN lanes of warp 0 sums a run of
+    // CH values, the runs' totals are scanned with shuffles, and V overwrites P's lower half (only the run's
+    // owner reads it; the upper half stays).  The sum carries the rounding errors of at most S/2 values of
+    // 2/R of the spectrum.  For M > 32 (radix-8 variants) warp 0 sums for all and every thread calls this.
+    static __device__ __forceinline__ void split(cpx<T> *x, cpx<T> *buf, int g)
+    {
+        constexpr int LN = G < 32 ? G : 32, CH = S / 2 / LN;
+        static_assert(CH * LN * 2 == S, "split");
+        const unsigned mask = lane_mask<G>();
+        auto sync = [&]() {
+            if constexpr (M > 32) __syncthreads();
+            else __syncwarp(mask);
+        };
+        if constexpr (M <= 32) __syncwarp(mask);
+        if (g < M) {
+#pragma unroll
+            for (int m = 0; m < R; ++m) buf[pos(g + M * m)] = x[m];
+        }
+        sync();
+        if (M <= 32 || g < LN) {
+            cpx<T> c[CH];
+#pragma unroll
+            for (int i = 0; i < CH; ++i) {
+                const int q = g * CH + i;
+                c[i] = buf[pos(q)];
+                if (i > 0 || g > 0) c[i] = c[i] + buf[pos(S - q)];   // q = 0: P_0 = V_0 (U_0 = 0)
+                if (i > 0) c[i] = c[i - 1] + c[i];
+            }
+            cpx<T> inc = c[CH - 1];
+#pragma unroll
+            for (int off = 1; off < LN; off <<= 1) {
+                const cpx<T> o = mk<T>(__shfl_up_sync(mask, inc.x, off, LN), __shfl_up_sync(mask, inc.y, off, LN));
+                if (g >= off) inc = inc + o;
+            }
+            cpx<T> ex = mk<T>(__shfl_up_sync(mask, inc.x, 1, LN), __shfl_up_sync(mask, inc.y, 1, LN));
+            if (g == 0) ex = mk<T>(0, 0);
+#pragma unroll
+            for (int i = 0; i < CH; ++i) buf[pos(g * CH + i)] = ex + c[i];
+        }
+        sync();
+        if (g < M) {
+#pragma unroll
+            for (int m = 0; m < R; ++m) {
+                const int q = g + M * m;
+                const cpx<T> v = m < H ? buf[pos(q)] : neg(buf[pos(S - 1 - q)]);   // V_{S-1-q} = -V_q
+                x[m] = g < M / 2 ? x[m] - v : v;
+            }
+            if (g == 0) {   // w_m = U_q at q = M/2 + M m
+#pragma unroll
+                for (int m = H; m < R; ++m) {
+                    const int q = M / 2 + M * m;
+                    x[m] = buf[pos(q)] + buf[pos(S - 1 - q)];
+                }
+            }
+        }
+    }
+
+    // S <- K_T S on the register values (kf: two rows of G entries per pair of values)
+    static __device__ __forceinline__ void kinetic(cpx<T> *x, const C *kf, int g)
+    {
+#pragma unroll
+        for (int pr = 0; pr < NS * H; ++pr) {
+            const int e0 = pr / H * R + pr % H, e1 = pr / H * R + R - 1 - pr % H;
+            x[e0] = cmul(x[e0], PR::ld(kf + (2 * pr) * G + g));
+            x[e1] = cmul(x[e1], PR::ld(kf + (2 * pr + 1) * G + g));
+        }
     }
 };
 
 // ------------------------------------------------------------------------------------------------
-// pointwise work on the E/odd layout: thread g visits k = g, g + G, ... < N/2 and the two elements
-// S_{2k} (at even_pos(k) = k) and S_{2k+1} (at odd_pos(k))
+// pointwise work.  The common step's factor and norm act on the registers (factor_regs).  Everything
+// rarer -- the first and last half-steps, jumps, caps, summary rows, rows beyond the static table, the KSU
+// factor and the read-out -- works on a copy of the registers in shared memory, element e of thread g at
+// e G + g, in loops over e: a thread only touches its own elements, and the step's code stays short.
+// Values carry the odd extension's sign (fused_plan.h).
 // ------------------------------------------------------------------------------------------------
 template <typename T, int N, int V> struct Pointwise {
-    using K = Fused<T, N, V>;
-    static constexpr bool PD = sizeof(T) == 4 && N >= 2048 && N <= 8192;
+    using P = FusedPlan<T, N, V>;
     using PR = Prec<T>;
     using C = typename Prec<T>::C;
-    static constexpr int G = K::G;
-
     using SC = typename Prec<T>::S;
-    static __device__ __forceinline__ SC stat(const Tables<T> &tb, const SC *tab, int c, int l, int j, bool full)
+    static constexpr int G = P::G, E = P::E, R = P::R, H = P::H, M = P::M, S = P::S, NS = P::NS;
+    static constexpr bool ADJ = sizeof(T) == 4;   // static rows: the two entries of a pair adjacent
+
+    static __device__ __forceinline__ int jof(int g, int e) { return plan_j(g, e, R, M, G); }
+    static __device__ __forceinline__ bool odd_half(int e) { return e % R >= H; }   // the register holds -u_j
+    static __device__ __forceinline__ int stat_idx(int g, int e)
     {
-        if (l < LTAB) return PR::ld_s(&tab[((size_t)c * LTAB + l) * N + j]);
+        const int m = e % R, h = m >= H, pr = e / R * H + (h ? R - 1 - m : m);
+        return ADJ ? 2 * (pr * G + g) + h : (2 * pr + h) * G + g;
+    }
+    static __device__ __forceinline__ SC stat(const Tables<T> &tb, const SC *tab, int c, int l, int g, int e, bool full)
+    {
+        if (l < LTAB) return PR::ld_s(&tab[((size_t)c * LTAB + l) * N + stat_idx(g, e)]);
+        const int j = jof(g, e);
         if (j == 0) return PR::make_s(0.0, 0.0);
         return static_far<T>(tb.coul[c], tb.M, tb.dt, l, j * tb.dr, full ? 2.0 : 1.0);
     }
 
+    static __device__ __forceinline__ void to_smem(const cpx<T> *x, cpx<T> *buf, int g)
+    {
+#pragma unroll
+        for (int e = 0; e < E; ++e) buf[e * G + g] = x[e];
+    }
+    static __device__ __forceinline__ void to_regs(cpx<T> *x, const cpx<T> *buf, int g)
+    {
+#pragma unroll
+        for (int e = 0; e < E; ++e) x[e] = buf[e * G + g];
+    }
+
+    // The dynamic factor exp(a) exp(i pi y) is close to 1 and changes little from step to step; it is applied
+    // as w + w f1 with f1 its deviation from 1, evaluated so that the rounding is relative to f1, not to 1 (a
+    // rounding of a value next to 1 would repeat identically every step and add up).
+    static __device__ __forceinline__ cpx<T> apply(cpx<T> w, T f1r, T f1i)
+    {
+        if constexpr (sizeof(T) == 4) return mk(fmaf(w.x, f1r, fmaf(-w.y, f1i, w.x)), fmaf(w.y, f1r, fmaf(w.x, f1i, w.y)));
+        else return mk(w.x + (w.x * f1r - w.y * f1i), w.y + (w.x * f1i + w.y * f1r));
+    }
+
+    // The step's factor on the registers: x <- stat2 dyn_a dyn_b x, accumulating sum exp(2 er_a r^2) |x_old|^2
+    // (the end-of-step norm / dr).  dyn = exp((er + i ei) r^2), er and ei multiplied by T^3; A = (er_a + er_b)
+    // dr^2, B = (ei_a + ei_b) dr^2 / pi, D = (er_a - er_b) dr^2, rounded once per step and multiplied with the
+    // exact j^2 (N <= 4096; rounded once above), so no rounding that repeats identically every step enters.
+    // exp(2 er_a r^2) = mag exp((er_a - er_b) r^2), the second factor 1 + z with |z| <~ 1e-4 (the temperature's
+    // change over one step): FP32 keeps the first order, FP64 the series to z^3.
+    // PHASE = false: gamma_hat = 0, B = 0 exactly, the phase series is skipped (its value would be 0).
+    template <bool PHASE>
+    static __device__ __forceinline__ void factor_regs(cpx<T> *x, const SC *row, int g, T A, T B, T D, SqAcc<T> &acc,
+                                                       SqAcc<T> &acc2)
+    {
+        const T Bpi = (T)3.14159265358979323846 * B;
+        const T qlim = fmax(-2 * A, fabs(Bpi));   // a >= -1/2 and |t| <= 1 where qlim j^2 <= 1
+#pragma unroll
+        for (int t = 0; t < NS; ++t) {
+            int lo, hi;
+            slot_points(g + t * G, R, M, lo, hi);
+#pragma unroll
+            for (int m = 0; m < H; ++m) {
+                cpx<T> &x0 = x[t * R + m], &x1 = x[t * R + R - 1 - m];
+                const int pr = t * H + m;
+                if constexpr (sizeof(T) == 4) {
+                    // the series of the pair (m, R-1-m) in packed FP32x2 instructions
+                    const float4 st = __ldg(reinterpret_cast<const float4 *>(row) + pr * G + g);
+                    const float2 j = make_float2((float)(lo + S * m), (float)(hi + S * m));
+                    const float2 j2 = __fmul2_rn(j, j);
+                    const float2 a2 = __fmul2_rn(make_float2(A, A), j2);
+                    float2 fr, fi = make_float2(0.f, 0.f), em;
+                    const float2 t2 = __fmul2_rn(make_float2(Bpi, Bpi), j2);
+                    // every j of row m is below S (m + 1): one uniform test says that all arguments of the row are
+                    // in the series' range
+                    const bool near = qlim * ((float)(S * (m + 1)) * (float)(S * (m + 1))) <= 1.0f;
+                    if (PHASE) {
+                        if (near) Dyn<float>::f1t2(a2, t2, &fr, &fi, &em);
+                        else Dyn<float>::far2(a2, t2, &fr, &fi, &em);
+                    } else {
+                        if (near) em = Dyn<float>::em1_2(a2);
+                        else Dyn<float>::far2(a2, t2, &fr, &fi, &em);
+                        fr = em;
+                    }
+                    const float2 z = __fmul2_rn(make_float2(D, D), j2);
+                    const float2 mag = __fadd2_rn(make_float2(1.f, 1.f), em), wt = __ffma2_rn(mag, z, mag);
+                    acc.add_w(x0, wt.x);
+                    acc2.add_w(x1, wt.y);
+                    const cpx<T> w0 = PR::mul_s(x0, mk(st.x, st.y)), w1 = PR::mul_s(x1, mk(st.z, st.w));
+                    x0 = PHASE ? apply(w0, fr.x, fi.x) : mk(fmaf(w0.x, fr.x, w0.x), fmaf(w0.y, fr.x, w0.y));
+                    x1 = PHASE ? apply(w1, fr.y, fi.y) : mk(fmaf(w1.x, fr.y, w1.x), fmaf(w1.y, fr.y, w1.y));
+                } else {
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        cpx<T> &xe = h ? x1 : x0;
+                        const T fj = (T)((h ? hi : lo) + S * m);
+                        T f1r, f1i = (T)0, em1;
+                        if (PHASE) {
+                            Dyn<T>::f1((A * fj) * fj, (B * fj) * fj, &f1r, &f1i, &em1);
+                        } else {
+                            em1 = exp((A * fj) * fj) - 1.0;
+                            f1r = em1;
+                        }
+                        const T z = (D * fj) * fj, mag = (T)1 + em1;
+                        (h ? acc2 : acc).add_w(xe, mag * ((T)1 + z * ((T)1 + z * ((T)0.5 + z * (T)(1.0 / 6.0)))));
+                        const cpx<T> w = PR::mul_s(xe, PR::ld_s(row + (2 * pr + h) * G + g));
+                        xe = PHASE ? apply(w, f1r, f1i) : mk(w.x + w.x * f1r, w.y + w.y * f1r);
+                    }
+                }
+            }
+        }
+    }
+
+    // The same in loops over the copy in shared memory, for every mode:
     // mode 0: x <- stat1 dyn_b x (the first half-step of a trajectory)
     // mode 1: x <- stat2 dyn_a dyn_b x; returns sum exp(2 er_a r^2) |x_old|^2 (end-of-step norm / dr)
     // mode 2: x <- stat1 dyn_a x; returns sum |x_new|^2
-    // dyn = exp((er + i ei) r^2), er and ei multiplied by T^3.  The caller passes the summed
-    // coefficients times dr^2 (phase / pi): A for the magnitude, B for the phase, D = (er_a - er_b) dr^2
-    // for the norm weight; they are rounded once per step and multiply the exact j twice, so no
-    // rounding that repeats identically every step enters the arguments.
-    static __device__ typename NormSum<T>::type factor(cpx<T> *buf, const Tables<T> &tb, int g, int c, int l, int mode,
-                                                       T A, T B, T D, double *red)
+    static __device__ __noinline__ typename NormSum<T>::type factor(cpx<T> *buf, const Tables<T> &tb, int g, int c, int l,
+                                                                    int mode, T A, T B, T D, double *red)
     {
-        SqAcc<T> acc, acc_odd;   // even and odd j accumulate separately (two dependency chains)
-        // a medium with gamma_hat = 0 has no dynamic phase (B = 0 exactly): the FP32 form then skips
-        // the sine and cosine series, whose value would be exactly 0 -- the same arithmetic
-        if (sizeof(T) == 4 && B == (T)0) factor_pts<false>(buf, tb, g, c, l, mode, A, B, D, acc, acc_odd);
-        else factor_pts<true>(buf, tb, g, c, l, mode, A, B, D, acc, acc_odd);
+        SqAcc<T> acc;
+        const SC *tab = (mode == 1) ? tb.statV2 : tb.statV;
+#pragma unroll 1
+        for (int e = 0; e < E; ++e) {
+            const T fj = (T)jof(g, e);
+            T f1r, f1i, em1, z;
+            if constexpr (sizeof(T) == 4) {
+                const T j2 = fj * fj;
+                Dyn<T>::f1t(A * j2, ((T)3.14159265358979323846 * B) * j2, &f1r, &f1i, &em1);
+                z = D * j2;
+            } else {
+                Dyn<T>::f1((A * fj) * fj, (B * fj) * fj, &f1r, &f1i, &em1);
+                z = (D * fj) * fj;
+            }
+            const T mag = (T)1 + em1;
+            cpx<T> v = buf[e * G + g];
+            if (mode == 1) {
+                if constexpr (sizeof(T) == 4) acc.add_w(v, mag + mag * z);
+                else acc.add_w(v, mag * ((T)1 + z * ((T)1 + z * ((T)0.5 + z * (T)(1.0 / 6.0)))));
+            }
+            v = apply(PR::mul_s(v, stat(tb, tab, c, l, g, e, mode == 1)), f1r, f1i);
+            if (mode == 2) acc.add_w(v, (T)1);
+            buf[e * G + g] = v;
+        }
         if (mode == 0) return {};
-        acc.merge(acc_odd);
         return slot_norm_sum<T, G>(acc, red);
     }
 
@@ -822,124 +981,35 @@ template <typename T, int N, int V> struct Pointwise {
     static __device__ typename NormSum<T>::type factor_ksu(cpx<T> *buf, const Tables<T> &tb, int g, int l, int mode,
                                                            const KsuT<T> &ka, const KsuT<T> &kb, double *red)
     {
-        SqAcc<T> acc, acc_odd;
+        SqAcc<T> acc;
         const SC *tab = (mode == 1) ? tb.statV2 : tb.statV;
         const T hdt = (T)0.5 * tb.ksu_dt;
-#pragma unroll 1
-        for (int k = g; k < N / 2; k += G) {
-#pragma unroll
-            for (int par = 0; par < 2; ++par) {
-                const int j = 2 * k + par;
-                const int p = par ? K::odd_pos(k) : K::even_pos(k);
-                const T fj = (T)j;
-                T A = (T)0, t = (T)0, z = (T)0;
-                if (j > 0) {
-                    T vda = (T)0, via = (T)0, vdb = (T)0, vib = (T)0;
-                    if (mode != 0) ksu_point<T>(tb, ka, fj, vda, via);
-                    if (mode != 2) ksu_point<T>(tb, kb, fj, vdb, vib);
-                    A = (via + vib) * hdt;
-                    t = -(vda + vdb) * hdt;
-                    z = (via - vib) * hdt;   // |K_V(n)|^2 = exp(A + z)
-                }
-                T f1r, f1i, em1;
-                if constexpr (sizeof(T) == 4) Dyn<T>::f1t(A, t, &f1r, &f1i, &em1);
-                else Dyn<T>::f1(A, t * (T)0.318309886183790671537767526745, &f1r, &f1i, &em1);
-                const T mag = (T)1 + em1;
-                cpx<T> v = buf[p];
-                SqAcc<T> &ac = par ? acc_odd : acc;
-                if (mode == 1) ac.add_w(v, mag * exp(z));
-                const cpx<T> w = PR::mul_s(v, stat(tb, tab, 0, l, j, mode == 1));
-                v = mk(w.x + (w.x * f1r - w.y * f1i), w.y + (w.x * f1i + w.y * f1r));
-                if (mode == 2) ac.add_w(v, (T)1);
-                buf[p] = v;
+#pragma unroll 2
+        for (int e = 0; e < E; ++e) {
+            const int j = jof(g, e);
+            const T fj = (T)j;
+            T A = (T)0, t = (T)0, z = (T)0;
+            if (j > 0) {
+                T vda = (T)0, via = (T)0, vdb = (T)0, vib = (T)0;
+                if (mode != 0) ksu_point<T>(tb, ka, fj, vda, via);
+                if (mode != 2) ksu_point<T>(tb, kb, fj, vdb, vib);
+                A = (via + vib) * hdt;
+                t = -(vda + vdb) * hdt;
+                z = (via - vib) * hdt;   // |K_V(n)|^2 = exp(A + z)
             }
+            T f1r, f1i, em1;
+            if constexpr (sizeof(T) == 4) Dyn<T>::f1t(A, t, &f1r, &f1i, &em1);
+            else Dyn<T>::f1(A, t * (T)0.318309886183790671537767526745, &f1r, &f1i, &em1);
+            const T mag = (T)1 + em1;
+            cpx<T> v = buf[e * G + g];
+            if (mode == 1) acc.add_w(v, mag * exp(z));
+            const cpx<T> w = PR::mul_s(v, stat(tb, tab, 0, l, g, e, mode == 1));
+            v = mk(w.x + (w.x * f1r - w.y * f1i), w.y + (w.x * f1i + w.y * f1r));
+            if (mode == 2) acc.add_w(v, (T)1);
+            buf[e * G + g] = v;
         }
         if (mode == 0) return {};
-        acc.merge(acc_odd);
         return slot_norm_sum<T, G>(acc, red);
-    }
-
-    template <bool phase>
-    static __device__ __forceinline__ void factor_pts(cpx<T> *buf, const Tables<T> &tb, int g, int c, int l, int mode,
-                                                      T A, T B, T D, SqAcc<T> &acc, SqAcc<T> &acc_odd)
-    {
-        const SC *tab = (mode == 1) ? tb.statV2 : tb.statV;
-        const T Bpi = (T)3.14159265358979323846 * B;   // the phase coefficient: t = pi B j^2
-#pragma unroll 2
-        for (int k = g; k < N / 2; k += G) {
-            // FP32 at N = 2048 .. 8192: the series of the pair (2k, 2k+1) in packed FP32x2 instructions
-            // (bit-identical; +1.6% / +2.4% / +0.7% at N = 2048 / 4096 / 8192, -0.9% at 1024 and 16384)
-            float2 F1R, F1I = make_float2(0.f, 0.f), EM1, Z;
-            if constexpr (PD) {
-                const float j0 = (float)(2 * k), j1 = (float)(2 * k + 1);
-                const float2 j2 = __fmul2_rn(make_float2(j0, j1), make_float2(j0, j1));
-                const float2 a2 = __fmul2_rn(make_float2(A, A), j2);
-                if (phase) {
-                    Dyn<float>::f1t2(a2, __fmul2_rn(make_float2(Bpi, Bpi), j2), &F1R, &F1I, &EM1);
-                } else {
-                    EM1 = Dyn<float>::em1_2(a2);
-                    F1R = EM1;
-                }
-                Z = __fmul2_rn(make_float2(D, D), j2);
-            }
-#pragma unroll
-            for (int par = 0; par < 2; ++par) {
-                const int j = 2 * k + par;
-                const int p = par ? K::odd_pos(k) : K::even_pos(k);
-                const T fj = (T)j;
-                // the dynamic factor exp(a) exp(i pi y) is close to 1 and changes little from step to
-                // step; it is applied as w + w f1 with f1 its deviation from 1, evaluated so that the
-                // rounding is relative to f1, not to 1 (a rounding of a value next to 1 would repeat
-                // identically every step and add up)
-                T f1r, f1i = (T)0, em1;
-                T z = (T)0;
-                if constexpr (PD) {
-                    f1r = par ? F1R.y : F1R.x;
-                    f1i = par ? F1I.y : F1I.x;
-                    em1 = par ? EM1.y : EM1.x;
-                    z = par ? Z.y : Z.x;
-                } else if constexpr (sizeof(T) == 4) {
-                    // j^2 is exact in FP32 up to N = 4096 (and rounded once above); the coefficients
-                    // change every step, so no rounding of a, t or z repeats from step to step
-                    const T j2 = fj * fj;
-                    if (phase) {
-                        Dyn<T>::f1t(A * j2, Bpi * j2, &f1r, &f1i, &em1);
-                    } else {   // gamma_hat = 0: the phase is 0 and f1 = exp(a) - 1 exactly as f1t gives it
-                        em1 = Dyn<T>::em1(A * j2);
-                        f1r = em1;
-                    }
-                    z = D * j2;
-                } else {
-                    Dyn<T>::f1((A * fj) * fj, (B * fj) * fj, &f1r, &f1i, &em1);
-                    z = (D * fj) * fj;
-                }
-                const T mag = (T)1 + em1;   // |exp(a)|, for the norm weight (working precision suffices)
-                cpx<T> v = buf[p];
-                SqAcc<T> &ac = par ? acc_odd : acc;
-                if (mode == 1) {
-                    // exp(2 er_a r^2) = mag * exp((er_a - er_b) r^2), the second factor 1 + z with
-                    // |z| <~ 1e-4 (the temperature's change over one step): FP32 keeps the first order
-                    // (z^2 / 2 < 1e-8 is below its rounding), FP64 the series to z^3
-                    if constexpr (sizeof(T) == 4) ac.add_w(v, mag + mag * z);
-                    else ac.add_w(v, mag * ((T)1 + z * ((T)1 + z * ((T)0.5 + z * (T)(1.0 / 6.0)))));
-                }
-                const cpx<T> w = PR::mul_s(v, stat(tb, tab, c, l, j, mode == 1));
-                if constexpr (sizeof(T) == 4) {   // w + w f1, fused
-                    v = phase ? mk(fmaf(w.x, f1r, fmaf(-w.y, f1i, w.x)), fmaf(w.y, f1r, fmaf(w.x, f1i, w.y)))
-                              : mk(fmaf(w.x, f1r, w.x), fmaf(w.y, f1r, w.y));
-                } else {
-                    v = mk(w.x + (w.x * f1r - w.y * f1i), w.y + (w.x * f1i + w.y * f1r));
-                }
-                if (mode == 2) ac.add_w(v, (T)1);
-                buf[p] = v;
-            }
-        }
-    }
-
-    static __device__ cpx<double> to_d(const typename Prec<double>::C &a) { return a; }
-    static __device__ cpx<double> to_d(const typename Prec<float>::C &a)
-    {
-        return mk((double)a.rh + (double)a.rl, (double)a.ih + (double)a.il);
     }
 
     // A jump after the factor of mode 1 (more steps follow) or mode 2 (after the last step).
@@ -953,23 +1023,21 @@ template <typename T, int N, int V> struct Pointwise {
     {
         const T dr2 = (T)(tb.dr * tb.dr);
         SqAcc<T> acc;
-        for (int k = g; k < N / 2; k += G) {
-            for (int par = 0; par < 2; ++par) {
-                const int j = 2 * k + par;
-                const int p = par ? K::odd_pos(k) : K::even_pos(k);
-                const T fj = (T)j, j2 = fj * fj;
-                cpx<T> v = buf[p];
-                if (after_last) {
-                    acc.add_w(v, dr2 * j2);
-                } else {
-                    acc.add_w(v, dr2 * j2 * k_exp(w2 * j2));
-                    v = PR::mul_s(PR::mul_s(v, PR::conj_s(stat(tb, tb.statV, c, l, j, false))), stat(tb, tb.statV, c2, l2, j, false));
-                    T sn, cs;
-                    k_sincospi(B * j2, &sn, &cs);
-                    const T m = k_exp(A * j2);
-                    v = v * mk(m * cs, m * sn);
-                    buf[p] = v;
-                }
+#pragma unroll 1
+        for (int e = 0; e < E; ++e) {
+            const T fj = (T)jof(g, e), j2 = fj * fj;
+            cpx<T> v = buf[e * G + g];
+            if (after_last) {
+                acc.add_w(v, dr2 * j2);
+            } else {
+                acc.add_w(v, dr2 * j2 * k_exp(w2 * j2));
+                v = PR::mul_s(PR::mul_s(v, PR::conj_s(stat(tb, tb.statV, c, l, g, e, false))),
+                              stat(tb, tb.statV, c2, l2, g, e, false));
+                T sn, cs;
+                k_sincospi(B * j2, &sn, &cs);
+                const T m = k_exp(A * j2);
+                v = v * mk(m * cs, m * sn);
+                buf[e * G + g] = v;
             }
         }
         return slot_norm<T, G>(acc, red);
@@ -978,14 +1046,14 @@ template <typename T, int N, int V> struct Pointwise {
     // Per-step summary row of the end-of-step state e = stat1 exp(A j^2 + i pi B j^2) x, x the state
     // before the closing half-step (A = erj K3, B = eij T3 of the step): norm, <r>, overlaps, FP64
     // accumulation; thread 0 writes the row.  One pass for the norm and <r> and one per basis state
-    // of the same l, so that few values stay live.  Only in the traced kernel (V = 4).
-    static __device__ __forceinline__ cpx<double> end_value(const cpx<T> *buf, const Tables<T> &tb, int c, int l, int j,
-                                                            int p, T A, T B)
+    // of the same l, so that few values stay live.  Only in the traced kernels (V = 4, 6).
+    static __device__ __forceinline__ cpx<double> end_value(const cpx<T> *buf, const Tables<T> &tb, int c, int l, int g,
+                                                            int e, T A, T B)
     {
-        const T fj = (T)j;
+        const T fj = (T)jof(g, e);
         T f1r, f1i, em1;
         Dyn<T>::f1((A * fj) * fj, (B * fj) * fj, &f1r, &f1i, &em1);
-        const cpx<T> w = PR::mul_s(buf[p], stat(tb, tb.statV, c, l, j, false));
+        const cpx<T> w = PR::mul_s(buf[e * G + g], stat(tb, tb.statV, c, l, g, e, false));
         return mk((double)(w.x + (w.x * f1r - w.y * f1i)), (double)(w.y + (w.x * f1i + w.y * f1r)));
     }
 
@@ -993,14 +1061,13 @@ template <typename T, int N, int V> struct Pointwise {
                                      double *red, qtraj_trace_rec *out, int step)
     {
         double n2 = 0.0, rr = 0.0;
-        for (int k = g; k < N / 2; k += G)
-            for (int par = 0; par < 2; ++par) {
-                const int j = 2 * k + par;
-                const cpx<double> e = end_value(buf, tb, c, l, j, par ? K::odd_pos(k) : K::even_pos(k), A, B);
-                const double m2 = e.x * e.x + e.y * e.y;
-                n2 += m2;
-                rr += (double)j * tb.dr * m2;
-            }
+#pragma unroll 1
+        for (int e = 0; e < E; ++e) {
+            const cpx<double> v = end_value(buf, tb, c, l, g, e, A, B);
+            const double m2 = v.x * v.x + v.y * v.y;
+            n2 += m2;
+            rr += (double)jof(g, e) * tb.dr * m2;
+        }
         n2 = slot_sum<G>(n2, red);
         rr = slot_sum<G>(rr, red);
         const double dr = tb.dr;
@@ -1017,14 +1084,13 @@ template <typename T, int N, int V> struct Pointwise {
             const int bl = s == 2 || s == 4 ? 1 : (s == 5 ? 2 : 0);
             double vr = 0.0, vi = 0.0;
             if (c == 0 && bl == l) {
-                for (int k = g; k < N / 2; k += G)
-                    for (int par = 0; par < 2; ++par) {
-                        const int j = 2 * k + par;
-                        const cpx<double> e = end_value(buf, tb, c, l, j, par ? K::odd_pos(k) : K::even_pos(k), A, B);
-                        const double ph = tb.eig[(size_t)s * N + j];
-                        vr += ph * e.x;
-                        vi += ph * e.y;
-                    }
+#pragma unroll 1
+                for (int e = 0; e < E; ++e) {
+                    const cpx<double> v = end_value(buf, tb, c, l, g, e, A, B);
+                    const double phi = tb.eig[(size_t)s * N + jof(g, e)], ph = odd_half(e) ? -phi : phi;
+                    vr += ph * v.x;
+                    vi += ph * v.y;
+                }
                 vr = slot_sum<G>(vr, red);
                 vi = slot_sum<G>(vi, red);
             }
@@ -1037,16 +1103,13 @@ template <typename T, int N, int V> struct Pointwise {
     // at a jump cap.
     static __device__ void undo_start(cpx<T> *buf, const Tables<T> &tb, int g, int c, int l, T A, T B)
     {
-        for (int k = g; k < N / 2; k += G) {
-            for (int par = 0; par < 2; ++par) {
-                const int j = 2 * k + par;
-                const int p = par ? K::odd_pos(k) : K::even_pos(k);
-                const T fj = (T)j, j2 = fj * fj;
-                T sn, cs;
-                k_sincospi(B * j2, &sn, &cs);
-                const T m = k_exp(A * j2);
-                buf[p] = PR::mul_s(buf[p], PR::conj_s(stat(tb, tb.statV, c, l, j, false))) * mk(m * cs, m * sn);
-            }
+#pragma unroll 1
+        for (int e = 0; e < E; ++e) {
+            const T fj = (T)jof(g, e), j2 = fj * fj;
+            T sn, cs;
+            k_sincospi(B * j2, &sn, &cs);
+            const T m = k_exp(A * j2);
+            buf[e * G + g] = PR::mul_s(buf[e * G + g], PR::conj_s(stat(tb, tb.statV, c, l, g, e, false))) * mk(m * cs, m * sn);
         }
     }
 
@@ -1054,13 +1117,8 @@ template <typename T, int N, int V> struct Pointwise {
     static __device__ void scale_r(cpx<T> *buf, const Tables<T> &tb, int g, double f)
     {
         const T s = (T)(tb.dr * f);
-        for (int k = g; k < N / 2; k += G) {
-            for (int par = 0; par < 2; ++par) {
-                const int j = 2 * k + par;
-                const int p = par ? K::odd_pos(k) : K::even_pos(k);
-                buf[p] = scale(buf[p], (T)j * s);
-            }
-        }
+#pragma unroll 1
+        for (int e = 0; e < E; ++e) buf[e * G + g] = scale(buf[e * G + g], (T)jof(g, e) * s);
     }
 };
 
@@ -1145,43 +1203,42 @@ __device__ int fetch_trajectory(const Tables<T> &tb, const LaunchArgs &a)
 }
 
 // Occupancy target of a kernel variant: variant 0 asks for 512 resident threads per SM in FP32
-// (<= 128 registers; at N = 4096 four CTAs of 128 threads, measured 8% faster on GB300 than three at
-// <= 168 registers once the static tables lost their low parts and the norm sums their compensation);
-// variant 1 asks for 640 (<= 102 registers, at the price of more spills), variants 2 and 3 (radix 8)
-// for 768 and 1024.  FP64 holds twice the state and takes what the compiler needs.
+// (<= 128 registers); variant 1 asks for 640 (<= 102 registers, at the price of spills), variants 2 and 3
+// (radix 8) for 768 and 1024.  FP64 holds twice the state and takes what the compiler needs.
 template <typename T, int N, int V> struct FusedBounds {
-    static constexpr int G = FusedPlan<N, V>::G;
-    static constexpr int THREADS = (V == 0 || V == 4 || V == 5) ? 512 : V == 1 ? 640 : V == 2 ? 768 : 1024;
+    static constexpr int G = FusedPlan<T, N, V>::G;
+    static constexpr int THREADS = V == 1 ? 640 : V == 2 || V == 6 ? 768 : V == 3 ? 1024 : 512;
     static constexpr int MB = THREADS / G > 32 ? 32 : (THREADS / G > 0 ? THREADS / G : 1);
     static constexpr int MIN_BLOCKS = sizeof(T) == 4 ? MB : 1;
 };
 
 template <typename T, int N, int V>
-__global__ void __launch_bounds__(FusedPlan<N, V>::G, (FusedBounds<T, N, V>::MIN_BLOCKS)) fused_kernel(Tables<T> tb, LaunchArgs a)
+__global__ void __launch_bounds__(FusedPlan<T, N, V>::G, (FusedBounds<T, N, V>::MIN_BLOCKS)) fused_kernel(Tables<T> tb, LaunchArgs a)
 {
-    using K = Fused<T, N, V>;
+    using P = FusedPlan<T, N, V>;
+    using K = Sine<T, N, V>;
     using PW = Pointwise<T, N, V>;
-    constexpr int G = K::G, E = K::E;
+    using NS2 = typename NormSum<T>::type;
+    constexpr int G = P::G, E = P::E, NS = P::NS;
+    constexpr bool KSU = V == 5;                  // the isotropic KSU potential: H_eff only, no jumps
+    constexpr bool TRACED = V == 4 || V == 6;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cpx<T> *buf = reinterpret_cast<cpx<T> *>(smem_raw);
-    using C = typename Prec<T>::C;
-    using P = FusedPlan<N, V>;
-    C *tw1 = reinterpret_cast<C *>(buf + P::BUF);
-    C *tw2 = tw1 + P::TW1;
-    Carry<T> *wtot = reinterpret_cast<Carry<T> *>(tw2 + P::TW2);
-    double *red = reinterpret_cast<double *>(wtot + (G / 32 + 1));
+    double *red = reinterpret_cast<double *>(buf + P::BUF);         // reductions of the rare paths
+    NS2 *redh = reinterpret_cast<NS2 *>(red + (G / 32 + 1));        // the step's norm
     __shared__ int s_traj;
-    // middle-pass twiddles, row m of a table holding W^(m k) for every k (tw1: [M1][R] of W_{R M1},
-    // tw2: [M2][R M1] of W_{R M1 M2}, the second only with a second middle pass), built once per CTA
-    for (int t = threadIdx.x; t < P::TW1; t += G)
-        tw1[t] = Prec<T>::ld(&tb.W[(t / P::R) * (t % P::R) * (N / P::TW1)]);
-    if (P::M2 > 1)
-        for (int t = threadIdx.x; t < P::TW2; t += G)
-            tw2[t] = Prec<T>::ld(&tb.W[(t / P::TW1) * (t % P::TW1) * (N / P::TW2)]);
 
     const int g = threadIdx.x;
     const double dr = tb.dr;
-    cpx<T> x[E];
+    int pb[NS], pm[NS];
+#pragma unroll
+    for (int t = 0; t < NS; ++t) {
+        int lo, hi;
+        slot_points(g + t * G, P::R, P::M, lo, hi);
+        pb[t] = K::pos(lo);
+        pm[t] = K::pos(P::S - lo);   // (slot 0 does not use them)
+    }
+    cpx<T> x[P::XN];
 
     for (;;) {
         if (g == 0) s_traj = fetch_trajectory(tb, a);
@@ -1191,114 +1248,138 @@ __global__ void __launch_bounds__(FusedPlan<N, V>::G, (FusedBounds<T, N, V>::MIN
         if (wk < 0) break;
         const bool grp = wk < a.n_groups;     // a group's no-jump run of this launch
         const int t = grp ? wk : wk - a.n_groups;
-        constexpr bool KSU = V == 5;           // the isotropic KSU potential: H_eff only, no jumps
         const bool nojump = a.nojump || grp || KSU;
 
-        const TrajDev d = grp ? a.gtrajs[t] : a.trajs[t];
-        const MediumDev md = tb.media[d.medium];
-        int l = tb.spec_l[d.spec], c = tb.spec_color[d.spec];
-        if (tb.ic_cplx) {
-            const double *ic = tb.ic + (size_t)d.spec * 2 * N;
-            for (int k = g; k < N / 2; k += G) {
-                buf[K::even_pos(k)] = mk<T>((T)ic[4 * k], (T)ic[4 * k + 1]);
-                buf[K::odd_pos(k)] = mk<T>((T)ic[4 * k + 2], (T)ic[4 * k + 3]);
-            }
-        } else {
-            const double *ic = tb.ic + (size_t)d.spec * N;
-            for (int k = g; k < N / 2; k += G) {
-                buf[K::even_pos(k)] = mk<T>((T)ic[2 * k], (T)0);
-                buf[K::odd_pos(k)] = mk<T>((T)ic[2 * k + 1], (T)0);
+        const TrajDev *dp = grp ? a.gtrajs + t : a.trajs + t;
+        const int spec = dp->spec, ns = dp->n_steps;
+        const MediumDev *mp = tb.media + dp->medium;
+        int l = tb.spec_l[spec], c = tb.spec_color[spec];
+        {
+            const double *ic = tb.ic + (size_t)spec * N * (tb.ic_cplx ? 2 : 1);
+#pragma unroll 4
+            for (int e = 0; e < E; ++e) {
+                const int j = PW::jof(g, e);
+                T re, im = (T)0;
+                if (tb.ic_cplx) {
+                    re = (T)ic[2 * j];
+                    im = (T)ic[2 * j + 1];
+                } else {
+                    re = (T)ic[j];
+                }
+                buf[e * G + g] = PW::odd_half(e) ? mk(-re, -im) : mk(re, im);
             }
         }
         uint32_t kdraw = 0;
-        Draws dw = draws(d.seed, 0u);
-        const double r0 = nojump ? 0.0 : dw.r;   // (no draw is used without jumps)
         Threshold<T> thr;
-        thr.set(nojump ? -1.0 : dw.r, dr);
-        int nj = 0, flags = 0, fj = -1, lj = -1, ended = 0, executed = 0;
-        uint32_t digest = DIGEST_BASIS;
         // r0 > r_max reaches here only when its group's no-jump record was not yet published: the paper
         // resolves r0 < p_NoJump by the shortcut first and r0 > r_max only otherwise.  The trajectory
         // is evolved: if its norm never falls to r0 it is the no-jump run (= the shortcut's record); the
         // first trigger shows r0 >= p_NoJump (the norm only decreases), and it ends as r_max does.
-        const bool rmax_pending = !nojump && !KSU && dw.r > tb.r_max;
+        bool rmax_pending = false;
+        {
+            const double r = nojump ? -1.0 : draws(dp->seed, 0u).r;   // (no draw is used without jumps)
+            thr.set(r, dr);
+            rmax_pending = !nojump && r > tb.r_max;
+        }
+        int nj = 0, flags = 0, fj = -1, lj = -1, ended = 0, executed = 0;
+        uint32_t digest = DIGEST_BASIS;
         bool rmax_hit = false;
-        const bool traced = V == 4 && !grp && a.trace_every > 0 && t < a.trace_n;
+        const bool traced = TRACED && !grp && a.trace_every > 0 && t < a.trace_n;
         int nrec = 0;
-        const int ns = d.n_steps;
-        // per-step scalars in the working precision: T^3 = A / (tau0 + n dtau)
-        const T mA = (T)md.A, mtau0 = (T)md.tau0, mdtau = (T)md.dtau;
-        const bool tabulated = md.kind == 1;
         int seg = 0;
         // T(tau_n)^3: Bjorken, or the table at tau_n = tau_1 + n dtau (out of line: rare, and inline it
         // would hold registers in the step loop)
         auto T3_of = [&](int n) -> T {
-            return tabulated ? table_T3_far<T>(tb.prof + 2 * (size_t)md.tab_off, md.tab_len, mtau0 + (T)n * mdtau, &seg)
-                             : mA / (mtau0 + (T)n * mdtau);
+            const T tau = (T)mp->tau0 + (T)n * (T)mp->dtau;
+            return mp->kind == 1 ? table_T3_far<T>(tb.prof + 2 * (size_t)mp->tab_off, mp->tab_len, tau, &seg)
+                                 : (T)mp->A / tau;
         };
         T T3b = T3_of(0);
-        T K3b = kappa_T3<T>(md.kfit, T3b);   // kappa_hat(T) T^3 when kappa_hat follows a lattice fit
+        T K3b = kappa_T3<T>(mp->kfit, T3b);   // kappa_hat(T) T^3 when kappa_hat follows a lattice fit
         KsuT<T> kb{};
         if constexpr (KSU) kb = ksu_at<T>(tb, T3b);
         if (ns > 0) {
-            __syncthreads();
             if constexpr (KSU) PW::factor_ksu(buf, tb, g, l, 0, kb, kb, red);
-            else PW::factor(buf, tb, g, c, l, 0, (T)md.erj[c] * K3b, (T)md.eij[c] * T3b, (T)0, red);
+            else PW::factor(buf, tb, g, c, l, 0, (T)mp->erj[c] * K3b, (T)mp->eij[c] * T3b, (T)0, red);
+            PW::to_regs(x, buf, g);
+            traj_sync<G>();   // the copies are read before the first pass writes its sequences
         }
 
         for (int n = 0; n < ns; ++n) {
             const T T3a = T3b, K3a = K3b;
             const bool last = (n + 1 == ns);
             T3b = T3_of(n + 1);
-            K3b = kappa_T3<T>(md.kfit, T3b);
-            __syncthreads();
+            K3b = kappa_T3<T>(mp->kfit, T3b);
 #pragma unroll 1
-            for (int h = 0; h < 2; ++h) K::dst(x, buf, tb, g, wtot, tw1, tw2, h == 1);
+            for (int h = 0; h < 2; ++h) {
+                K::first(x, buf, tb.TA, g, pb, pm);
+                traj_sync<G>();
+                K::mid(x, buf, tb.TM, tb.TI, tb.TS, g);
+                traj_sync<G>();
+                K::last(x, buf, tb.TM, g);
+                if (h == 0) {
+                    K::kinetic(x, tb.KF, g);
+                    traj_sync<G>();
+                }
+            }
             executed = n + 1;
-            const T erj = (T)md.erj[c], eij = (T)md.eij[c];
-            if constexpr (V == 4) {   // the traced twin of variant 0: per-step summary rows
+            const T erj = (T)mp->erj[c], eij = (T)mp->eij[c];
+            bool in_smem = false;   // the state is in the shared-memory copy (else in the registers)
+            if constexpr (TRACED) {   // per-step summary rows
                 if (traced && ((n + 1) % a.trace_every == 0 || last) && nrec < a.trace_cap) {
+                    traj_sync<G>();
+                    PW::to_smem(x, buf, g);
                     PW::trace_row(buf, tb, g, c, l, erj * K3a, eij * T3a, red,
                                   a.trace + (size_t)t * a.trace_cap + nrec, n + 1);
                     ++nrec;
-                    __syncthreads();
                 }
             }
             const T Tsum = last ? T3a : T3a + T3b, Ksum = last ? K3a : K3a + K3b;
-            typename NormSum<T>::type n2s;   // norm^2 / dr
-            if constexpr (KSU) {
-                const KsuT<T> ka = kb;
-                kb = ksu_at<T>(tb, T3b);
-                n2s = PW::factor_ksu(buf, tb, g, l, last ? 2 : 1, ka, kb, red);
+            const T cA = erj * Ksum, cB = eij * Tsum, cD = last ? (T)0 : erj * (K3a - K3b);
+            NS2 n2s;   // norm^2 / dr
+            // (phases beyond 1e5: far2's reduction would lose them)
+            if (KSU || last || l >= LTAB || !(fabs(cB) * (T)N * (T)N < (T)3e4)) {
+                traj_sync<G>();   // all have read the transform's output
+                PW::to_smem(x, buf, g);
+                in_smem = true;
+                if constexpr (KSU) {
+                    const KsuT<T> ka = kb;
+                    kb = ksu_at<T>(tb, T3b);
+                    n2s = PW::factor_ksu(buf, tb, g, l, last ? 2 : 1, ka, kb, red);
+                } else {
+                    n2s = PW::factor(buf, tb, g, c, l, last ? 2 : 1, cA, cB, cD, red);
+                }
             } else {
-                n2s = PW::factor(buf, tb, g, c, l, last ? 2 : 1, erj * Ksum, eij * Tsum,
-                                 last ? (T)0 : erj * (K3a - K3b), red);
+                SqAcc<T> acc, acc2;
+                const typename Prec<T>::S *row = tb.statV2 + ((size_t)c * LTAB + l) * N;
+                if (cB == (T)0) PW::template factor_regs<false>(x, row, g, cA, cB, cD, acc, acc2);
+                else PW::template factor_regs<true>(x, row, g, cA, cB, cD, acc, acc2);
+                acc.merge(acc2);
+                n2s = step_norm<T, G>(acc, redh);   // synchronises: all have read the transform's output
             }
+            bool stop = false;
             if (!thr.finite(n2s)) {
                 flags |= QTRAJ_F_NONFINITE;
                 ended = 1;
                 if (g == 0) atomicOr(a.status, 1);
-                break;
-            }
-            if (!nojump) {
+                stop = true;
+            } else if (!nojump) {
                 if (thr.near(n2s, border_eps<T>())) flags |= QTRAJ_F_BORDERLINE;
-                const bool trig = thr.reached(n2s);
-                if (trig && rmax_pending) {
-                    rmax_hit = true;
-                    ended = 1;
-                    break;
-                }
-                if (trig) {
+                if (thr.reached(n2s)) {
+                    if (!in_smem) PW::to_smem(x, buf, g);
+                    in_smem = true;
+                    const Draws dw = draws(dp->seed, kdraw);
                     // a trajectory stopped by a cap keeps its end-of-step state
                     const bool cap_j = tb.max_jumps >= 0 && nj >= tb.max_jumps;
                     const int l_new = (dw.ul < (double)l / (2.0 * l + 1.0)) ? l - 1 : l + 1;
                     const int c_new = (c == 1 && dw.uc < tb.p_os) ? 0 : 1;
                     const bool cap_l = !cap_j && tb.l_cap >= 0 && l_new > tb.l_cap;
-                    if (cap_j || cap_l) {
-                        if (!last) {
-                            __syncthreads();
-                            PW::undo_start(buf, tb, g, c, l, -(T)md.erj[c] * K3b, -(T)md.eij[c] * T3b);
-                        }
+                    if (rmax_pending) {
+                        rmax_hit = true;
+                        ended = 1;
+                        stop = true;
+                    } else if (cap_j || cap_l) {
+                        if (!last) PW::undo_start(buf, tb, g, c, l, -(T)mp->erj[c] * K3b, -(T)mp->eij[c] * T3b);
                         ended = 1;
                         if (cap_j) {
                             flags |= QTRAJ_F_MAXJUMPS;
@@ -1309,36 +1390,41 @@ __global__ void __launch_bounds__(FusedPlan<N, V>::G, (FusedBounds<T, N, V>::MIN
                             lj = n;
                             digest = digest_jump(digest, n, l, c);
                         }
-                        break;
+                        stop = true;
+                    } else {
+                        if (fj < 0) fj = n;
+                        // r times the end-of-step state, renormalised; the start half-step already applied
+                        // is turned into the new colour's and l's
+                        const double dr2 = tb.dr * tb.dr, T3d = (double)T3b, K3d = (double)K3b;
+                        const T w2 = last ? (T)0 : (T)(-2.0 * mp->er[c] * K3d * dr2);
+                        const T dA = last ? (T)0 : (T)((mp->er[c_new] - mp->er[c]) * K3d * dr2);
+                        const T dB = last ? (T)0 : (T)((mp->ei[c_new] - mp->ei[c]) * T3d * dr2 * 0.31830988618379067154);
+                        const double s = PW::jump_turn(buf, tb, g, c, l, c_new, l_new, last, w2, dA, dB, red) * dr;
+                        PW::scale_r(buf, tb, g, 1.0 / sqrt(s));
+                        l = l_new; c = c_new; ++nj;
+                        lj = n;
+                        digest = digest_jump(digest, n, l, c);
+                        ++kdraw;
+                        thr.set(draws(dp->seed, kdraw).r, dr);
                     }
-                    if (fj < 0) fj = n;
-                    // r times the end-of-step state, renormalised; the start half-step already applied
-                    // is turned into the new colour's and l's
-                    __syncthreads();
-                    const double dr2 = tb.dr * tb.dr, T3d = (double)T3b, K3d = (double)K3b;
-                    const T w2 = last ? (T)0 : (T)(-2.0 * md.er[c] * K3d * dr2);
-                    const T dA = last ? (T)0 : (T)((md.er[c_new] - md.er[c]) * K3d * dr2);
-                    const T dB = last ? (T)0 : (T)((md.ei[c_new] - md.ei[c]) * T3d * dr2 * 0.31830988618379067154);
-                    const double s = PW::jump_turn(buf, tb, g, c, l, c_new, l_new, last, w2, dA, dB, red) * dr;
-                    const double f = 1.0 / sqrt(s);
-                    __syncthreads();
-                    PW::scale_r(buf, tb, g, f);
-                    l = l_new; c = c_new; ++nj;
-                    lj = n;
-                    digest = digest_jump(digest, n, l, c);
-                    ++kdraw;
-                    dw = draws(d.seed, kdraw);
-                    thr.set(dw.r, dr);
                 }
             }
+            if (stop) {
+                if (!in_smem) PW::to_smem(x, buf, g);
+                break;
+            }
+            if (in_smem && !last) {
+                PW::to_regs(x, buf, g);
+                traj_sync<G>();
+            }
         }
-        __syncthreads();
 
-        // observables (FP64)
+        // observables (FP64) from the shared-memory copy
         double acc = 0.0;
-        for (int k = g; k < N / 2; k += G) {
-            const cpx<T> a0 = buf[K::even_pos(k)], a1 = buf[K::odd_pos(k)];
-            acc += (double)a0.x * a0.x + (double)a0.y * a0.y + (double)a1.x * a1.x + (double)a1.y * a1.y;
+#pragma unroll 4
+        for (int e = 0; e < E; ++e) {
+            const cpx<T> v = buf[e * G + g];
+            acc += (double)v.x * v.x + (double)v.y * v.y;
         }
         const double n2 = slot_sum<G>(acc, red) * dr;
         double ovr[NBASIS], ovi[NBASIS];
@@ -1350,28 +1436,29 @@ __global__ void __launch_bounds__(FusedPlan<N, V>::G, (FusedBounds<T, N, V>::MIN
             if (ended || c != 0 || basis_l[s] != l) continue;
             const double *phi = tb.eig + (size_t)s * N;
             double pr = 0.0, pi = 0.0;
-            for (int k = g; k < N / 2; k += G) {
-                const cpx<T> a0 = buf[K::even_pos(k)], a1 = buf[K::odd_pos(k)];
-                const double f0 = phi[2 * k], f1 = phi[2 * k + 1];
-                pr += f0 * (double)a0.x + f1 * (double)a1.x;
-                pi += f0 * (double)a0.y + f1 * (double)a1.y;
+#pragma unroll 4
+            for (int e = 0; e < E; ++e) {
+                const cpx<T> v = buf[e * G + g];
+                const double f = phi[PW::jof(g, e)], fs = PW::odd_half(e) ? -f : f;
+                pr += fs * (double)v.x;
+                pi += fs * (double)v.y;
             }
             ovr[s] = slot_sum<G>(pr, red) * dr;
             ovi[s] = slot_sum<G>(pi, red) * dr;
         }
         if (a.states && !grp) {
             double *st = a.states + (size_t)t * N * 2;
-            for (int k = g; k < N / 2; k += G) {
-                const cpx<T> a0 = buf[K::even_pos(k)], a1 = buf[K::odd_pos(k)];
-                st[4 * k] = (double)a0.x;
-                st[4 * k + 1] = (double)a0.y;
-                st[4 * k + 2] = (double)a1.x;
-                st[4 * k + 3] = (double)a1.y;
+#pragma unroll 4
+            for (int e = 0; e < E; ++e) {
+                const cpx<T> v = buf[e * G + g];
+                const int j = PW::jof(g, e);
+                const double sg = PW::odd_half(e) ? -1.0 : 1.0;
+                st[2 * j] = sg * (double)v.x;
+                st[2 * j + 1] = sg * (double)v.y;
             }
         }
         if (g == 0) {
             qtraj_obs o;
-            const int sp = d.spec;
             for (int s = 0; s < NBASIS; ++s) {
                 o.ov_re[s] = ovr[s];
                 o.ov_im[s] = ovi[s];
@@ -1380,16 +1467,16 @@ __global__ void __launch_bounds__(FusedPlan<N, V>::G, (FusedBounds<T, N, V>::MIN
                     // with jumps the estimator takes the normalised state; without (KSU) the norm lost
                     // to V_I is the dissociation, and the overlap is taken unnormalised
                     const double prob = (ovr[s] * ovr[s] + ovi[s] * ovi[s]) / (KSU ? 1.0 : n2);
-                    if (tb.ov0_zero[sp * NBASIS + s]) sv = prob;
+                    if (tb.ov0_zero[spec * NBASIS + s]) sv = prob;
                     else {
-                        const double a0 = tb.ov0[(sp * NBASIS + s) * 2], b0 = tb.ov0[(sp * NBASIS + s) * 2 + 1];
+                        const double a0 = tb.ov0[(spec * NBASIS + s) * 2], b0 = tb.ov0[(spec * NBASIS + s) * 2 + 1];
                         sv = prob / (a0 * a0 + b0 * b0);
                     }
                 }
                 o.surv[s] = sv;
             }
             o.norm2 = n2;
-            o.r0 = r0;
+            o.r0 = nojump ? 0.0 : draws(dp->seed, 0u).r;
             o.l = l;
             o.color = c;
             o.n_jumps = nj;
@@ -1401,8 +1488,8 @@ __global__ void __launch_bounds__(FusedPlan<N, V>::G, (FusedBounds<T, N, V>::MIN
             if (rmax_hit) {   // the r_max record, with the steps that found r0 >= p_NoJump
                 for (int s = 0; s < NBASIS; ++s) { o.surv[s] = 0; o.ov_re[s] = 0; o.ov_im[s] = 0; }
                 o.norm2 = 1.0;
-                o.l = tb.spec_l[d.spec];
-                o.color = tb.spec_color[d.spec];
+                o.l = tb.spec_l[spec];
+                o.color = tb.spec_color[spec];
                 o.flags = flags | QTRAJ_F_RMAX;
             }
             if (grp) {
@@ -1421,23 +1508,17 @@ __global__ void __launch_bounds__(FusedPlan<N, V>::G, (FusedBounds<T, N, V>::MIN
 // shared-memory bytes of one CTA
 template <typename T, int N, int V> constexpr int fused_smem_bytes()
 {
-    using P = FusedPlan<N, V>;
-    return P::BUF * (int)sizeof(cpx<T>) +
-           (P::TW1 + P::TW2) *
-               (int)sizeof(typename Prec<T>::C) +
-           (P::G / 32 + 1) * (int)sizeof(Carry<T>) + (P::G / 32 + 1) * 8 + 16;
+    using P = FusedPlan<T, N, V>;
+    return P::BUF * (int)sizeof(cpx<T>) + (P::G / 32 + 1) * 16;
 }
 
-// Launches fused_kernel<T, N, V> as one persistent wave (SMs x resident CTAs, at most max_ctas when
+// Launches a trajectory kernel as one persistent wave (SMs x resident CTAs, at most max_ctas when
 // max_ctas > 0, at most one CTA per trajectory) after setting its shared-memory size; fills info
-// (query_only: launches nothing).  Every instantiation unit dispatches its grid sizes to this helper.
-template <typename T, int N, int V>
-cudaError_t fused_go(const Tables<T> &tb, const LaunchArgs &a, int sm_count, int max_ctas, cudaStream_t s,
-                     FusedInfo *info, bool query_only)
+// (query_only: launches nothing).
+template <typename T>
+cudaError_t launch_wave(void (*k)(Tables<T>, LaunchArgs), int G, int R, int smem, const Tables<T> &tb, const LaunchArgs &a,
+                        int sm_count, int max_ctas, cudaStream_t s, FusedInfo *info, bool query_only)
 {
-    auto k = fused_kernel<T, N, V>;
-    constexpr int G = FusedPlan<N, V>::G;
-    constexpr int smem = fused_smem_bytes<T, N, V>();
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     int occ = 0;
@@ -1449,7 +1530,7 @@ cudaError_t fused_go(const Tables<T> &tb, const LaunchArgs &a, int sm_count, int
         e = cudaFuncGetAttributes(&fa, k);
         if (e != cudaSuccess) return e;
         info->G = G;
-        info->R = FusedPlan<N, V>::R;
+        info->R = R;
         info->smem = smem;
         info->ctas_per_sm = occ;
         info->regs = fa.numRegs;
@@ -1461,6 +1542,16 @@ cudaError_t fused_go(const Tables<T> &tb, const LaunchArgs &a, int sm_count, int
     if (grid > work) grid = work;
     k<<<(int)grid, G, smem, s>>>(tb, a);
     return cudaGetLastError();
+}
+
+// Every instantiation unit dispatches its grid sizes to this helper.
+template <typename T, int N, int V>
+cudaError_t fused_go(const Tables<T> &tb, const LaunchArgs &a, int sm_count, int max_ctas, cudaStream_t s,
+                     FusedInfo *info, bool query_only)
+{
+    using P = FusedPlan<T, N, V>;
+    return launch_wave(fused_kernel<T, N, V>, P::G, P::R, fused_smem_bytes<T, N, V>(), tb, a, sm_count, max_ctas, s, info,
+                       query_only);
 }
 
 } // namespace qt

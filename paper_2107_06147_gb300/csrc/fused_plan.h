@@ -1,0 +1,97 @@
+// fused_plan.h -- the decomposition of the fused kernel's sine transform for every grid size, shared by
+// the kernel and by the host code that lays its tables out.
+//
+// The DST-I of N points is the length-2N FFT of the odd extension, done as a radix-R pass, a middle
+// transform of M = 2N/R^2 points (one pass M1, or two passes M1 x M2) and a radix-R pass, of which only
+// the half that the odd symmetry leaves independent is computed (fused.cuh).  The state lives in registers
+// as N/R "slots" of R values; slot s, value m is the grid point
+//     j = lo + S m (m < R/2),   hi + S (R-1-m) (m >= R/2),      S = 2N/R = R M,
+// whose register holds u_j for m < R/2 and -u_j for m >= R/2 (the odd extension at lo + S m).  Thread g of
+// G = N/E holds the slots g, g + G, ... (E/R of them).
+#pragma once
+#include <cuda_runtime.h>
+
+namespace qt {
+
+struct PlanDims { int R, E, M1, M2; };
+
+// rad8: the radix-8 plans of the launch variants 2 and 3 (FP32, N = 2048 and 4096)
+__host__ __device__ constexpr PlanDims plan_dims(int N, bool f64, bool rad8)
+{
+    if (rad8 && !f64 && N == 2048) return {8, 16, 8, 8};
+    if (rad8 && !f64 && N == 4096) return {8, 16, 16, 8};
+    switch (N) {
+    case 16: return {4, 4, 2, 1};
+    case 32: return {4, 4, 4, 1};
+    case 64: return {4, 4, 8, 1};
+    case 128: return {8, 8, 4, 1};
+    case 256: return {8, 8, 8, 1};
+    case 512: return f64 ? PlanDims{8, 8, 16, 1} : PlanDims{16, 16, 4, 1};
+    case 1024: return {16, 16, 8, 1};
+    case 2048: return {16, 16, 16, 1};
+    case 4096: return f64 ? PlanDims{16, 32, 32, 1} : PlanDims{16, 16, 32, 1};
+    case 8192: return {32, 32, 16, 1};
+    default: return {32, 32, 32, 1};   // 16384
+    }
+}
+
+// The slot's base points.  Slot s = kk M + q1 belongs to the residue b = kk + R q1 modulo S and holds the
+// points j = +-b (mod S).  kk = 0 holds the residues 0 and R/2 modulo R: q1 = 0 the points that are
+// multiples of S/2 (two half-length sequences in one slot), 0 < q1 < M/2 the residue R q1, and
+// q1 >= M/2 the residue R/2 + R q1.
+__host__ __device__ __forceinline__ void slot_points(int s, int R, int M, int &lo, int &hi)
+{
+    const int S = R * M, kk = s / M, q1 = s % M;
+    if (s == 0) {
+        lo = 0;
+        hi = S / 2;
+        return;
+    }
+    const int b = kk ? kk + R * q1 : (q1 < M / 2 ? R * q1 : R / 2 + R * q1);
+    lo = b;
+    hi = S - b;
+}
+
+// grid point of element e (slot e / R of thread g, value e % R)
+__host__ __device__ __forceinline__ int plan_j(int g, int e, int R, int M, int G)
+{
+    int lo, hi;
+    slot_points(g + (e / R) * G, R, M, lo, hi);
+    const int m = e % R;
+    return m < R / 2 ? lo + R * M * m : hi + R * M * (R - 1 - m);
+}
+
+// Tables with one entry per grid point are laid out in the order the threads read them: the pair of
+// elements (m, R-1-m) of a slot together, threads side by side.  16-byte entries (kinetic factors, FP64
+// static factors): two rows of G entries per pair; 8-byte entries (FP32 static factors): the two entries
+// of a thread's pair adjacent, one 16-byte load.  Element e of the entry at index i of thread g:
+__host__ __device__ __forceinline__ void plan_entry(int i, bool adjacent, int R, int G, int &g, int &e)
+{
+    int pr, h;
+    if (adjacent) {
+        pr = i / 2 / G;
+        g = i / 2 % G;
+        h = i & 1;
+    } else {
+        pr = i / (2 * G);
+        h = i / G % 2;
+        g = i % G;
+    }
+    const int t = pr / (R / 2), m = pr % (R / 2);
+    e = t * R + (h ? R - 1 - m : m);
+}
+
+// host view of a plan
+struct Plan {
+    int N, R, E, M, M1, M2, G, S, NS;
+    bool tw_last;   // W_S^{b1 q1} is applied by the last pass (else by the middle one)
+};
+__host__ __device__ constexpr bool plan_tw_last(PlanDims d) { return d.M2 > 1 || d.M1 >= d.R; }
+inline Plan make_plan(int N, bool f64, int variant)
+{
+    const PlanDims d = plan_dims(N, f64, variant == 2 || variant == 3);
+    const int M = d.M1 * d.M2;
+    return {N, d.R, d.E, M, d.M1, d.M2, N / d.E, d.R * M, N / d.R, plan_tw_last(d)};
+}
+
+} // namespace qt

@@ -80,10 +80,11 @@ template <> struct Prec<double> {
     static __host__ Rl make_r(double v) { return v; }
     static __device__ __forceinline__ cpx<double> mul(cpx<double> x, C w) { return x * w; }
     static __device__ __forceinline__ C conj(C w) { return {w.x, -w.y}; }
-    static __device__ __forceinline__ cpx<double> mul2(cpx<double> x, C w) { return x * w; }
+    static __device__ __forceinline__ C nconj(C w) { return {-w.x, w.y}; }
     static __device__ __forceinline__ cpx<double> mulr(cpx<double> x, Rl s) { return scale(x, s); }
     static __device__ __forceinline__ C ld(const C *p) { return ldg(p); }
-    static __device__ __forceinline__ Rl ldr(const Rl *p) { return __ldg(p); }
+    static __device__ __forceinline__ Rl re(C w) { return w.x; }
+    static __device__ __forceinline__ Rl im(C w) { return w.y; }
     static __device__ __forceinline__ C from_double(double re, double im) { return {re, im}; }
     // static potential factors (tables of exp(-i V_static dt/2), exp(-i V_static dt)): one double each
     using S = cpx<double>;
@@ -94,9 +95,6 @@ template <> struct Prec<double> {
 };
 template <> struct Prec<float> {
     struct alignas(16) C { float rh, ih, rl, il; };
-    // The sine pre-factors keep their low parts: rounded to single FP32 they passed the paired
-    // ensemble study (8.9e-6 / 6.6e-6 at N = 8192 / 4096) and ran 2.5-3.5% faster, but the same
-    // rounding every step biased the no-jump norm by +1.3e-8 per step at N = 64.
     struct alignas(8) Rl { float h, l; };
     static __host__ C make(double re, double im)
     {
@@ -113,15 +111,8 @@ template <> struct Prec<float> {
         const float lr = fmaf(x.x, w.rl, -x.y * w.il), li = fmaf(x.x, w.il, x.y * w.rl);
         return {fmaf(x.x, w.rh, fmaf(-x.y, w.ih, lr)), fmaf(x.x, w.ih, fmaf(x.y, w.rh, li))};
     }
-    // the same product as mul, in packed FP32x2 instructions (bit-identical results)
-    static __device__ __forceinline__ cpx<float> mul2(cpx<float> x, C w)
-    {
-        const float2 xx = make_float2(x.x, x.x), yy = make_float2(-x.y, x.y);
-        const float2 l = __ffma2_rn(xx, make_float2(w.rl, w.il), __fmul2_rn(yy, make_float2(w.il, w.rl)));
-        const float2 r = __ffma2_rn(xx, make_float2(w.rh, w.ih), __ffma2_rn(yy, make_float2(w.ih, w.rh), l));
-        return {r.x, r.y};
-    }
     static __device__ __forceinline__ C conj(C w) { return {w.rh, -w.ih, w.rl, -w.il}; }
+    static __device__ __forceinline__ C nconj(C w) { return {-w.rh, w.ih, -w.rl, w.il}; }
     static __device__ __forceinline__ cpx<float> mulr(cpx<float> x, Rl s)
     {
         return {fmaf(x.x, s.h, x.x * s.l), fmaf(x.y, s.h, x.y * s.l)};
@@ -136,6 +127,8 @@ template <> struct Prec<float> {
         const float2 v = __ldg(reinterpret_cast<const float2 *>(p));
         return {v.x, v.y};
     }
+    static __device__ __forceinline__ Rl re(C w) { return {w.rh, w.rl}; }
+    static __device__ __forceinline__ Rl im(C w) { return {w.ih, w.il}; }
     static __device__ __forceinline__ C from_double(double re, double im)
     {
         const float rh = (float)re, ih = (float)im;
@@ -155,13 +148,12 @@ template <> struct Prec<float> {
     static __device__ __forceinline__ S conj_s(S w) { return {w.x, -w.y}; }
 };
 
-// a * (rh + i ih) with the constant's low parts (rl, il) in FP32 (PK: the packed product); plain
-// product in FP64
-template <typename T, bool PK = false> __device__ __forceinline__ cpx<T> mulk(cpx<T> a, double re, double im)
+// a * (rh + i ih) with the constant's low parts (rl, il) in FP32; plain product in FP64
+template <typename T> __device__ __forceinline__ cpx<T> mulk(cpx<T> a, double re, double im)
 {
     if constexpr (sizeof(T) == 4) {
         const Prec<float>::C w{(float)re, (float)im, (float)(re - (double)(float)re), (float)(im - (double)(float)im)};
-        return PK ? Prec<float>::mul2(a, w) : Prec<float>::mul(a, w);
+        return Prec<float>::mul(a, w);
     } else {
         return a * mk<T>(re, im);
     }
@@ -227,26 +219,52 @@ __device__ __forceinline__ Draws draws(unsigned long long seed, uint32_t k)
 // ------------------------------------------------------------------------------------------------
 // x * exp(-2 pi i j/16) for a compile-time j (after unrolling the switch folds away); the constants
 // cos(pi/8), sin(pi/8), sqrt(1/2) enter with their FP32 low parts in the FP32 form
-template <typename T, bool PK = false> __device__ __forceinline__ cpx<T> tw16(cpx<T> a, int j)
+template <typename T> __device__ __forceinline__ cpx<T> tw16(cpx<T> a, int j)
 {
     constexpr double c1 = 0.92387953251128675613, s1 = 0.38268343236508977173, h = 0.70710678118654752440;
     switch (j & 15) {
     case 0: return a;
-    case 1: return mulk<T, PK>(a, c1, -s1);
+    case 1: return mulk<T>(a, c1, -s1);
     case 2: return mk(mulkr<T>(a.x + a.y, h), mulkr<T>(a.y - a.x, h));
-    case 3: return mulk<T, PK>(a, s1, -c1);
+    case 3: return mulk<T>(a, s1, -c1);
     case 4: return mul_mi(a);
-    case 5: return mulk<T, PK>(a, -s1, -c1);
+    case 5: return mulk<T>(a, -s1, -c1);
     case 6: return mk(mulkr<T>(a.y - a.x, h), mulkr<T>(-a.x - a.y, h));
-    case 7: return mulk<T, PK>(a, -c1, -s1);
+    case 7: return mulk<T>(a, -c1, -s1);
     case 8: return mk(-a.x, -a.y);
-    case 9: return mulk<T, PK>(a, -c1, s1);
+    case 9: return mulk<T>(a, -c1, s1);
     case 10: return mk(mulkr<T>(-a.x - a.y, h), mulkr<T>(a.x - a.y, h));
-    case 11: return mulk<T, PK>(a, -s1, c1);
+    case 11: return mulk<T>(a, -s1, c1);
     case 12: return mul_i(a);
-    case 13: return mulk<T, PK>(a, s1, c1);
+    case 13: return mulk<T>(a, s1, c1);
     case 14: return mk(mulkr<T>(a.x - a.y, h), mulkr<T>(a.x + a.y, h));
-    default: return mulk<T, PK>(a, c1, s1);
+    default: return mulk<T>(a, c1, s1);
+    }
+}
+
+// x * exp(-2 pi i j/32) for a compile-time j
+template <typename T> __device__ __forceinline__ cpx<T> tw32(cpx<T> a, int j)
+{
+    constexpr double c1 = 0.98078528040323044913, s1 = 0.19509032201612826785;   // cos, sin(pi/16)
+    constexpr double c3 = 0.83146961230254523708, s3 = 0.55557023301960222474;   // cos, sin(3 pi/16)
+    switch (j & 31) {
+    case 1: return mulk<T>(a, c1, -s1);
+    case 3: return mulk<T>(a, c3, -s3);
+    case 5: return mulk<T>(a, s3, -c3);
+    case 7: return mulk<T>(a, s1, -c1);
+    case 9: return mulk<T>(a, -s1, -c1);
+    case 11: return mulk<T>(a, -s3, -c3);
+    case 13: return mulk<T>(a, -c3, -s3);
+    case 15: return mulk<T>(a, -c1, -s1);
+    case 17: return mulk<T>(a, -c1, s1);
+    case 19: return mulk<T>(a, -c3, s3);
+    case 21: return mulk<T>(a, -s3, c3);
+    case 23: return mulk<T>(a, -s1, c1);
+    case 25: return mulk<T>(a, s1, c1);
+    case 27: return mulk<T>(a, s3, c3);
+    case 29: return mulk<T>(a, c3, s3);
+    case 31: return mulk<T>(a, c1, s1);
+    default: return tw16<T>(a, j / 2);
     }
 }
 
@@ -397,12 +415,21 @@ static_assert(sizeof(qtraj_trace_rec) == 80, "qtraj_trace_rec layout");
 // Read-only context tables (device pointers) and scalars.
 template <typename T> struct Tables {
     using C = typename Prec<T>::C;
+    // plain form and FP32 KSU kernel, natural order
     const C *W;                        // N twiddles exp(-2 pi i t / N)
     const C *WL;                       // last-pass twiddles W^(m g): sections [R][N/(2R)] for R = 16, 8, 4
     const C *KT;                       // N kinetic factors exp(-i T_kin(p_k) dt) * 2/N, k = 0..N-1
     const typename Prec<T>::Rl *sinpre; // N values sin(pi j / N)
+    const typename Prec<T>::S *statP;  // [2][LTAB][N] exp(-i (V_coul + l(l+1)/(M r^2)) dt/2)
+    // fused form, in the order of the kernel's threads (fused_plan.h)
+    const C *KF;                       // N kinetic factors exp(-i T_kin(p_k) dt) * (-1/(2N))
+    const C *TA;                       // first-pass twiddles W_2N^(b k): [R/2][N/R], k = 1 .. R/2
+    const C *TM;                       // W_S^(b1 q1): [b1][q1] applied by the last pass, else [q1][b1]
+    const C *TS;                       // [R/2] (1/(2 sin(pi k/R)), cot(pi k/R)/2): the sequences' positions 0, S/2
+    const C *TI;                       // between two middle passes: W_M^(m2 k1), [k1][m2]
     const typename Prec<T>::S *statV;  // [2][LTAB][N] exp(-i (V_coul + l(l+1)/(M r^2)) dt/2)
     const typename Prec<T>::S *statV2; // [2][LTAB][N] the same over a full step, exp(-i (...) dt)
+                                       // (both in natural order for the FP32 KSU kernel)
     const double *eig;     // [NBASIS][N] Coulomb basis, discretely normalised
     const double *ic;      // initial states, discretely normalised: [n_spec][N] real, or
                            // [n_spec][N][2] (re, im) when ic_cplx (after a vacuum evolution)
@@ -466,7 +493,7 @@ struct LaunchArgs {
 template <typename T>
 __device__ __forceinline__ typename Prec<T>::S static_factor(const Tables<T> &tb, int N, int c, int l, int j)
 {
-    if (l < LTAB) return Prec<T>::ld_s(&tb.statV[((size_t)c * LTAB + l) * N + j]);
+    if (l < LTAB) return Prec<T>::ld_s(&tb.statP[((size_t)c * LTAB + l) * N + j]);
     if (j == 0) return Prec<T>::make_s(0.0, 0.0);
     const double r = j * tb.dr;
     const double V = tb.coul[c] / r + (double)l * (l + 1) / (tb.M * r * r);
