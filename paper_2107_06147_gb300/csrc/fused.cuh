@@ -37,6 +37,8 @@
 // share the butterfly of slot 0 the same way, separated in closed form (special_in, special_mid).
 // Which points a thread holds: fused_plan.h.
 #pragma once
+#include <type_traits>
+
 #include "fused_launch.cuh"
 #include "fused_plan.h"
 #include "qtraj_device.cuh"
@@ -148,6 +150,31 @@ template <int G> __device__ __forceinline__ double slot_sum(double v, double *re
     for (int off = W / 2; off > 0; off >>= 1) v += __shfl_xor_sync(mask, v, off, W);
     if constexpr (G <= 32) v = __shfl_sync(mask, v, 0, W);
     return cross_warp<G>(v, red);
+}
+
+// the same for K values at once, with two barriers in all; red holds >= K G/32 doubles
+template <int G, int K> __device__ __forceinline__ void slot_sums(double (&v)[K], double *red)
+{
+    constexpr int W = G < 32 ? G : 32;
+    const unsigned mask = lane_mask<G>();
+#pragma unroll
+    for (int i = 0; i < K; ++i) {
+#pragma unroll
+        for (int off = W / 2; off > 0; off >>= 1) v[i] += __shfl_xor_sync(mask, v[i], off, W);
+        if constexpr (G <= 32) v[i] = __shfl_sync(mask, v[i], 0, W);
+        else if ((threadIdx.x & 31) == 0) red[i * (G / 32) + (threadIdx.x >> 5)] = v[i];
+    }
+    if constexpr (G > 32) {
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < K; ++i) {
+            double s = 0.0;
+#pragma unroll
+            for (int w = 0; w < G / 32; ++w) s += red[i * (G / 32) + w];
+            v[i] = s;
+        }
+        __syncthreads();
+    }
 }
 
 // squared norm over the G threads of a trajectory; FP32 forms reduce in double-float all the way and
@@ -1264,6 +1291,8 @@ __device__ int fetch_trajectory(const Tables<T> &tb, const LaunchArgs &a)
     }
 }
 
+constexpr int fused_red = 7;   // sums reduced at once (slot_sums)
+
 // Occupancy target of a kernel variant: variant 0 asks for 512 resident threads per SM in FP32
 // (<= 128 registers); variant 1 asks for 640 (<= 102 registers, at the price of spills), variants 2 and 3
 // (radix 8) for 768 and 1024.  FP64 holds twice the state and takes what the compiler needs.
@@ -1281,13 +1310,13 @@ __global__ void __launch_bounds__(FusedPlan<T, N, V>::G, (FusedBounds<T, N, V>::
     using K = Sine<T, N, V>;
     using PW = Pointwise<T, N, V>;
     using NS2 = typename NormSum<T>::type;
-    constexpr int G = P::G, E = P::E, NS = P::NS;
+    constexpr int G = P::G, E = P::E, NS = P::NS, RED = fused_red;
     constexpr bool KSU = V == 5;                  // the isotropic KSU potential: H_eff only, no jumps
     constexpr bool TRACED = V == 4 || V == 6;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cpx<T> *buf = reinterpret_cast<cpx<T> *>(smem_raw);
     double *red = reinterpret_cast<double *>(buf + P::BUF);         // reductions of the rare paths
-    NS2 *redh = reinterpret_cast<NS2 *>(red + (G / 32 + 1));        // the step's norm
+    NS2 *redh = reinterpret_cast<NS2 *>(red + RED * (G / 32 + 1));  // the step's norm
     __shared__ int s_traj;
 
     const int g = threadIdx.x;
@@ -1481,33 +1510,44 @@ __global__ void __launch_bounds__(FusedPlan<T, N, V>::G, (FusedBounds<T, N, V>::
             }
         }
 
-        // observables (FP64) from the shared-memory copy
-        double acc = 0.0;
-#pragma unroll 4
-        for (int e = 0; e < E; ++e) {
-            const cpx<T> v = buf[e * G + g];
-            acc += (double)v.x * v.x + (double)v.y * v.y;
-        }
-        const double n2 = slot_sum<G>(acc, red) * dr;
-        double ovr[NBASIS], ovi[NBASIS];
+        // observables (FP64) from the shared-memory copy, the norm and the overlaps of the state's l in one pass:
+        // the conversions and sums run on the narrow FP64 pipe (160 of its instructions a warp at 16 values a
+        // thread and l = 0, 256 with a pass for each sum)
+        double n2, ovr[NBASIS] = {0, 0, 0, 0, 0, 0}, ovi[NBASIS] = {0, 0, 0, 0, 0, 0};
         const int basis_l[NBASIS] = {0, 0, 1, 0, 1, 2};
+        auto observe = [&](auto nb, int s0, int s1, int s2) {
+            constexpr int NB = decltype(nb)::value;
+            const double *phi[3] = {tb.eig + (size_t)s0 * N, tb.eig + (size_t)s1 * N, tb.eig + (size_t)s2 * N};
+            double v[1 + 2 * NB];
 #pragma unroll
-        for (int s = 0; s < NBASIS; ++s) {
-            ovr[s] = 0.0;
-            ovi[s] = 0.0;
-            if (ended || c != 0 || basis_l[s] != l) continue;
-            const double *phi = tb.eig + (size_t)s * N;
-            double pr = 0.0, pi = 0.0;
+            for (int i = 0; i < 1 + 2 * NB; ++i) v[i] = 0.0;
 #pragma unroll 4
             for (int e = 0; e < E; ++e) {
-                const cpx<T> v = buf[e * G + g];
-                const double f = phi[PW::jof(g, e)], fs = PW::odd_half(e) ? -f : f;
-                pr += fs * (double)v.x;
-                pi += fs * (double)v.y;
+                const cpx<T> u = buf[e * G + g];
+                const double re = (double)u.x, im = (double)u.y;
+                v[0] = fma(re, re, fma(im, im, v[0]));
+                const int j = PW::jof(g, e);
+                const bool neg = PW::odd_half(e);
+#pragma unroll
+                for (int i = 0; i < NB; ++i) {
+                    const double f = phi[i][j], fs = neg ? -f : f;
+                    v[1 + 2 * i] = fma(fs, re, v[1 + 2 * i]);
+                    v[2 + 2 * i] = fma(fs, im, v[2 + 2 * i]);
+                }
             }
-            ovr[s] = slot_sum<G>(pr, red) * dr;
-            ovi[s] = slot_sum<G>(pi, red) * dr;
-        }
+            slot_sums<G>(v, red);
+            n2 = v[0] * dr;
+            const int sel[3] = {s0, s1, s2};
+#pragma unroll
+            for (int i = 0; i < NB; ++i) {
+                ovr[sel[i]] = v[1 + 2 * i] * dr;
+                ovi[sel[i]] = v[2 + 2 * i] * dr;
+            }
+        };
+        if (ended || c != 0 || l > 2) observe(std::integral_constant<int, 0>{}, 0, 0, 0);
+        else if (l == 0) observe(std::integral_constant<int, 3>{}, 0, 1, 3);
+        else if (l == 1) observe(std::integral_constant<int, 2>{}, 2, 4, 0);
+        else observe(std::integral_constant<int, 1>{}, 5, 0, 0);
         if (a.states && !grp) {
             double *st = a.states + (size_t)t * N * 2;
 #pragma unroll 4
@@ -1571,7 +1611,7 @@ __global__ void __launch_bounds__(FusedPlan<T, N, V>::G, (FusedBounds<T, N, V>::
 template <typename T, int N, int V> constexpr int fused_smem_bytes()
 {
     using P = FusedPlan<T, N, V>;
-    return P::BUF * (int)sizeof(cpx<T>) + (P::G / 32 + 1) * 16;
+    return P::BUF * (int)sizeof(cpx<T>) + (P::G / 32 + 1) * (fused_red + 1) * 8;
 }
 
 // Launches a trajectory kernel as one persistent wave (SMs x resident CTAs, at most max_ctas when
