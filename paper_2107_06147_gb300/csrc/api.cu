@@ -102,8 +102,8 @@ struct qtraj_ctx {
     qtraj_params p{};
     int device = 0, sm_count = 0;
     // read-only tables
-    void *W = nullptr, *WL = nullptr, *KT = nullptr, *sinpre = nullptr, *statP = nullptr;   // plain, FP32 KSU
-    void *KF = nullptr, *TA = nullptr, *TM = nullptr, *TI = nullptr, *TS = nullptr, *statV = nullptr, *statV2 = nullptr;   // fused
+    void *W = nullptr, *WL = nullptr, *KT = nullptr, *sinpre = nullptr;   // FP32 KSU
+    void *KF = nullptr, *TA = nullptr, *TM = nullptr, *TI = nullptr, *TS = nullptr, *statV = nullptr, *statV2 = nullptr;
     double *eig = nullptr;
     double *ic = nullptr, *ov0 = nullptr;
     int *ov0_zero = nullptr, *spec_l = nullptr, *spec_color = nullptr;
@@ -211,8 +211,8 @@ Layout layout(const qtraj_ctx *c, int n)
     if (c->p.save_states) o = align256(o + sizeof(double) * 2 * (size_t)c->N * n);
     L.plain = o;
     if (c->p.form == QTRAJ_PLAIN) {
-        o = align256(o + 4 * sizeof(cpx<double>) * (size_t)c->N * n);   // psi, y, z, s
-        o = align256(o + sizeof(double) * (size_t)n);                  // n2
+        o = align256(o + sizeof(cpx<double>) * ((size_t)c->N + 2 * plain_seq(c->N)) * n);   // psi, sa, sb
+        o = align256(o + sizeof(double) * (size_t)plain_parts(c->N) * n);                   // n2
         o = align256(o + sizeof(PlainState) * (size_t)n);
     }
     L.total = o;
@@ -332,15 +332,13 @@ template <typename T> qtraj_status build_tables(qtraj_ctx *c)
         CK(cudaMalloc(&c->phi_tab, sizeof(T) * tab.size()));
         CK(cudaMemcpy(c->phi_tab, tab.data(), sizeof(T) * tab.size(), cudaMemcpyHostToDevice));
     }
-    // the forms' own tables: the plain form's in natural order, the fused kernel's in its threads' order
-    // (a plain context needs the latter for the vacuum evolution of its initial states)
+    // the FP32 KSU kernel's own tables in natural order, else both forms' in their threads' order
     using PS = typename Prec<T>::S;
     const size_t nstat = (size_t)2 * LTAB * N;
-    const bool plain = c->p.form == QTRAJ_PLAIN, fused = !plain || c->p.t_vacuum > 0;
-    const bool ksu32 = c->p.potential == 1 && sizeof(T) == 4;   // its own kernel (fused_ksu32.cuh)
+    const bool ksu32 = c->p.potential == 1 && sizeof(T) == 4;   // fused_ksu32.cuh
     const Plan p = make_plan(N, sizeof(T) == 8, c->p.potential == 1 ? 0 : c->p.variant);
     qtraj_status st = QTRAJ_OK;
-    if (plain || ksu32) {
+    if (ksu32) {
         std::vector<PC> W(N), KT(N);
         std::vector<PR> sp(N);
         for (int t = 0; t < N; ++t) {
@@ -352,19 +350,16 @@ template <typename T> qtraj_status build_tables(qtraj_ctx *c)
         if ((st = upload(&c->W, W)) != QTRAJ_OK || (st = upload(&c->KT, KT)) != QTRAJ_OK ||
             (st = upload(&c->sinpre, sp)) != QTRAJ_OK)
             return st;
-        if (ksu32) {
-            // last-pass twiddles W^(m g) for m < R, g < G = N/(2R), one compact section [R][G] (N/2 entries)
-            // per radix R = 16, 8, 4: the threads of a warp read consecutive entries
-            std::vector<PC> WL((size_t)3 * (N / 2));
-            for (int sec = 0; sec < 3; ++sec) {
-                const int R = 16 >> sec, G = N / (2 * R);
-                for (int m = 0; m < R; ++m)
-                    for (int g = 0; g < G; ++g) WL[(size_t)sec * (N / 2) + (size_t)m * G + g] = W[(size_t)m * g];
-            }
-            if ((st = upload(&c->WL, WL)) != QTRAJ_OK) return st;
+        // last-pass twiddles W^(m g) for m < R, g < G = N/(2R), one compact section [R][G] (N/2 entries)
+        // per radix R = 16, 8, 4: the threads of a warp read consecutive entries
+        std::vector<PC> WL((size_t)3 * (N / 2));
+        for (int sec = 0; sec < 3; ++sec) {
+            const int R = 16 >> sec, G = N / (2 * R);
+            for (int m = 0; m < R; ++m)
+                for (int g = 0; g < G; ++g) WL[(size_t)sec * (N / 2) + (size_t)m * G + g] = W[(size_t)m * g];
         }
-    }
-    if (fused && !ksu32) {
+        if ((st = upload(&c->WL, WL)) != QTRAJ_OK) return st;
+    } else {
         auto root = [&](long k, long n) {   // exp(-2 pi i k / n)
             const double a = -2.0 * PI * (double)(k % n) / (double)n;
             return Prec<T>::make(std::cos(a), std::sin(a));
@@ -392,12 +387,12 @@ template <typename T> qtraj_status build_tables(qtraj_ctx *c)
             (st = upload(&c->TS, TS)) != QTRAJ_OK)
             return st;
     }
-    const int ntab = (plain ? 1 : 0) + (fused ? 2 : 0);
-    if ((plain && cudaMalloc(&c->statP, sizeof(PS) * nstat) != cudaSuccess) ||
-        (fused && (cudaMalloc(&c->statV, sizeof(PS) * nstat) != cudaSuccess ||
-                   cudaMalloc(&c->statV2, sizeof(PS) * nstat) != cudaSuccess))) {
+    const bool half2 = c->p.form != QTRAJ_PLAIN || c->p.t_vacuum > 0;   // the fused kernel's full-step rows
+    if (cudaMalloc(&c->statV, sizeof(PS) * nstat) != cudaSuccess ||
+        (half2 && cudaMalloc(&c->statV2, sizeof(PS) * nstat) != cudaSuccess)) {
         cudaGetLastError();
-        return fail(QTRAJ_ENOMEM, "cudaMalloc of the static space-kernel tables (%zu bytes)", ntab * sizeof(PS) * nstat);
+        return fail(QTRAJ_ENOMEM, "cudaMalloc of the static space-kernel tables (%zu bytes)",
+                    (half2 ? 2 : 1) * sizeof(PS) * nstat);
     }
     // a private non-blocking stream: building a context waits for nothing else on the device
     cudaStream_t s = nullptr;
@@ -407,7 +402,6 @@ template <typename T> qtraj_status build_tables(qtraj_ctx *c)
         if (out)
             stat_rows<T><<<blocks, 256, 0, s>>>((PS *)out, N, c->dr, c->M, c->dt, coul[0], coul[1], span, R, p.M, p.G);
     };
-    rows(c->statP, 1.0, 0);
     rows(c->statV, 1.0, ksu32 ? 0 : p.R);
     rows(c->statV2, 2.0, ksu32 ? 0 : p.R);
     cudaError_t e = cudaGetLastError();
@@ -426,7 +420,6 @@ template <typename T> Tables<T> tables(const qtraj_ctx *c)
     t.WL = (const PC *)c->WL;
     t.KT = (const PC *)c->KT;
     t.sinpre = (const typename Prec<T>::Rl *)c->sinpre;
-    t.statP = (const typename Prec<T>::S *)c->statP;
     t.KF = (const PC *)c->KF;
     t.TA = (const PC *)c->TA;
     t.TM = (const PC *)c->TM;
@@ -775,7 +768,6 @@ void qtraj_destroy(qtraj_ctx *c)
     free_ptr(c->WL);
     free_ptr(c->KT);
     free_ptr(c->sinpre);
-    free_ptr(c->statP);
     free_ptr(c->KF);
     free_ptr(c->TA);
     free_ptr(c->TM);
@@ -1068,15 +1060,13 @@ qtraj_status qtraj_evolve(qtraj_ctx *c, int batch, const qtraj_medium *media, in
     }
     CK(cudaEventRecord(c->ev0, s));
     if (c->p.form == QTRAJ_PLAIN) {
-        const size_t nN = (size_t)c->n_traj * N;
-        cpx<double> *base = (cpx<double> *)(c->ws + c->off_plain);
+        const size_t nt = (size_t)c->n_traj, seq = plain_seq(N);
         PlainBuffers pb;
-        pb.psi = base;
-        pb.y = base + nN;
-        pb.z = base + 2 * nN;
-        pb.s = base + 3 * nN;
-        pb.n2 = (double *)(c->ws + align256(c->off_plain + 4 * sizeof(cpx<double>) * nN));
-        pb.st = (PlainState *)((char *)pb.n2 + align256(sizeof(double) * c->n_traj));
+        pb.psi = (cpx<double> *)(c->ws + c->off_plain);
+        pb.sa = pb.psi + nt * N;
+        pb.sb = pb.sa + nt * seq;
+        pb.n2 = (double *)(c->ws + align256(c->off_plain + sizeof(cpx<double>) * (N + 2 * seq) * nt));
+        pb.st = (PlainState *)((char *)pb.n2 + align256(sizeof(double) * plain_parts(N) * nt));
         const Tables<double> tb = tables<double>(c);
         if (n_groups > 0) {
             int gmax = 0;

@@ -415,13 +415,12 @@ static_assert(sizeof(qtraj_trace_rec) == 80, "qtraj_trace_rec layout");
 // Read-only context tables (device pointers) and scalars.
 template <typename T> struct Tables {
     using C = typename Prec<T>::C;
-    // plain form and FP32 KSU kernel, natural order
+    // FP32 KSU kernel, natural order
     const C *W;                        // N twiddles exp(-2 pi i t / N)
     const C *WL;                       // last-pass twiddles W^(m g): sections [R][N/(2R)] for R = 16, 8, 4
     const C *KT;                       // N kinetic factors exp(-i T_kin(p_k) dt) * 2/N, k = 0..N-1
     const typename Prec<T>::Rl *sinpre; // N values sin(pi j / N)
-    const typename Prec<T>::S *statP;  // [2][LTAB][N] exp(-i (V_coul + l(l+1)/(M r^2)) dt/2)
-    // fused form, in the order of the kernel's threads (fused_plan.h)
+    // both forms, in the order of the kernels' threads (fused_plan.h)
     const C *KF;                       // N kinetic factors exp(-i T_kin(p_k) dt) * (-1/(2N))
     const C *TA;                       // first-pass twiddles W_2N^(b k): [R/2][N/R], k = 1 .. R/2
     const C *TM;                       // W_S^(b1 q1): [b1][q1] applied by the last pass, else [q1][b1]
@@ -486,36 +485,5 @@ struct LaunchArgs {
     qtraj_obs *gobs;
     int *gready;
 };
-
-// static part of the half-step space kernel for (colour, l, j); rows beyond the table are
-// evaluated in FP64 on the fly.  A jump moves l by one, and l(l+1) grows by 2 per jump on average
-// (l -> l+1 with probability (l+1)/(2l+1)), so l >= 256 takes some 33,000 jumps.
-template <typename T>
-__device__ __forceinline__ typename Prec<T>::S static_factor(const Tables<T> &tb, int N, int c, int l, int j)
-{
-    if (l < LTAB) return Prec<T>::ld_s(&tb.statP[((size_t)c * LTAB + l) * N + j]);
-    if (j == 0) return Prec<T>::make_s(0.0, 0.0);
-    const double r = j * tb.dr;
-    const double V = tb.coul[c] / r + (double)l * (l + 1) / (tb.M * r * r);
-    double s, co;
-    sincos(-V * tb.dt * 0.5, &s, &co);
-    return Prec<T>::make_s(co, s);
-}
-
-// T-dependent part exp((er + i ei) T^3 r^2) of the half-step space kernel
-__device__ __forceinline__ cpx<float> dyn_factor(float er, float ei, float r2)
-{
-    float s, c;
-    sincosf(ei * r2, &s, &c);
-    const float m = expf(er * r2);
-    return mk(m * c, m * s);
-}
-__device__ __forceinline__ cpx<double> dyn_factor(double er, double ei, double r2)
-{
-    double s, c;
-    sincos(ei * r2, &s, &c);
-    const double m = exp(er * r2);
-    return mk(m * c, m * s);
-}
 
 } // namespace qt
