@@ -296,9 +296,14 @@ template <int N> struct NftPointwise {
         return static_far<T>(tb.coul[c], tb.M, tb.dt, l, j * tb.dr, full ? 2.0 : 1.0);
     }
 
-    // The KSU counterpart of factor (same modes, same w + w f1 form): the dynamic exponent of the
-    // half-step at temperature T is (V_I - i (V_R + a/r)) dt/2 at each point, evaluated per point;
-    // ka, kb are the per-step scalars of T_n (the closing half-step) and T_{n+1} (the opening one).
+    // The potential factor and a norm sum that tells a non-finite state (there are no jumps, so nothing else is
+    // done with it and the sum leaves out the weight |K_V|^2, an expf a point):
+    // mode 0: x <- stat1 dyn_b x (the first half-step of a trajectory)
+    // mode 1: x <- stat2 dyn_a dyn_b x; returns sum |x_old|^2
+    // mode 2: x <- stat1 dyn_a x; returns sum |x_new|^2
+    // The dynamic exponent of the half-step at temperature T is (V_I - i (V_R + a/r)) dt/2 at each point, evaluated
+    // per point and applied as w + w f1 (fused.cuh); ka, kb are the per-step scalars of T_n (the closing half-step)
+    // and T_{n+1} (the opening one).
     static __device__ typename NormSum<T>::type factor_ksu(cpx<T> *buf, const Tables<T> &tb, int g, int l, int mode,
                                                            const KsuT<T> &ka, const KsuT<T> &kb, double *red)
     {
@@ -312,22 +317,19 @@ template <int N> struct NftPointwise {
                 const int j = 2 * k + par;
                 const int p = par ? K::odd_pos(k) : K::even_pos(k);
                 const T fj = (T)j;
-                T A = (T)0, t = (T)0, z = (T)0;
+                T A = (T)0, t = (T)0;
                 if (j > 0) {
                     T vda = (T)0, via = (T)0, vdb = (T)0, vib = (T)0;
                     if (mode != 0) ksu_point<T>(tb, ka, fj, vda, via);
                     if (mode != 2) ksu_point<T>(tb, kb, fj, vdb, vib);
                     A = (via + vib) * hdt;
                     t = -(vda + vdb) * hdt;
-                    z = (via - vib) * hdt;   // |K_V(n)|^2 = exp(A + z)
                 }
                 T f1r, f1i, em1;
-                if constexpr (sizeof(T) == 4) Dyn<T>::f1t(A, t, &f1r, &f1i, &em1);
-                else Dyn<T>::f1(A, t * (T)0.318309886183790671537767526745, &f1r, &f1i, &em1);
-                const T mag = (T)1 + em1;
+                Dyn<T>::f1t(A, t, &f1r, &f1i, &em1);
                 cpx<T> v = buf[p];
                 SqAcc<T> &ac = par ? acc_odd : acc;
-                if (mode == 1) ac.add_w(v, mag * exp(z));
+                if (mode == 1) ac.add_w(v, (T)1);
                 const cpx<T> w = PR::mul_s(v, stat(tb, tab, 0, l, j, mode == 1));
                 v = mk(w.x + (w.x * f1r - w.y * f1i), w.y + (w.x * f1i + w.y * f1r));
                 if (mode == 2) ac.add_w(v, (T)1);
@@ -338,7 +340,6 @@ template <int N> struct NftPointwise {
         acc.merge(acc_odd);
         return slot_norm_sum<T, G>(acc, red);
     }
-
 };
 
 template <int N> struct KsuBounds {
