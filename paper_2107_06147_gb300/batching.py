@@ -31,7 +31,7 @@ class UnevenBatch:
         Ns = np.asarray(Ns)
         self.n = len(Ns)
         self.groups = []
-        for N in sorted(set(int(x) for x in Ns)):
+        for N in sorted(set(int(x) for x in Ns), reverse=True):   # the longest launches start first
             ids = np.nonzero(Ns == N)[0]
             ids = ids[np.argsort([-_lifetime(media[t]) for t in ids], kind="stable")]
             L = float(Ls[ids[0]]) if Ls is not None else N * dr
@@ -45,15 +45,16 @@ class UnevenBatch:
                 spec_idx.append(spec_keys[key])
             eng = qtraj.Engine(qtraj.Config(N=N, L=L, dt=dt, precision=precision, use_rmin=use_rmin))
             eng.init(spec_list, len(ids), spec_idx=np.array(spec_idx, np.int32))
-            self.groups.append({"N": N, "ids": ids, "eng": eng, "media": [media[t] for t in ids],
-                                "stream": torch.cuda.Stream()})
+            # the media and their indices laid out once: a call only brings seeds
+            self.groups.append({"N": N, "ids": ids, "eng": eng,
+                                "media": (qtraj.Medium * len(ids))(*[media[t] for t in ids]),
+                                "idx": np.arange(len(ids), dtype=np.int32), "stream": torch.cuda.Stream()})
 
     def evolve(self, seeds):
         """Launches every group on its own stream; returns immediately."""
         seeds = np.asarray(seeds, dtype=np.uint64)
         for g in self.groups:
-            g["eng"].evolve(g["media"], seeds[g["ids"]], np.arange(len(g["ids"]), dtype=np.int32),
-                            stream=g["stream"])
+            g["eng"].evolve(g["media"], seeds[g["ids"]], g["idx"], stream=g["stream"])
 
     def observables(self):
         out = np.zeros(self.n, dtype=qtraj.OBS_DTYPE)

@@ -134,7 +134,6 @@ struct qtraj_ctx {
     bool evolved = false;
     int last_batch = 0, last_groups = 0, last_n_media = 0, launches = 0;
     std::vector<int> group_pair;
-    std::vector<int> host_steps;
 };
 
 namespace {
@@ -969,47 +968,12 @@ qtraj_status qtraj_evolve(qtraj_ctx *c, int batch, const qtraj_medium *media, in
     cudaStream_t s = (cudaStream_t)stream;
     const int N = c->N;
 
-    std::vector<MediumDev> md(n_media);
-    std::vector<int> steps(n_media);
-    for (int m = 0; m < n_media; ++m) {
-        const qtraj_medium &q = media[m];
-        if (const char *why = medium_check(q, c->prof_host.empty() ? nullptr : c->prof_host.data(),
-                                           (int)(c->prof_host.size() / 2)))
-            return fail(QTRAJ_EINVAL, "medium %d: %s", m, why);
-        if (c->p.potential == 1 && !(q.Tf >= KSU_TF_MIN))
-            return fail(QTRAJ_EINVAL, "medium %d: the KSU potential needs Tf >= %g GeV", m, KSU_TF_MIN);
-        steps[m] = medium_steps(c->dt, q, c->prof_host.data());
-        md[m] = encode_medium(c, q);
-    }
-    std::vector<TrajDev> tr(batch);
-    std::map<std::pair<int, int>, int> gmap;
-    std::vector<TrajDev> gt;
-    std::vector<int> gpair;
-    int max_steps = 0;
-    for (int t = 0; t < batch; ++t) {
-        const int mi = medium_idx ? medium_idx[t] : (n_media == 1 ? 0 : t);
-        if (mi < 0 || mi >= n_media) return fail(QTRAJ_EINVAL, "medium_idx[%d] out of range", t);
-        const int sp = c->spec_idx[t];
-        auto key = std::make_pair(sp, mi);
-        auto it = gmap.find(key);
-        int g;
-        if (it == gmap.end()) {
-            g = (int)gt.size();
-            gmap[key] = g;
-            gt.push_back(TrajDev{0ull, sp, mi, steps[mi], g});
-            gpair.push_back(sp * n_media + mi);
-        } else {
-            g = it->second;
-        }
-        tr[t] = TrajDev{(unsigned long long)seeds[t], sp, mi, steps[mi], g};
-        if (steps[mi] > max_steps) max_steps = steps[mi];
-    }
-    // the rMin shortcut belongs to the jump algorithm; the KSU evolution has no jumps
-    const int n_groups = c->p.use_rmin && c->p.potential == 0 ? (int)gt.size() : 0;
-
-    // staging: media | trajs | group trajs
-    const size_t b_md = sizeof(MediumDev) * n_media, b_tr = sizeof(TrajDev) * batch, b_gt = sizeof(TrajDev) * gt.size();
-    const size_t need = align256(b_md) + align256(b_tr) + align256(b_gt) + 256;
+    // The descriptors are written straight into the pinned staging buffer (media | trajs | group trajs).  A batch
+    // with a medium per trajectory spent most of the call in a std::map of the (state, medium) groups, which only
+    // the rMin shortcut uses (the KSU evolution has no jumps and no shortcut).
+    const bool grouped = c->p.use_rmin && c->p.potential == 0;
+    const size_t b_md = sizeof(MediumDev) * n_media, b_tr = sizeof(TrajDev) * batch;
+    const size_t need = align256(b_md) + align256(b_tr) + (grouped ? align256(b_tr) : 0) + 256;
     CK(cudaEventSynchronize(c->ev_stage));   // the previous upload has left the staging buffer
     if (need > c->h_stage_bytes) {
         if (c->h_stage) cudaFreeHost(c->h_stage);
@@ -1018,16 +982,52 @@ qtraj_status qtraj_evolve(qtraj_ctx *c, int batch, const qtraj_medium *media, in
         CK(cudaMallocHost(&c->h_stage, need));
         c->h_stage_bytes = need;
     }
+    char *h = (char *)c->h_stage;
+    MediumDev *md = (MediumDev *)h;
+    TrajDev *tr = (TrajDev *)(h + align256(b_md)), *gt = (TrajDev *)(h + align256(b_md) + align256(b_tr));
+    std::vector<int> steps(n_media);
+    const double *prof = c->prof_host.empty() ? nullptr : c->prof_host.data();
+    for (int m = 0; m < n_media; ++m) {
+        const qtraj_medium &q = media[m];
+        if (const char *why = medium_check(q, prof, (int)(c->prof_host.size() / 2)))
+            return fail(QTRAJ_EINVAL, "medium %d: %s", m, why);
+        if (c->p.potential == 1 && !(q.Tf >= KSU_TF_MIN))
+            return fail(QTRAJ_EINVAL, "medium %d: the KSU potential needs Tf >= %g GeV", m, KSU_TF_MIN);
+        steps[m] = medium_steps(c->dt, q, c->prof_host.data());
+        md[m] = encode_medium(c, q);
+    }
+    // the group of a (state, medium) pair: a flat table, or a map where the pairs outnumber the trajectories by far
+    const size_t pairs = (size_t)c->n_spec * n_media;
+    const bool flat = pairs <= 64 * (size_t)batch + 65536;
+    std::vector<int> gtab(grouped && flat ? pairs : 0, -1);
+    std::map<size_t, int> gmap;
+    std::vector<int> gpair;
+    int max_steps = 0, n_groups = 0;
+    for (int t = 0; t < batch; ++t) {
+        const int mi = medium_idx ? medium_idx[t] : (n_media == 1 ? 0 : t);
+        if (mi < 0 || mi >= n_media) return fail(QTRAJ_EINVAL, "medium_idx[%d] out of range", t);
+        const int sp = c->spec_idx[t];
+        int g = 0;
+        if (grouped) {
+            const size_t key = (size_t)sp * n_media + mi;
+            int &slot = flat ? gtab[key] : gmap.emplace(key, -1).first->second;
+            if (slot < 0) {
+                slot = n_groups++;
+                gt[slot] = TrajDev{0ull, sp, mi, steps[mi], slot};
+                gpair.push_back((int)key);
+            }
+            g = slot;
+        }
+        tr[t] = TrajDev{(unsigned long long)seeds[t], sp, mi, steps[mi], g};
+        if (steps[mi] > max_steps) max_steps = steps[mi];
+    }
+    const size_t b_gt = sizeof(TrajDev) * n_groups;
     if (n_media > c->media_cap) {
         CK(cudaStreamSynchronize(s));
         free_typed(c->media);
         CK(cudaMalloc(&c->media, sizeof(MediumDev) * n_media));
         c->media_cap = n_media;
     }
-    char *h = (char *)c->h_stage;
-    std::memcpy(h, md.data(), b_md);
-    std::memcpy(h + align256(b_md), tr.data(), b_tr);
-    std::memcpy(h + align256(b_md) + align256(b_tr), gt.data(), b_gt);
     TrajDev *d_tr = (TrajDev *)(c->ws + c->off_trajs);
     TrajDev *d_gt = (TrajDev *)(c->ws + c->off_gtrajs);
     qtraj_obs *d_obs = (qtraj_obs *)(c->ws + c->off_obs);
@@ -1035,9 +1035,9 @@ qtraj_status qtraj_evolve(qtraj_ctx *c, int batch, const qtraj_medium *media, in
     int *d_ctr = (int *)(c->ws + c->off_ctr);
     int *d_status = d_ctr + 1;
     double *d_states = c->p.save_states ? (double *)(c->ws + c->off_states) : nullptr;
-    CK(cudaMemcpyAsync(c->media, h, b_md, cudaMemcpyHostToDevice, s));
-    if (b_tr) CK(cudaMemcpyAsync(d_tr, h + align256(b_md), b_tr, cudaMemcpyHostToDevice, s));
-    if (b_gt) CK(cudaMemcpyAsync(d_gt, h + align256(b_md) + align256(b_tr), b_gt, cudaMemcpyHostToDevice, s));
+    CK(cudaMemcpyAsync(c->media, md, b_md, cudaMemcpyHostToDevice, s));
+    if (b_tr) CK(cudaMemcpyAsync(d_tr, tr, b_tr, cudaMemcpyHostToDevice, s));
+    if (b_gt) CK(cudaMemcpyAsync(d_gt, gt, b_gt, cudaMemcpyHostToDevice, s));
     CK(cudaEventRecord(c->ev_stage, s));
     CK(cudaMemsetAsync(d_ctr, 0, 256, s));
 
@@ -1045,8 +1045,7 @@ qtraj_status qtraj_evolve(qtraj_ctx *c, int batch, const qtraj_medium *media, in
     c->last_batch = batch;
     c->last_groups = n_groups;
     c->last_n_media = n_media;
-    c->group_pair = gpair;
-    c->host_steps = steps;
+    c->group_pair = std::move(gpair);
 
     LaunchArgs ga{d_gt, n_groups, d_gobs, nullptr, d_ctr, d_status, nullptr, 1};
     LaunchArgs ma{d_tr, batch, d_obs, d_gobs, d_ctr, d_status, d_states, 0};
@@ -1070,7 +1069,7 @@ qtraj_status qtraj_evolve(qtraj_ctx *c, int batch, const qtraj_medium *media, in
         const Tables<double> tb = tables<double>(c);
         if (n_groups > 0) {
             int gmax = 0;
-            for (auto &g : gt) gmax = g.n_steps > gmax ? g.n_steps : gmax;
+            for (int g = 0; g < n_groups; ++g) gmax = std::max(gmax, gt[g].n_steps);
             CK(plain_run(tb, ga, N, gmax, pb, s, &c->launches));
         }
         CK(cudaEventRecord(c->ev1, s));
@@ -1078,7 +1077,6 @@ qtraj_status qtraj_evolve(qtraj_ctx *c, int batch, const qtraj_medium *media, in
     } else {
         // one launch: the groups' no-jump runs are its first work items, and a trajectory takes the
         // shortcut once its group's record is published (ms_nojump is then 0)
-        FusedInfo fi;
         LaunchArgs fa = ma;
         fa.group = nullptr;
         fa.gtrajs = d_gt;
@@ -1087,8 +1085,8 @@ qtraj_status qtraj_evolve(qtraj_ctx *c, int batch, const qtraj_medium *media, in
         fa.gready = n_groups > 0 ? (int *)(c->ws + c->off_gready) : nullptr;
         if (n_groups > 0) CK(cudaMemsetAsync(fa.gready, 0, sizeof(int) * (size_t)n_groups, s));
         CK(cudaEventRecord(c->ev1, s));
-        if (c->p.precision == QTRAJ_FP32) CK(fused_launch_f32(N, tables<float>(c), fa, c->sm_count, 0, s, &fi, false, c->p.variant));
-        else CK(fused_launch_f64(N, tables<double>(c), fa, c->sm_count, 0, s, &fi, false, c->p.variant));
+        if (c->p.precision == QTRAJ_FP32) CK(fused_launch_f32(N, tables<float>(c), fa, c->sm_count, 0, s, nullptr, false, c->p.variant));
+        else CK(fused_launch_f64(N, tables<double>(c), fa, c->sm_count, 0, s, nullptr, false, c->p.variant));
         ++c->launches;
     }
     CK(cudaEventRecord(c->ev2, s));

@@ -244,7 +244,13 @@ qtraj_status qtraj_submit(qtraj_server *s, const qtraj_traj_desc *traj, int n, u
     if (n <= 0) return failf(QTRAJ_EINVAL, "n must be positive");
     if (s->reqs.count(request_id)) return failf(QTRAJ_EINVAL, "request id %llu is queued or not yet returned",
                                                 (unsigned long long)request_id);
+    // a request's trajectories mostly repeat one grid size, state and medium: checked and costed once per run
+    auto same = [&](int t) {
+        return t > 0 && traj[t].N == traj[t - 1].N && traj[t].spec == traj[t - 1].spec &&
+               std::memcmp(&traj[t].medium, &traj[t - 1].medium, sizeof(qtraj_medium)) == 0;
+    };
     for (int t = 0; t < n; ++t) {
+        if (same(t)) continue;
         if (!s->n_index.count(traj[t].N)) return failf(QTRAJ_EINVAL, "trajectory %d: grid size %d not served", t, traj[t].N);
         if (traj[t].spec < 0 || traj[t].spec >= (int)s->specs.size())
             return failf(QTRAJ_EINVAL, "trajectory %d: spec %d outside the catalogue", t, traj[t].spec);
@@ -256,12 +262,16 @@ qtraj_status qtraj_submit(qtraj_server *s, const qtraj_traj_desc *traj, int n, u
     r->out.assign(n, qtraj_obs{});
     r->remaining = n;
     r->seq = s->seq++;
+    double w = 0.0;
     for (int t = 0; t < n; ++t) {
-        const qtraj_medium &m = traj[t].medium;
-        // the Bjorken medium's steps, as the engine counts them (work estimate only)
-        const double tau_f = m.tau0 * std::pow(m.T0 / m.Tf, 3.0);
-        const double steps = m.T0 > m.Tf ? std::ceil((tau_f - m.tau0) / (0.1973269804 * s->cfg.dt)) : 0.0;
-        r->work += (double)traj[t].N * std::log2((double)traj[t].N) * steps;
+        if (!same(t)) {
+            const qtraj_medium &m = traj[t].medium;
+            // the Bjorken medium's steps, as the engine counts them (work estimate only)
+            const double tau_f = m.tau0 * std::pow(m.T0 / m.Tf, 3.0);
+            const double steps = m.T0 > m.Tf ? std::ceil((tau_f - m.tau0) / (0.1973269804 * s->cfg.dt)) : 0.0;
+            w = (double)traj[t].N * std::log2((double)traj[t].N) * steps;
+        }
+        r->work += w;
     }
     s->reqs[request_id] = std::move(r);
     s->waiting.push_back(request_id);
@@ -333,15 +343,12 @@ qtraj_status launch(qtraj_server *s, PerN &pn, Slot &sl)
         while (pp.next < pp.idx.size() && n < sl.cap) {
             const int k = pp.idx[pp.next++];
             const qtraj_traj_desc &d = r.desc[k];
-            const auto key = std::make_tuple(d.medium.T0, d.medium.tau0, d.medium.Tf, d.medium.kappa_hat, d.medium.gamma_hat);
-            auto it = mkey.find(key);
-            int mi;
-            if (it == mkey.end()) {
-                mi = (int)sl.media.size();
-                mkey.emplace(key, mi);
-                sl.media.push_back(d.medium);
-            } else {
-                mi = it->second;
+            int mi = sl.medium_idx.empty() ? -1 : sl.medium_idx.back();
+            if (mi < 0 || std::memcmp(&d.medium, &sl.media[mi], sizeof(qtraj_medium)) != 0) {
+                const auto key = std::make_tuple(d.medium.T0, d.medium.tau0, d.medium.Tf, d.medium.kappa_hat, d.medium.gamma_hat);
+                const auto ins = mkey.emplace(key, (int)sl.media.size());
+                mi = ins.first->second;
+                if (ins.second) sl.media.push_back(d.medium);
             }
             sl.spec_idx.push_back(d.spec);
             sl.medium_idx.push_back(mi);
@@ -381,9 +388,12 @@ qtraj_status qtraj_poll(qtraj_server *s, uint64_t *done_ids, int capacity, int *
             collect(s, sl);
         }
     admit(s);
-    for (PerN &pn : s->perN)
+    // the largest grids first: their launches are the longest and the others fill in beside them
+    for (auto it = s->n_index.rbegin(); it != s->n_index.rend(); ++it) {
+        PerN &pn = s->perN[it->second];
         for (Slot &sl : pn.slots)
             if (!sl.busy && !pn.pending.empty()) SOK(launch(s, pn, sl));
+    }
     while (*n_done < capacity && !s->done.empty()) {
         done_ids[(*n_done)++] = s->done.front();
         s->done.pop_front();

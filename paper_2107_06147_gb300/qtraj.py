@@ -298,7 +298,7 @@ class Engine:
 
     def evolve(self, media, seeds, medium_idx=None, batch: int | None = None, stream=None):
         batch = len(seeds) if batch is None else batch
-        arr = (Medium * len(media))(*media)
+        arr = media if isinstance(media, C.Array) else (Medium * len(media))(*media)   # a list, or laid out once
         self._seeds = np.ascontiguousarray(seeds, dtype=np.uint64)
         idx = None
         if medium_idx is not None:
@@ -310,7 +310,7 @@ class Engine:
         self.batch = batch
 
     def observables(self, stream=None, check_finite: bool = True) -> np.ndarray:
-        out = np.zeros(self.batch, dtype=OBS_DTYPE)
+        out = np.empty(self.batch, dtype=OBS_DTYPE)
         st = self.lib.qtraj_observables(self.ctx, C.c_void_p(out.ctypes.data), 0, C.c_void_p(_stream_ptr(stream)))
         if st != 5 or check_finite:
             _check(st, self.ctx)
