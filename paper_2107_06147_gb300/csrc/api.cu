@@ -103,7 +103,10 @@ struct qtraj_ctx {
     int device = 0, sm_count = 0;
     // read-only tables
     void *W = nullptr, *WL = nullptr, *KT = nullptr, *sinpre = nullptr;   // FP32 KSU
-    void *KF = nullptr, *TA = nullptr, *TM = nullptr, *TI = nullptr, *TS = nullptr, *statV = nullptr, *statV2 = nullptr;
+    struct TabSet {   // the tables in the order of one plan (fused_plan.h)
+        void *KF = nullptr, *TA = nullptr, *TM = nullptr, *TI = nullptr, *TS = nullptr, *statV = nullptr, *statV2 = nullptr;
+        void **all[7] = {&KF, &TA, &TM, &TI, &TS, &statV, &statV2};
+    } fused, plain;
     double *eig = nullptr;
     double *ic = nullptr, *ov0 = nullptr;
     int *ov0_zero = nullptr, *spec_l = nullptr, *spec_color = nullptr;
@@ -253,6 +256,66 @@ template <typename V> qtraj_status upload(void **out, const std::vector<V> &v)
     return QTRAJ_OK;
 }
 
+// the transform's tables and the kinetic factors in the order of plan p
+template <typename T>
+qtraj_status build_set(const qtraj_ctx *c, qtraj_ctx::TabSet &t, const Plan &p, const std::vector<std::pair<double, double>> &kt)
+{
+    using PC = typename Prec<T>::C;
+    const int N = c->N;
+    auto root = [&](long k, long n) {   // exp(-2 pi i k / n)
+        const double a = -2.0 * PI * (double)(k % n) / (double)n;
+        return Prec<T>::make(std::cos(a), std::sin(a));
+    };
+    std::vector<PC> KF(N), TA((size_t)p.R / 2 * p.NS), TM(p.S), TI((size_t)p.M1 * p.M2), TS(p.R / 2);
+    for (int i = 0; i < N; ++i) {
+        int g, e;
+        plan_entry(i, false, p.R, p.G, g, e);
+        const int j = plan_j(g, e, p.R, p.M, p.G);
+        const double f = j == 0 ? 0.0 : -0.5 / N;   // two transforms X = -2i S, and the inverse's 2/N
+        KF[i] = Prec<T>::make(kt[j].first * f, kt[j].second * f);
+    }
+    for (int s = 0; s < p.NS; ++s) {
+        int lo, hi;
+        slot_points(s, p.R, p.M, lo, hi);
+        for (int k = 1; k <= p.R / 2; ++k) TA[(size_t)(k - 1) * p.NS + s] = root((long)lo * k, 2L * N);
+    }
+    for (int b1 = 0; b1 < p.R; ++b1)
+        for (int q1 = 0; q1 < p.M; ++q1) TM[p.tw_last ? b1 * p.M + q1 : q1 * p.R + b1] = root((long)b1 * q1, p.S);
+    for (int k1 = 0; k1 < p.M1; ++k1)
+        for (int m2 = 0; m2 < p.M2; ++m2) TI[(size_t)k1 * p.M2 + m2] = root((long)m2 * k1, p.M);
+    for (int k = 1; k < p.R / 2; ++k) TS[k] = Prec<T>::make(0.5 / std::sin(PI * k / p.R), 0.5 / std::tan(PI * k / p.R));
+    qtraj_status st = QTRAJ_OK;
+    if ((st = upload(&t.KF, KF)) != QTRAJ_OK || (st = upload(&t.TA, TA)) != QTRAJ_OK || (st = upload(&t.TM, TM)) != QTRAJ_OK ||
+        (st = upload(&t.TI, TI)) != QTRAJ_OK)
+        return st;
+    return upload(&t.TS, TS);
+}
+
+// the static potential rows in the order of plan p (nullptr: natural), of a half and (full) a whole step
+template <typename T>
+qtraj_status build_static(const qtraj_ctx *c, qtraj_ctx::TabSet &t, const Plan *p, const double *coul, bool full)
+{
+    using PS = typename Prec<T>::S;
+    const size_t n = (size_t)2 * LTAB * c->N;
+    if (cudaMalloc(&t.statV, sizeof(PS) * n) != cudaSuccess || (full && cudaMalloc(&t.statV2, sizeof(PS) * n) != cudaSuccess)) {
+        cudaGetLastError();
+        return fail(QTRAJ_ENOMEM, "cudaMalloc of the static space-kernel tables (%zu bytes)", (full ? 2 : 1) * sizeof(PS) * n);
+    }
+    // a private non-blocking stream: building a context waits for nothing else on the device
+    cudaStream_t s = nullptr;
+    CK(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
+    const int blocks = (int)std::min<size_t>((n + 255) / 256, 4096);
+    for (int h = 0; h < (full ? 2 : 1); ++h)
+        stat_rows<T><<<blocks, 256, 0, s>>>((PS *)(h ? t.statV2 : t.statV), c->N, c->dr, c->M, c->dt, coul[0], coul[1],
+                                            h ? 2.0 : 1.0, p ? p->R : 0, p ? p->M : 0, p ? p->G : 1);
+    cudaError_t e = cudaGetLastError();
+    const cudaError_t e2 = cudaStreamSynchronize(s);
+    if (e == cudaSuccess) e = e2;
+    cudaStreamDestroy(s);
+    CK(e);
+    return QTRAJ_OK;
+}
+
 template <typename T> qtraj_status build_tables(qtraj_ctx *c)
 {
     using PC = typename Prec<T>::C;
@@ -331,13 +394,8 @@ template <typename T> qtraj_status build_tables(qtraj_ctx *c)
         CK(cudaMalloc(&c->phi_tab, sizeof(T) * tab.size()));
         CK(cudaMemcpy(c->phi_tab, tab.data(), sizeof(T) * tab.size(), cudaMemcpyHostToDevice));
     }
-    // the FP32 KSU kernel's own tables in natural order, else both forms' in their threads' order
-    using PS = typename Prec<T>::S;
-    const size_t nstat = (size_t)2 * LTAB * N;
-    const bool ksu32 = c->p.potential == 1 && sizeof(T) == 4;   // fused_ksu32.cuh
-    const Plan p = make_plan(N, sizeof(T) == 8, c->p.potential == 1 ? 0 : c->p.variant);
-    qtraj_status st = QTRAJ_OK;
-    if (ksu32) {
+    if (c->p.potential == 1 && sizeof(T) == 4) {
+        // the FP32 KSU kernel's tables in natural order (fused_ksu32.cuh)
         std::vector<PC> W(N), KT(N);
         std::vector<PR> sp(N);
         for (int t = 0; t < N; ++t) {
@@ -346,9 +404,6 @@ template <typename T> qtraj_status build_tables(qtraj_ctx *c)
             sp[t] = Prec<T>::make_r(std::sin(PI * (double)t / N));
             KT[t] = Prec<T>::make(kt[t].first * 2.0 / N, kt[t].second * 2.0 / N);
         }
-        if ((st = upload(&c->W, W)) != QTRAJ_OK || (st = upload(&c->KT, KT)) != QTRAJ_OK ||
-            (st = upload(&c->sinpre, sp)) != QTRAJ_OK)
-            return st;
         // last-pass twiddles W^(m g) for m < R, g < G = N/(2R), one compact section [R][G] (N/2 entries)
         // per radix R = 16, 8, 4: the threads of a warp read consecutive entries
         std::vector<PC> WL((size_t)3 * (N / 2));
@@ -357,75 +412,42 @@ template <typename T> qtraj_status build_tables(qtraj_ctx *c)
             for (int m = 0; m < R; ++m)
                 for (int g = 0; g < G; ++g) WL[(size_t)sec * (N / 2) + (size_t)m * G + g] = W[(size_t)m * g];
         }
-        if ((st = upload(&c->WL, WL)) != QTRAJ_OK) return st;
-    } else {
-        auto root = [&](long k, long n) {   // exp(-2 pi i k / n)
-            const double a = -2.0 * PI * (double)(k % n) / (double)n;
-            return Prec<T>::make(std::cos(a), std::sin(a));
-        };
-        std::vector<PC> KF(N), TA((size_t)p.R / 2 * p.NS), TM(p.S), TI((size_t)p.M1 * p.M2), TS(p.R / 2);
-        for (int i = 0; i < N; ++i) {
-            int g, e;
-            plan_entry(i, false, p.R, p.G, g, e);
-            const int j = plan_j(g, e, p.R, p.M, p.G);
-            const double f = j == 0 ? 0.0 : -0.5 / N;   // two transforms X = -2i S, and the inverse's 2/N
-            KF[i] = Prec<T>::make(kt[j].first * f, kt[j].second * f);
-        }
-        for (int s = 0; s < p.NS; ++s) {
-            int lo, hi;
-            slot_points(s, p.R, p.M, lo, hi);
-            for (int k = 1; k <= p.R / 2; ++k) TA[(size_t)(k - 1) * p.NS + s] = root((long)lo * k, 2L * N);
-        }
-        for (int b1 = 0; b1 < p.R; ++b1)
-            for (int q1 = 0; q1 < p.M; ++q1) TM[p.tw_last ? b1 * p.M + q1 : q1 * p.R + b1] = root((long)b1 * q1, p.S);
-        for (int k1 = 0; k1 < p.M1; ++k1)
-            for (int m2 = 0; m2 < p.M2; ++m2) TI[(size_t)k1 * p.M2 + m2] = root((long)m2 * k1, p.M);
-        for (int k = 1; k < p.R / 2; ++k) TS[k] = Prec<T>::make(0.5 / std::sin(PI * k / p.R), 0.5 / std::tan(PI * k / p.R));
-        if ((st = upload(&c->KF, KF)) != QTRAJ_OK || (st = upload(&c->TA, TA)) != QTRAJ_OK ||
-            (st = upload(&c->TM, TM)) != QTRAJ_OK || (st = upload(&c->TI, TI)) != QTRAJ_OK ||
-            (st = upload(&c->TS, TS)) != QTRAJ_OK)
+        qtraj_status st = QTRAJ_OK;
+        if ((st = upload(&c->W, W)) != QTRAJ_OK || (st = upload(&c->KT, KT)) != QTRAJ_OK ||
+            (st = upload(&c->sinpre, sp)) != QTRAJ_OK || (st = upload(&c->WL, WL)) != QTRAJ_OK)
             return st;
+        return build_static<T>(c, c->fused, nullptr, coul, true);
     }
-    const bool half2 = c->p.form != QTRAJ_PLAIN || c->p.t_vacuum > 0;   // the fused kernel's full-step rows
-    if (cudaMalloc(&c->statV, sizeof(PS) * nstat) != cudaSuccess ||
-        (half2 && cudaMalloc(&c->statV2, sizeof(PS) * nstat) != cudaSuccess)) {
-        cudaGetLastError();
-        return fail(QTRAJ_ENOMEM, "cudaMalloc of the static space-kernel tables (%zu bytes)",
-                    (half2 ? 2 : 1) * sizeof(PS) * nstat);
-    }
-    // a private non-blocking stream: building a context waits for nothing else on the device
-    cudaStream_t s = nullptr;
-    CK(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
-    const int blocks = (int)std::min<size_t>((nstat + 255) / 256, 4096);
-    auto rows = [&](void *out, double span, int R) {
-        if (out)
-            stat_rows<T><<<blocks, 256, 0, s>>>((PS *)out, N, c->dr, c->M, c->dt, coul[0], coul[1], span, R, p.M, p.G);
-    };
-    rows(c->statV, 1.0, ksu32 ? 0 : p.R);
-    rows(c->statV2, 2.0, ksu32 ? 0 : p.R);
-    cudaError_t e = cudaGetLastError();
-    const cudaError_t e2 = cudaStreamSynchronize(s);
-    if (e == cudaSuccess) e = e2;
-    cudaStreamDestroy(s);
-    CK(e);
+    // a plain context runs the fused kernel only for the vacuum evolution of its initial states
+    const int variant = c->p.potential == 1 ? 0 : c->p.variant;
+    const Plan pf = make_plan(N, sizeof(T) == 8, variant >= 2 ? PLAN_RAD8 : PLAN_FUSED), pp = make_plan(N, true, PLAN_PLAIN);
+    qtraj_status st = QTRAJ_OK;
+    if (c->p.form != QTRAJ_PLAIN || c->p.t_vacuum > 0)
+        if ((st = build_set<T>(c, c->fused, pf, kt)) != QTRAJ_OK || (st = build_static<T>(c, c->fused, &pf, coul, true)) != QTRAJ_OK)
+            return st;
+    if (c->p.form == QTRAJ_PLAIN)
+        if ((st = build_set<T>(c, c->plain, pp, kt)) != QTRAJ_OK || (st = build_static<T>(c, c->plain, &pp, coul, false)) != QTRAJ_OK)
+            return st;
     return QTRAJ_OK;
 }
 
-template <typename T> Tables<T> tables(const qtraj_ctx *c)
+// the kernels' view of the context; plain: with the plain form's tables
+template <typename T> Tables<T> tables(const qtraj_ctx *c, bool plain = false)
 {
+    const qtraj_ctx::TabSet &ts = plain ? c->plain : c->fused;
     Tables<T> t;
     using PC = typename Prec<T>::C;
     t.W = (const PC *)c->W;
     t.WL = (const PC *)c->WL;
     t.KT = (const PC *)c->KT;
     t.sinpre = (const typename Prec<T>::Rl *)c->sinpre;
-    t.KF = (const PC *)c->KF;
-    t.TA = (const PC *)c->TA;
-    t.TM = (const PC *)c->TM;
-    t.TI = (const PC *)c->TI;
-    t.TS = (const PC *)c->TS;
-    t.statV = (const typename Prec<T>::S *)c->statV;
-    t.statV2 = (const typename Prec<T>::S *)c->statV2;
+    t.KF = (const PC *)ts.KF;
+    t.TA = (const PC *)ts.TA;
+    t.TM = (const PC *)ts.TM;
+    t.TI = (const PC *)ts.TI;
+    t.TS = (const PC *)ts.TS;
+    t.statV = (const typename Prec<T>::S *)ts.statV;
+    t.statV2 = (const typename Prec<T>::S *)ts.statV2;
     t.eig = c->eig;
     t.ic = c->ic;
     t.ov0 = c->ov0;
@@ -767,13 +789,8 @@ void qtraj_destroy(qtraj_ctx *c)
     free_ptr(c->WL);
     free_ptr(c->KT);
     free_ptr(c->sinpre);
-    free_ptr(c->KF);
-    free_ptr(c->TA);
-    free_ptr(c->TM);
-    free_ptr(c->TI);
-    free_ptr(c->TS);
-    free_ptr(c->statV);
-    free_ptr(c->statV2);
+    for (qtraj_ctx::TabSet *t : {&c->fused, &c->plain})
+        for (void **p : t->all) free_ptr(*p);
     free_ptr(c->phi_tab);
     free_typed(c->eig);
     free_typed(c->ic);
@@ -1066,7 +1083,7 @@ qtraj_status qtraj_evolve(qtraj_ctx *c, int batch, const qtraj_medium *media, in
         pb.sb = pb.sa + nt * seq;
         pb.n2 = (double *)(c->ws + align256(c->off_plain + sizeof(cpx<double>) * (N + 2 * seq) * nt));
         pb.st = (PlainState *)((char *)pb.n2 + align256(sizeof(double) * plain_parts(N) * nt));
-        const Tables<double> tb = tables<double>(c);
+        const Tables<double> tb = tables<double>(c, true);
         if (n_groups > 0) {
             int gmax = 0;
             for (int g = 0; g < n_groups; ++g) gmax = std::max(gmax, gt[g].n_steps);

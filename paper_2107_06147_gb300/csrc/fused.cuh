@@ -47,9 +47,9 @@ namespace qt {
 
 // V selects the launch variant (fused_launch.cuh): 0, 1 the plan of the grid size with 512 or 640 resident
 // threads per SM, 2 and 3 the radix-8 plans with 768 and 1024; 4 and 6 the traced twins of 0 and 2, 5 the
-// KSU twin of 0.
+// KSU twin of 0, 7 the plain form's kernels (plain_step.cuh).
 template <typename T, int N, int V = 0> struct FusedPlan {
-    static constexpr PlanDims D = plan_dims(N, sizeof(T) == 8, V == 2 || V == 3 || V == 6);
+    static constexpr PlanDims D = plan_dims(N, sizeof(T) == 8, V == 2 || V == 3 || V == 6 ? PLAN_RAD8 : V == 7 ? PLAN_PLAIN : PLAN_FUSED);
     static constexpr int R = D.R, E = D.E, M1 = D.M1, M2 = D.M2;
     static constexpr int H = R / 2;              // sequences
     static constexpr int M = M1 * M2;            // length of the middle transform
@@ -450,8 +450,11 @@ template <> struct Dyn<double> {
     template <bool PHASE> static __device__ __forceinline__ cpx<double> cexp(double a, double t, double *m)
     {
         double s = 0.0, c = 1.0, e;
-        if (fabs(a) <= 0.03125 && (!PHASE || fabs(t) <= 0.03125)) {
-            e = 1.0 / 40320.0;
+        if (fabs(a) <= 0.125 && (!PHASE || fabs(t) <= 0.125)) {
+            e = 1.0 / 39916800.0;
+            e = fma(e, a, 1.0 / 3628800.0);
+            e = fma(e, a, 1.0 / 362880.0);
+            e = fma(e, a, 1.0 / 40320.0);
             e = fma(e, a, 1.0 / 5040.0);
             e = fma(e, a, 1.0 / 720.0);
             e = fma(e, a, 1.0 / 120.0);
@@ -462,8 +465,8 @@ template <> struct Dyn<double> {
             e = fma(e, a, 1.0);
             if (PHASE) {
                 const double u = t * t;
-                s = fma(fma(fma(-1.0 / 5040.0, u, 1.0 / 120.0), u, -1.0 / 6.0), u, 1.0) * t;
-                c = fma(fma(fma(-1.0 / 720.0, u, 1.0 / 24.0), u, -0.5), u, 1.0);
+                s = fma(fma(fma(fma(1.0 / 362880.0, u, -1.0 / 5040.0), u, 1.0 / 120.0), u, -1.0 / 6.0), u, 1.0) * t;
+                c = fma(fma(fma(fma(fma(-1.0 / 3628800.0, u, 1.0 / 40320.0), u, -1.0 / 720.0), u, 1.0 / 24.0), u, -0.5), u, 1.0);
             }
         } else {
             e = exp(a);
@@ -889,6 +892,7 @@ template <typename T, int N, int V> struct Pointwise {
     using C = typename Prec<T>::C;
     using SC = typename Prec<T>::S;
     static constexpr int G = P::G, E = P::E, R = P::R, H = P::H, M = P::M, S = P::S, NS = P::NS;
+    static constexpr bool RUN = sizeof(T) == 8 && H > 2;   // recurrence along a slot (factor_regs)
     static constexpr bool ADJ = sizeof(T) == 4;   // static rows: the two entries of a pair adjacent
 
     static __device__ __forceinline__ int jof(int g, int e) { return plan_j(g, e, R, M, G); }
@@ -970,7 +974,7 @@ template <typename T, int N, int V> struct Pointwise {
         const T qlim = fmax(-2 * A, fabs(Bpi));   // a >= -1/2 and |t| <= 1 where qlim j^2 <= 1
         cpx<T> qe;
         T qw;
-        if constexpr (sizeof(T) == 8) {
+        if constexpr (RUN) {
             const T s2 = (T)2 * S * S;
             qe = Dyn<double>::template cexp<PHASE>(A * s2, Bpi * s2, &qw);
             qw *= Dyn<double>::near1(D * s2);
@@ -980,7 +984,7 @@ template <typename T, int N, int V> struct Pointwise {
             int lo, hi;
             slot_points(g + t * G, R, M, lo, hi);
             Run ul, uh;
-            if constexpr (sizeof(T) == 8) {
+            if constexpr (RUN) {
                 ul.template start<PHASE>(A, Bpi, D, (T)lo);
                 uh.template start<PHASE>(A, Bpi, D, (T)hi);
             }
@@ -1019,10 +1023,15 @@ template <typename T, int N, int V> struct Pointwise {
                     for (int h = 0; h < 2; ++h) {
                         cpx<T> &xe = h ? x1 : x0;
                         Run &u = h ? uh : ul;
+                        if constexpr (!RUN) {
+                            const T j2 = (T)((h ? hi : lo) + S * m) * (T)((h ? hi : lo) + S * m);
+                            u.e = Dyn<double>::template cexp<PHASE>(A * j2, Bpi * j2, &u.w);
+                            u.w *= Dyn<double>::near1(D * j2);
+                        }
                         (h ? acc2 : acc).add_w(xe, u.w);
                         const cpx<T> w = PR::mul_s(xe, PR::ld_s(row + (2 * pr + h) * G + g));
                         xe = PHASE ? w * u.e : scale(w, u.e.x);
-                        if (m + 1 < H) u.template step<PHASE>(qe, qw);
+                        if (RUN && m + 1 < H) u.template step<PHASE>(qe, qw);
                     }
                 }
             }
@@ -1038,7 +1047,7 @@ template <typename T, int N, int V> struct Pointwise {
     {
         SqAcc<T> acc;
         const SC *tab = (mode == 1) ? tb.statV2 : tb.statV;
-#pragma unroll 1
+#pragma unroll 4
         for (int e = 0; e < E; ++e) {
             const T fj = (T)jof(g, e);
             T f1r, f1i, em1, z;

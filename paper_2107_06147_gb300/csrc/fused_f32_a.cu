@@ -10,8 +10,6 @@ cudaError_t fused_launch_f32_b(int N, const Tables<float> &tb, const LaunchArgs 
 cudaError_t fused_launch_f32(int N, const Tables<float> &tb, const LaunchArgs &a, int sm_count, int max_ctas,
                              cudaStream_t s, FusedInfo *info, bool query_only, int variant)
 {
-    // the per-step summary runs the traced twin of variant 0, the KSU potential its own kernel
-    if (a.trace_every > 0 || tb.potential == 1) variant = 0;
     switch (N) {
     case 16: return tb.potential == 1 ? ksu32_go<16>(tb, a, sm_count, max_ctas, s, info, query_only)
                                   : a.trace_every > 0 ? fused_go<float, 16, 4>(tb, a, sm_count, max_ctas, s, info, query_only)

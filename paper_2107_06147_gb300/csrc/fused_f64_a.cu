@@ -9,8 +9,6 @@ cudaError_t fused_launch_f64_b(int N, const Tables<double> &tb, const LaunchArgs
 cudaError_t fused_launch_f64(int N, const Tables<double> &tb, const LaunchArgs &a, int sm_count, int max_ctas,
                              cudaStream_t s, FusedInfo *info, bool query_only, int variant)
 {
-    // the per-step summary runs the traced twin of variant 0, the KSU potential its own twin of it
-    if (a.trace_every > 0 || tb.potential == 1) variant = 0;
     switch (N) {
     case 16: return tb.potential == 1 ? fused_go<double, 16, 5>(tb, a, sm_count, max_ctas, s, info, query_only)
                                   : a.trace_every > 0 ? fused_go<double, 16, 4>(tb, a, sm_count, max_ctas, s, info, query_only)

@@ -15,18 +15,37 @@ namespace qt {
 
 struct PlanDims { int R, E, M1, M2; };
 
-// rad8: the radix-8 plans of the launch variants 2 and 3 (FP32, N = 2048 and 4096)
-__host__ __device__ constexpr PlanDims plan_dims(int N, bool f64, bool rad8)
+// The plans.  FP32 up to N = 4096 and FP64: 16 values a thread where two warps of a trajectory then share an SM
+// quarter and its instruction fetch, 32 above (fewer exchanges).  Small grids run few trajectories at a time more
+// often than thousands, so theirs are the plans of the shortest step: an FP64 instruction takes a warp 64 cycles
+// whatever its lanes do and an SM completes one every 19, so FP64 wants four warps with little each (us a step of 8
+// trajectories / 10^6 trajectory-steps a second of a full device, FP64: N = 512 radix 4, 8 x 8 28.0 / 7.7, radix 8,
+// 16 41.9 / 8.5; N = 1024 radix 8, 8 x 4 44.4 / 3.9, radix 16, 8 65.7 / 4.6; N = 256 radix 4, 4 x 8 22.5 / 15.9,
+// radix 8, 8 34.4 / 16.9.  FP32: N = 512 radix 8, 16 2.9 / 226, radix 16, 4 4.2 / 284; N = 128 radix 4, 16 2.2 /
+// 642, radix 8, 4 2.9 / 602).  At N = 256 (FP32) and above the throughput lost outweighs the step.
+// RAD8: the radix-8 plans of the launch variants 2 and 3 (FP32, N = 2048 and 4096); PLAIN: the plain form's, one
+// middle pass and at most 32 of a sequence's slots (plain_step.cuh).
+enum PlanKind { PLAN_FUSED = 0, PLAN_RAD8 = 1, PLAN_PLAIN = 2 };
+__host__ __device__ constexpr PlanDims plan_dims(int N, bool f64, PlanKind kind)
 {
-    if (rad8 && !f64 && N == 2048) return {8, 16, 8, 8};
-    if (rad8 && !f64 && N == 4096) return {8, 16, 16, 8};
+    if (kind == PLAN_RAD8 && !f64 && N == 2048) return {8, 16, 8, 8};
+    if (kind == PLAN_RAD8 && !f64 && N == 4096) return {8, 16, 16, 8};
+    if (f64 && kind != PLAN_PLAIN) {
+        switch (N) {
+        case 128: return {4, 4, 4, 4};
+        case 256: return {4, 4, 4, 8};
+        case 512: return {4, 4, 8, 8};
+        case 1024: return {8, 8, 8, 4};
+        default: break;
+        }
+    }
     switch (N) {
     case 16: return {4, 4, 2, 1};
     case 32: return {4, 4, 4, 1};
     case 64: return {4, 4, 8, 1};
-    case 128: return {8, 8, 4, 1};
+    case 128: return {4, 4, 16, 1};
     case 256: return {8, 8, 8, 1};
-    case 512: return f64 ? PlanDims{8, 8, 16, 1} : PlanDims{16, 16, 4, 1};
+    case 512: return {8, 8, 16, 1};
     case 1024: return {16, 16, 8, 1};
     case 2048: return {16, 16, 16, 1};
     case 4096: return f64 ? PlanDims{16, 32, 32, 1} : PlanDims{16, 16, 32, 1};
@@ -87,9 +106,9 @@ struct Plan {
     bool tw_last;   // W_S^{b1 q1} is applied by the last pass (else by the middle one)
 };
 __host__ __device__ constexpr bool plan_tw_last(PlanDims d) { return d.M2 > 1 || d.M1 >= d.R; }
-inline Plan make_plan(int N, bool f64, int variant)
+inline Plan make_plan(int N, bool f64, PlanKind kind)
 {
-    const PlanDims d = plan_dims(N, f64, variant == 2 || variant == 3);
+    const PlanDims d = plan_dims(N, f64, kind);
     const int M = d.M1 * d.M2;
     return {N, d.R, d.E, M, d.M1, d.M2, N / d.E, d.R * M, N / d.R, plan_tw_last(d)};
 }

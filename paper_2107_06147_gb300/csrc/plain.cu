@@ -260,7 +260,7 @@ cudaError_t plain_run(const Tables<double> &tb, const LaunchArgs &a, int N, int 
     const int B = a.n_traj;
     if (B == 0) return cudaSuccess;
     const PlainOps *ops = ops_of(N);
-    const Plan p = make_plan(N, true, 0);
+    const Plan p = make_plan(N, true, PLAN_PLAIN);
     const Order ord{p.R, p.M, p.G};
     plain_setup<<<B, PB, 0, stream>>>(tb, a, buf.st, buf.psi, N, ord);
     plain_finalize_empty<<<B, PB, 0, stream>>>(tb, a, buf.st, buf.psi, N, ord);

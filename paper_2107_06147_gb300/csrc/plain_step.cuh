@@ -16,9 +16,9 @@ __device__ __forceinline__ bool plain_running(const PlainState &s, const TrajDev
 }
 
 template <int N> struct PlainStep {
-    using P = FusedPlan<double, N, 0>;
-    using K = Sine<double, N, 0>;
-    using PW = Pointwise<double, N, 0>;
+    using P = FusedPlan<double, N, 7>;
+    using K = Sine<double, N, 7>;
+    using PW = Pointwise<double, N, 7>;
     using PR = Prec<double>;
     static constexpr int G = P::G, E = P::E, R = P::R, H = P::H, M = P::M, S = P::S, NS = P::NS;
     static constexpr int TB = G < 32 ? G : 32, NB = G / TB;   // threads of a block, blocks of a trajectory
