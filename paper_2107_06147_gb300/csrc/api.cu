@@ -104,8 +104,10 @@ struct qtraj_ctx {
     // read-only tables
     void *W = nullptr, *WL = nullptr, *KT = nullptr, *sinpre = nullptr;   // FP32 KSU
     struct TabSet {   // the tables in the order of one plan (fused_plan.h)
-        void *KF = nullptr, *TA = nullptr, *TM = nullptr, *TI = nullptr, *TS = nullptr, *statV = nullptr, *statV2 = nullptr;
-        void **all[7] = {&KF, &TA, &TM, &TI, &TS, &statV, &statV2};
+        void *dirs = nullptr, *parts = nullptr;                           // KF | TA | TM | TI and TH | TS
+        size_t ta = 0, tm = 0, ti = 0, ts = 0;                            // where these begin
+        void *statV = nullptr, *statV2 = nullptr;
+        void **all[4] = {&dirs, &parts, &statV, &statV2};
     } fused, plain;
     double *eig = nullptr;
     double *ic = nullptr, *ov0 = nullptr;
@@ -256,59 +258,116 @@ template <typename V> qtraj_status upload(void **out, const std::vector<V> &v)
     return QTRAJ_OK;
 }
 
-// the transform's tables and the kinetic factors in the order of plan p
-template <typename T>
-qtraj_status build_set(const qtraj_ctx *c, qtraj_ctx::TabSet &t, const Plan &p, const std::vector<std::pair<double, double>> &kt)
+// Constants as directions (Prec<float>::D): a warp tries the 8193 float neighbours of the larger component and keeps
+// the pair of the nearest direction (the smallest step among equals), then the real factor that is left.  Pairs
+// within 64 steps are left out unless exact: y + y d with |d| near 2^-24 rounds back to y for every y, so a d that
+// small would be lost, always in the same sense (the no-jump norm then drifted by -5e-9 a step at N = 64; -4e-10
+// without them).  The search is in FP32: t = th + tl, the product p t in error-free parts.
+__global__ void find_directions(const cpx<double> *w, Prec<float>::D *out, int n)
 {
-    using PC = typename Prec<T>::C;
-    const int N = c->N;
-    auto root = [&](long k, long n) {   // exp(-2 pi i k / n)
-        const double a = -2.0 * PI * (double)(k % n) / (double)n;
-        return Prec<T>::make(std::cos(a), std::sin(a));
-    };
-    std::vector<PC> KF(N), TA((size_t)p.R / 2 * p.NS), TM(p.S), TI((size_t)p.M1 * p.M2), TS(p.R / 2);
-    for (int i = 0; i < N; ++i) {
-        int g, e;
-        plan_entry(i, false, p.R, p.G, g, e);
-        const int j = plan_j(g, e, p.R, p.M, p.G);
-        const double f = j == 0 ? 0.0 : -0.5 / N;   // two transforms X = -2i S, and the inverse's 2/N
-        KF[i] = Prec<T>::make(kt[j].first * f, kt[j].second * f);
+    const int i = (int)(blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32), lane = threadIdx.x & 31;
+    if (i >= n) return;
+    const cpx<double> z = w[i];
+    const bool sw = fabs(z.y) > fabs(z.x);
+    const double big = sw ? z.y : z.x, t = big != 0.0 ? (sw ? z.x : z.y) / big : 0.0;
+    const float p0 = (float)big, th = (float)t, tl = (float)(t - (double)th);
+    const bool exact = (double)p0 == big;
+    float best = 3e38f;
+    int at = 0;
+    for (int k = lane - 4096; k <= 4096; k += 32) {
+        const float p = __int_as_float(__float_as_int(p0) + k), h = p * th;
+        const float lo = fmaf(p, tl, fmaf(p, th, -h)), q = h + lo, err = fabsf((h - q) + lo);
+        if (abs(k) < 64 && !(k == 0 && err == 0.f && exact)) continue;
+        if (err < best || (err == best && abs(k) < abs(at))) {
+            best = err;
+            at = k;
+        }
     }
-    for (int s = 0; s < p.NS; ++s) {
-        int lo, hi;
-        slot_points(s, p.R, p.M, lo, hi);
-        for (int k = 1; k <= p.R / 2; ++k) TA[(size_t)(k - 1) * p.NS + s] = root((long)lo * k, 2L * N);
+    for (int off = 16; off > 0; off >>= 1) {
+        const float b = __shfl_xor_sync(0xffffffffu, best, off);
+        const int a = __shfl_xor_sync(0xffffffffu, at, off);
+        if (b < best || (b == best && (abs(a) < abs(at) || (abs(a) == abs(at) && a < at)))) {
+            best = b;
+            at = a;
+        }
     }
-    for (int b1 = 0; b1 < p.R; ++b1)
-        for (int q1 = 0; q1 < p.M; ++q1) TM[p.tw_last ? b1 * p.M + q1 : q1 * p.R + b1] = root((long)b1 * q1, p.S);
-    for (int k1 = 0; k1 < p.M1; ++k1)
-        for (int m2 = 0; m2 < p.M2; ++m2) TI[(size_t)k1 * p.M2 + m2] = root((long)m2 * k1, p.M);
-    for (int k = 1; k < p.R / 2; ++k) TS[k] = Prec<T>::make(0.5 / std::sin(PI * k / p.R), 0.5 / std::tan(PI * k / p.R));
-    qtraj_status st = QTRAJ_OK;
-    if ((st = upload(&t.KF, KF)) != QTRAJ_OK || (st = upload(&t.TA, TA)) != QTRAJ_OK || (st = upload(&t.TM, TM)) != QTRAJ_OK ||
-        (st = upload(&t.TI, TI)) != QTRAJ_OK)
-        return st;
-    return upload(&t.TS, TS);
+    if (lane == 0) {
+        const float p = p0 != 0.f ? __int_as_float(__float_as_int(p0) + at) : 0.f, q = (float)((double)p * t);
+        const double r = sw ? q : p, im = sw ? p : q, n2 = r * r + im * im;
+        out[i] = Prec<float>::D{(float)r, (float)im, n2 > 0.0 ? (float)((z.x * r + z.y * im) / n2 - 1.0) : 0.f, 0.f};
+    }
 }
 
-// the static potential rows in the order of plan p (nullptr: natural), of a half and (full) a whole step
+// The tables in the order of plan p: the transform's and the kinetic factors, and the static potential rows of a
+// half and (full) a whole step; p = nullptr: only the rows, in natural order.
 template <typename T>
-qtraj_status build_static(const qtraj_ctx *c, qtraj_ctx::TabSet &t, const Plan *p, const double *coul, bool full)
+qtraj_status build_set(const qtraj_ctx *c, qtraj_ctx::TabSet &t, const Plan *p, const double *coul, bool full,
+                       const std::vector<std::pair<double, double>> &kt)
 {
+    using PC = typename Prec<T>::C;
     using PS = typename Prec<T>::S;
-    const size_t n = (size_t)2 * LTAB * c->N;
-    if (cudaMalloc(&t.statV, sizeof(PS) * n) != cudaSuccess || (full && cudaMalloc(&t.statV2, sizeof(PS) * n) != cudaSuccess)) {
+    using Z = cpx<double>;
+    const int N = c->N;
+    std::vector<Z> dirs;
+    std::vector<PC> parts;
+    if (p) {
+        auto root = [&](long k, long n) {   // exp(-2 pi i k / n)
+            const double a = -2.0 * PI * (double)(k % n) / (double)n;
+            return Z{std::cos(a), std::sin(a)};
+        };
+        const int H = p->R / 2;
+        t.ta = N;
+        t.tm = t.ta + (size_t)(H - 1) * p->NS;
+        t.ti = t.tm + p->S;
+        t.ts = p->NS;
+        dirs.resize(t.ti + (size_t)p->M1 * p->M2);
+        parts.resize(t.ts + H);
+        for (int i = 0; i < N; ++i) {
+            int g, e;
+            plan_entry(i, false, p->R, p->G, g, e);
+            const int j = plan_j(g, e, p->R, p->M, p->G);
+            const double f = j == 0 ? 0.0 : -0.5 / N;   // two transforms X = -2i S, and the inverse's 2/N
+            dirs[i] = Z{kt[j].first * f, kt[j].second * f};
+        }
+        for (int s = 0; s < p->NS; ++s) {
+            int lo, hi;
+            slot_points(s, p->R, p->M, lo, hi);
+            for (int k = 1; k < H; ++k) dirs[t.ta + (size_t)(k - 1) * p->NS + s] = root((long)lo * k, 2L * N);
+            const Z th = root((long)lo * H, 2L * N);
+            parts[s] = Prec<T>::make(th.x, th.y);
+        }
+        for (int b1 = 0; b1 < p->R; ++b1)
+            for (int q1 = 0; q1 < p->M; ++q1)
+                dirs[t.tm + (p->tw_last ? b1 * p->M + q1 : q1 * p->R + b1)] = root((long)b1 * q1, p->S);
+        for (int k1 = 0; k1 < p->M1; ++k1)
+            for (int m2 = 0; m2 < p->M2; ++m2) dirs[t.ti + (size_t)k1 * p->M2 + m2] = root((long)m2 * k1, p->M);
+        for (int k = 1; k < H; ++k) parts[t.ts + k] = Prec<T>::make(0.5 / std::sin(PI * k / p->R), 0.5 / std::tan(PI * k / p->R));
+    }
+    const size_t n = (size_t)2 * LTAB * N;
+    if (cudaMalloc(&t.statV, sizeof(PS) * n) != cudaSuccess || (full && cudaMalloc(&t.statV2, sizeof(PS) * n) != cudaSuccess) ||
+        (p && (cudaMalloc(&t.dirs, sizeof(typename Prec<T>::D) * dirs.size()) != cudaSuccess ||
+               cudaMalloc(&t.parts, sizeof(PC) * parts.size()) != cudaSuccess))) {
         cudaGetLastError();
-        return fail(QTRAJ_ENOMEM, "cudaMalloc of the static space-kernel tables (%zu bytes)", (full ? 2 : 1) * sizeof(PS) * n);
+        return fail(QTRAJ_ENOMEM, "cudaMalloc of the tables (%zu bytes)", (full ? 2 : 1) * sizeof(PS) * n);
     }
     // a private non-blocking stream: building a context waits for nothing else on the device
     cudaStream_t s = nullptr;
     CK(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
+    cudaError_t e = cudaSuccess;
+    if (p) {
+        // (the constants in 64 bits pass through the memory of the rows, which are filled after them)
+        static_assert(sizeof(Z) * 4 <= sizeof(float) * 2 * 2 * LTAB, "dirs fit the rows");
+        void *w = sizeof(T) == 8 ? t.dirs : t.statV;
+        e = cudaMemcpyAsync(w, dirs.data(), sizeof(Z) * dirs.size(), cudaMemcpyHostToDevice, s);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(t.parts, parts.data(), sizeof(PC) * parts.size(), cudaMemcpyHostToDevice, s);
+        if (sizeof(T) == 4)
+            find_directions<<<((int)dirs.size() + 7) / 8, 256, 0, s>>>((const Z *)w, (Prec<float>::D *)t.dirs, (int)dirs.size());
+    }
     const int blocks = (int)std::min<size_t>((n + 255) / 256, 4096);
     for (int h = 0; h < (full ? 2 : 1); ++h)
-        stat_rows<T><<<blocks, 256, 0, s>>>((PS *)(h ? t.statV2 : t.statV), c->N, c->dr, c->M, c->dt, coul[0], coul[1],
+        stat_rows<T><<<blocks, 256, 0, s>>>((PS *)(h ? t.statV2 : t.statV), N, c->dr, c->M, c->dt, coul[0], coul[1],
                                             h ? 2.0 : 1.0, p ? p->R : 0, p ? p->M : 0, p ? p->G : 1);
-    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaGetLastError();
     const cudaError_t e2 = cudaStreamSynchronize(s);
     if (e == cudaSuccess) e = e2;
     cudaStreamDestroy(s);
@@ -416,19 +475,16 @@ template <typename T> qtraj_status build_tables(qtraj_ctx *c)
         if ((st = upload(&c->W, W)) != QTRAJ_OK || (st = upload(&c->KT, KT)) != QTRAJ_OK ||
             (st = upload(&c->sinpre, sp)) != QTRAJ_OK || (st = upload(&c->WL, WL)) != QTRAJ_OK)
             return st;
-        return build_static<T>(c, c->fused, nullptr, coul, true);
+        return build_set<T>(c, c->fused, nullptr, coul, true, kt);
     }
     // a plain context runs the fused kernel only for the vacuum evolution of its initial states
     const int variant = c->p.potential == 1 ? 0 : c->p.variant;
     const Plan pf = make_plan(N, sizeof(T) == 8, variant >= 2 ? PLAN_RAD8 : PLAN_FUSED), pp = make_plan(N, true, PLAN_PLAIN);
     qtraj_status st = QTRAJ_OK;
     if (c->p.form != QTRAJ_PLAIN || c->p.t_vacuum > 0)
-        if ((st = build_set<T>(c, c->fused, pf, kt)) != QTRAJ_OK || (st = build_static<T>(c, c->fused, &pf, coul, true)) != QTRAJ_OK)
-            return st;
-    if (c->p.form == QTRAJ_PLAIN)
-        if ((st = build_set<T>(c, c->plain, pp, kt)) != QTRAJ_OK || (st = build_static<T>(c, c->plain, &pp, coul, false)) != QTRAJ_OK)
-            return st;
-    return QTRAJ_OK;
+        if ((st = build_set<T>(c, c->fused, &pf, coul, true, kt)) != QTRAJ_OK) return st;
+    if (c->p.form == QTRAJ_PLAIN) st = build_set<T>(c, c->plain, &pp, coul, false, kt);
+    return st;
 }
 
 // the kernels' view of the context; plain: with the plain form's tables
@@ -437,15 +493,17 @@ template <typename T> Tables<T> tables(const qtraj_ctx *c, bool plain = false)
     const qtraj_ctx::TabSet &ts = plain ? c->plain : c->fused;
     Tables<T> t;
     using PC = typename Prec<T>::C;
+    using PD = typename Prec<T>::D;
     t.W = (const PC *)c->W;
     t.WL = (const PC *)c->WL;
     t.KT = (const PC *)c->KT;
     t.sinpre = (const typename Prec<T>::Rl *)c->sinpre;
-    t.KF = (const PC *)ts.KF;
-    t.TA = (const PC *)ts.TA;
-    t.TM = (const PC *)ts.TM;
-    t.TI = (const PC *)ts.TI;
-    t.TS = (const PC *)ts.TS;
+    t.KF = (const PD *)ts.dirs;
+    t.TA = t.KF + ts.ta;
+    t.TH = (const PC *)ts.parts;
+    t.TM = t.KF + ts.tm;
+    t.TI = t.KF + ts.ti;
+    t.TS = t.TH + ts.ts;
     t.statV = (const typename Prec<T>::S *)ts.statV;
     t.statV2 = (const typename Prec<T>::S *)ts.statV2;
     t.eig = c->eig;

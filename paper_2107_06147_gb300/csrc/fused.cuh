@@ -587,11 +587,13 @@ template <typename T> __device__ __forceinline__ void ksu_point(const Tables<T> 
     vi = -k.gI * ksu_phi(tb, x);
 }
 
-// in-place DFT of RR values (natural order in); output k lands in slot operm(k)
-template <typename T, int RR> struct DFTI {
+// in-place DFT of RR values (natural order in); output k lands in slot operm(k).  HL: the FP32 constants in hi + lo
+// parts (the KSU kernel), else as directions (Prec<float>::D)
+template <typename T, int RR, bool HL = false> struct DFTI {
+    static __device__ __forceinline__ cpx<T> tw(cpx<T> a, int j) { return HL ? tw16<T>(a, j) : tw32<T>(a, 2 * j); }
     static __device__ __forceinline__ constexpr int operm(int k)
     {
-        if constexpr (RR == 32) return (k % 4) * 8 + DFTI<T, 8>::operm(k / 4);
+        if constexpr (RR == 32) return (k % 4) * 8 + DFTI<T, 8, HL>::operm(k / 4);
         else if constexpr (RR == 16) return (k % 4) * 4 + k / 4;
         else if constexpr (RR == 8) return (k % 4) * 2 + k / 4;
         else return k;
@@ -607,14 +609,14 @@ template <typename T, int RR> struct DFTI {
                 x[24 + n2] = tw32<T>(x[24 + n2], n2 * 3);
             }
 #pragma unroll
-            for (int k1 = 0; k1 < 4; ++k1) DFTI<T, 8>::run(x + 8 * k1);
+            for (int k1 = 0; k1 < 4; ++k1) DFTI<T, 8, HL>::run(x + 8 * k1);
         } else if constexpr (RR == 16) {
 #pragma unroll
             for (int n2 = 0; n2 < 4; ++n2) {
                 dft4(x[n2], x[4 + n2], x[8 + n2], x[12 + n2]);       // k1 of column n2 at slot n2 + 4 k1
-                x[4 + n2] = tw16<T>(x[4 + n2], n2 * 1);
-                x[8 + n2] = tw16<T>(x[8 + n2], n2 * 2);
-                x[12 + n2] = tw16<T>(x[12 + n2], n2 * 3);
+                x[4 + n2] = tw(x[4 + n2], n2 * 1);
+                x[8 + n2] = tw(x[8 + n2], n2 * 2);
+                x[12 + n2] = tw(x[12 + n2], n2 * 3);
             }
 #pragma unroll
             for (int k1 = 0; k1 < 4; ++k1) dft4(x[4 * k1], x[4 * k1 + 1], x[4 * k1 + 2], x[4 * k1 + 3]);
@@ -622,9 +624,9 @@ template <typename T, int RR> struct DFTI {
 #pragma unroll
             for (int n2 = 0; n2 < 2; ++n2) {
                 dft4(x[n2], x[2 + n2], x[4 + n2], x[6 + n2]);        // k1 of column n2 at slot n2 + 2 k1
-                x[2 + n2] = tw16<T>(x[2 + n2], 2 * n2 * 1);
-                x[4 + n2] = tw16<T>(x[4 + n2], 2 * n2 * 2);
-                x[6 + n2] = tw16<T>(x[6 + n2], 2 * n2 * 3);
+                x[2 + n2] = tw(x[2 + n2], 2 * n2 * 1);
+                x[4 + n2] = tw(x[4 + n2], 2 * n2 * 2);
+                x[6 + n2] = tw(x[6 + n2], 2 * n2 * 3);
             }
 #pragma unroll
             for (int k1 = 0; k1 < 4; ++k1) dft2(x[2 * k1], x[2 * k1 + 1]);
@@ -650,10 +652,11 @@ template <typename T, int N, int V> struct Sine {
     using PR = Prec<T>;
     using C = typename Prec<T>::C;
     static constexpr int R = P::R, H = P::H, G = P::G, M = P::M, S = P::S, NS = P::NS, SEQ = P::SEQ;
-    // (the hi+lo products stay scalar: as packed FP32x2 instructions, with their operands regrouped, they ran 8%
+    // (the products stay scalar: as packed FP32x2 instructions, with their operands regrouped, hi+lo products ran 8%
     // slower at N = 8192 and 4% at 16384)
+    using D = typename Prec<T>::D;
     using DR = DFTI<T, R>;
-    static __device__ __forceinline__ cpx<T> cmul(cpx<T> x, C w) { return PR::mul(x, w); }
+    static __device__ __forceinline__ cpx<T> cmul(cpx<T> x, D w) { return PR::muld(x, w); }
     static __device__ __forceinline__ cpx<T> neg(cpx<T> a) { return mk(-a.x, -a.y); }
 
     // addresses of position b of a sequence and of its mirror S - b
@@ -697,7 +700,8 @@ template <typename T, int N, int V> struct Sine {
 
     // First pass: the slots' DFTs, twiddles, and the writes of every sequence at b and -b.  pb, pm: the
     // addresses of b and S - b of the thread's slots.
-    static __device__ __forceinline__ void first(cpx<T> *x, cpx<T> *buf, const C *ta, int g, const int *pb, const int *pm)
+    static __device__ __forceinline__ void first(cpx<T> *x, cpx<T> *buf, const D *ta, const C *tha, int g,
+                                                 const int *pb, const int *pm)
     {
         if (g == 0) special_in(x);
 #pragma unroll
@@ -707,16 +711,16 @@ template <typename T, int N, int V> struct Sine {
             if (t == 0 && g == 0) {
                 special_out(v, buf);
             } else {
-                const C *w = ta + g + t * G;
+                const D *w = ta + g + t * G;
                 cpx<T> *ob = buf + pb[t], *om = buf + pm[t];
 #pragma unroll
                 for (int k = 1; k < H; ++k) {
-                    const C wk = PR::ld(w + (k - 1) * P::NSLOT);
+                    const D wk = PR::ldd(w + (k - 1) * P::NSLOT);
                     ob[k * SEQ] = cmul(v[DR::operm(k)], wk);
-                    om[k * SEQ] = cmul(v[DR::operm(R - k)], PR::nconj(wk));
+                    om[k * SEQ] = cmul(v[DR::operm(R - k)], PR::ncj(wk));
                 }
                 // the sequence P = U + V at b: u + th z, at -b: -u - conj(th) z, th = e^(-i pi b/S)
-                const C th = PR::ld(w + (H - 1) * P::NSLOT);
+                const C th = PR::ld(tha + g + t * G);
                 const cpx<T> u = v[0], z = v[DR::operm(H)];
                 const cpx<T> s = PR::mulr(z, PR::re(th)), d = PR::mulr(z, PR::im(th));
                 const cpx<T> a = u + s, b = mul_i(d);
@@ -730,7 +734,7 @@ template <typename T, int N, int V> struct Sine {
     // b1 + R (LO o + LM m), m < RM.  TW 0: none, 1: the last pass's twiddle W_S^(b1 q1) from tm [q1][b1]
     // (M2 = 1), 2: the inner twiddle W_M^(m2 k1) from ti [k1][m2] (o = m2).
     template <int RM, int RO, int LO, int LM, int TW, bool FIRST>
-    static __device__ __forceinline__ void mid_pass(cpx<T> *x, cpx<T> *buf, const C *tw, const C *ts, int g)
+    static __device__ __forceinline__ void mid_pass(cpx<T> *x, cpx<T> *buf, const D *tw, const C *ts, int g)
     {
         constexpr int NB = N / RM, PER = (NB + G - 1) / G;
         const int b1 = g % R;   // the same for all of a thread's butterflies (R divides G)
@@ -749,14 +753,14 @@ template <typename T, int N, int V> struct Sine {
         }
 #pragma unroll
         for (int m = 0; m < RM; ++m) {
-            C w{};
-            if (m && TW == 1) w = PR::ld(tw + m * R + b1);
+            D w{};
+            if (m && TW == 1) w = PR::ldd(tw + m * R + b1);
 #pragma unroll
             for (int q = 0; q < PER; ++q) {
                 const int i = g + q * G;
                 if (NB % G == 0 || i < NB) {
                     const int o = i / R % RO, kk = i / (R * RO);
-                    if (m && TW == 2) w = PR::ld(tw + m * RO + o);
+                    if (m && TW == 2) w = PR::ldd(tw + m * RO + o);
                     cpx<T> v = x[q * RM + DFTI<T, RM>::operm(m)];
                     if (m && TW) v = cmul(v, w);
                     buf[kk * SEQ + b1 + (R + 1) * (LO * o + LM * m)] = v;
@@ -765,7 +769,7 @@ template <typename T, int N, int V> struct Sine {
         }
     }
 
-    static __device__ __forceinline__ void mid(cpx<T> *x, cpx<T> *buf, const C *tm, const C *ti, const C *ts, int g)
+    static __device__ __forceinline__ void mid(cpx<T> *x, cpx<T> *buf, const D *tm, const D *ti, const C *ts, int g)
     {
         if constexpr (P::M2 == 1) {
             mid_pass<P::M1, 1, 0, 1, P::TWL ? 0 : 1, true>(x, buf, tm, ts, g);
@@ -778,21 +782,21 @@ template <typename T, int N, int V> struct Sine {
     }
 
     // Last pass: X_{b + S q2} into value q2 of every slot (natural order)
-    static __device__ __forceinline__ void last(cpx<T> *x, cpx<T> *buf, const C *tm, int g)
+    static __device__ __forceinline__ void last(cpx<T> *x, cpx<T> *buf, const D *tm, int g)
     {
         constexpr bool SAME = G % M == 0;   // a thread's slots share q1
         cpx<T> y[NS * R];
 #pragma unroll
         for (int b1 = 0; b1 < R; ++b1) {
-            C w{};
-            if (P::TWL && SAME && b1) w = PR::ld(tm + b1 * M + g % M);
+            D w{};
+            if (P::TWL && SAME && b1) w = PR::ldd(tm + b1 * M + g % M);
 #pragma unroll
             for (int t = 0; t < NS; ++t) {
                 const int s = g + t * G, q1 = s % M;
                 const int loc = P::M2 == 1 ? q1 : q1 / P::M1 + P::M2 * (q1 % P::M1);
                 cpx<T> v = buf[s / M * SEQ + (R + 1) * loc + b1];
                 if (P::TWL && b1) {
-                    if (!SAME) w = PR::ld(tm + b1 * M + q1);
+                    if (!SAME) w = PR::ldd(tm + b1 * M + q1);
                     v = cmul(v, w);
                 }
                 y[t * R + b1] = v;
@@ -813,7 +817,7 @@ template <typename T, int N, int V> struct Sine {
     // P_{-i}) for q < S/2, through the kk = 0 sequence's own shared memory: each of LN lanes of warp 0 sums a run of
     // CH values, the runs' totals are scanned with shuffles, and V overwrites P's lower half (only the run's
     // owner reads it; the upper half stays).  The sum carries the rounding errors of at most S/2 values of
-    // 2/R of the spectrum.  For M > 32 (radix-8 variants) warp 0 sums for all and every thread calls this.
+    // 2/R of the spectrum, both ends tied down.  For M > 32 (radix-8 variants) warp 0 sums for all and every thread calls this.
     static __device__ __forceinline__ void split(cpx<T> *x, cpx<T> *buf, int g)
     {
         constexpr int LN = G < 32 ? G : 32, CH = S / 2 / LN;
@@ -846,8 +850,13 @@ template <typename T, int N, int V> struct Sine {
             }
             cpx<T> ex = mk<T>(__shfl_up_sync(mask, inc.x, 1, LN), __shfl_up_sync(mask, inc.y, 1, LN));
             if (g == 0) ex = mk<T>(0, 0);
+            // the sum's other end is known too, V_{S/2-1} = -P_{S/2}: what it misses is spread linearly over the sum,
+            // which takes the rounding errors of a random walk to those of a bridge (a third of the variance)
+            const cpx<T> end = mk<T>(__shfl_sync(mask, inc.x, LN - 1, LN), __shfl_sync(mask, inc.y, LN - 1, LN));
+            const cpx<T> miss = scale(end + buf[pos(S / 2)], (T)(-2.0 / S));
+            ex = ex + scale(miss, (T)(g * CH + 1));
 #pragma unroll
-            for (int i = 0; i < CH; ++i) buf[pos(g * CH + i)] = ex + c[i];
+            for (int i = 0; i < CH; ++i) buf[pos(g * CH + i)] = ex + (c[i] + scale(miss, (T)i));
         }
         sync();
         if (g < M) {
@@ -868,13 +877,13 @@ template <typename T, int N, int V> struct Sine {
     }
 
     // S <- K_T S on the register values (kf: two rows of G entries per pair of values)
-    static __device__ __forceinline__ void kinetic(cpx<T> *x, const C *kf, int g)
+    static __device__ __forceinline__ void kinetic(cpx<T> *x, const D *kf, int g)
     {
 #pragma unroll
         for (int pr = 0; pr < NS * H; ++pr) {
             const int e0 = pr / H * R + pr % H, e1 = pr / H * R + R - 1 - pr % H;
-            x[e0] = cmul(x[e0], PR::ld(kf + (2 * pr) * G + g));
-            x[e1] = cmul(x[e1], PR::ld(kf + (2 * pr + 1) * G + g));
+            x[e0] = cmul(x[e0], PR::ldd(kf + (2 * pr) * G + g));
+            x[e1] = cmul(x[e1], PR::ldd(kf + (2 * pr + 1) * G + g));
         }
     }
 };
@@ -1412,7 +1421,7 @@ __global__ void __launch_bounds__(FusedPlan<T, N, V>::G, (FusedBounds<T, N, V>::
             K3b = kappa_T3<T>(mp->kfit, T3b);
 #pragma unroll 1
             for (int h = 0; h < 2; ++h) {
-                K::first(x, buf, tb.TA, g, pb, pm);
+                K::first(x, buf, tb.TA, tb.TH, g, pb, pm);
                 traj_sync<G>();
                 K::mid(x, buf, tb.TM, tb.TI, tb.TS, g);
                 traj_sync<G>();

@@ -77,7 +77,7 @@ template <int N> struct NftSine {
     using C = typename Prec<T>::C;
     using RL = typename Prec<T>::Rl;
     static constexpr int R = P::R, G = P::G, NR = P::NR, E = 2 * R;
-    using DR = DFTI<T, R>;
+    using DR = DFTI<T, R, true>;
     static __device__ __forceinline__ cpx<T> cmul(cpx<T> x, C w) { return PR::mul(x, w); }
 
     static __device__ __forceinline__ int pad(int j) { return j + j / R; }
@@ -207,10 +207,10 @@ template <int N> struct NftSine {
 #pragma unroll
             for (int q = 0; q < PER; ++q) {
                 const int i = g + q * G;
-                DFTI<T, RM>::run(x + q * RM);
+                DFTI<T, RM, true>::run(x + q * RM);
                 const int base = (i - k) * RM + k;
 #pragma unroll
-                for (int m = 0; m < RM; ++m) buf[pad(base + m * PP)] = x[q * RM + DFTI<T, RM>::operm(m)];
+                for (int m = 0; m < RM; ++m) buf[pad(base + m * PP)] = x[q * RM + DFTI<T, RM, true>::operm(m)];
             }
             __syncthreads();
         }

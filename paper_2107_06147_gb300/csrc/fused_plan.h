@@ -21,8 +21,9 @@ struct PlanDims { int R, E, M1, M2; };
 // whatever its lanes do and an SM completes one every 19, so FP64 wants four warps with little each (us a step of 8
 // trajectories / 10^6 trajectory-steps a second of a full device, FP64: N = 512 radix 4, 8 x 8 28.0 / 7.7, radix 8,
 // 16 41.9 / 8.5; N = 1024 radix 8, 8 x 4 44.4 / 3.9, radix 16, 8 65.7 / 4.6; N = 256 radix 4, 4 x 8 22.5 / 15.9,
-// radix 8, 8 34.4 / 16.9.  FP32: N = 512 radix 8, 16 2.9 / 226, radix 16, 4 4.2 / 284; N = 128 radix 4, 16 2.2 /
-// 642, radix 8, 4 2.9 / 602).  At N = 256 (FP32) and above the throughput lost outweighs the step.
+// radix 8, 8 34.4 / 16.9.  FP32: N = 128 radix 4, 16 2.2 / 642, radix 8, 4 2.9 / 602).  FP32 at N = 256 and above
+// keeps the larger radix: the throughput lost outweighs the step (N = 512 radix 8, 16 2.9 / 226, radix 16, 4 4.2 /
+// 284), and the share of the spectrum that goes through a running sum, 2/R, sets the rounding noise.
 // RAD8: the radix-8 plans of the launch variants 2 and 3 (FP32, N = 2048 and 4096); PLAIN: the plain form's, one
 // middle pass and at most 32 of a sequence's slots (plain_step.cuh).
 enum PlanKind { PLAN_FUSED = 0, PLAN_RAD8 = 1, PLAN_PLAIN = 2 };
@@ -45,7 +46,7 @@ __host__ __device__ constexpr PlanDims plan_dims(int N, bool f64, PlanKind kind)
     case 64: return {4, 4, 8, 1};
     case 128: return {4, 4, 16, 1};
     case 256: return {8, 8, 8, 1};
-    case 512: return {8, 8, 16, 1};
+    case 512: return f64 ? PlanDims{8, 8, 16, 1} : PlanDims{16, 16, 4, 1};
     case 1024: return {16, 16, 8, 1};
     case 2048: return {16, 16, 16, 1};
     case 4096: return f64 ? PlanDims{16, 32, 32, 1} : PlanDims{16, 16, 32, 1};

@@ -90,7 +90,7 @@ __global__ void __launch_bounds__(PlainStep<N>::TB) plain_first(Tables<double> t
 #pragma unroll
     for (int e = 0; e < L::E; ++e) x[e] = psi[e * L::G + p.g];
     L::half_step(x, tb, tb.media[a.trajs[p.b].medium], buf.st[p.b].c, buf.st[p.b].l, n, p.g);
-    L::K::first(x, buf.sa + (size_t)p.b * L::P::BUF, tb.TA, p.g, p.pb, p.pm);
+    L::K::first(x, buf.sa + (size_t)p.b * L::P::BUF, tb.TA, tb.TH, p.g, p.pb, p.pm);
 }
 
 template <int N>
@@ -113,7 +113,7 @@ __global__ void __launch_bounds__(PlainStep<N>::TB) plain_kinetic(Tables<double>
     cpx<double> x[L::P::XN];
     L::K::last(x, buf.sa + (size_t)p.b * L::P::BUF, tb.TM, p.g);
     L::K::kinetic(x, tb.KF, p.g);
-    L::K::first(x, buf.sb + (size_t)p.b * L::P::BUF, tb.TA, p.g, p.pb, p.pm);
+    L::K::first(x, buf.sb + (size_t)p.b * L::P::BUF, tb.TA, tb.TH, p.g, p.pb, p.pm);
 }
 
 // end of the step: last pass, space half-step, the block's part of the norm
