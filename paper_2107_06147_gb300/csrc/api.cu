@@ -106,8 +106,8 @@ struct qtraj_ctx {
     struct TabSet {   // the tables in the order of one plan (fused_plan.h)
         void *dirs = nullptr, *parts = nullptr;                           // KF | TA | TM | TI and TH | TS
         size_t ta = 0, tm = 0, ti = 0, ts = 0;                            // where these begin
-        void *statV = nullptr, *statV2 = nullptr;
-        void **all[4] = {&dirs, &parts, &statV, &statV2};
+        void *statV = nullptr, *statV2 = nullptr, *eigo = nullptr;
+        void **all[5] = {&dirs, &parts, &statV, &statV2, &eigo};
     } fused, plain;
     double *eig = nullptr;
     double *ic = nullptr, *ov0 = nullptr;
@@ -310,6 +310,15 @@ qtraj_status build_set(const qtraj_ctx *c, qtraj_ctx::TabSet &t, const Plan *p, 
     const int N = c->N;
     std::vector<Z> dirs;
     std::vector<PC> parts;
+    std::vector<typename Prec<T>::Rl> eigo;
+    if (p && full) {   // the overlap basis in the order of the values, with the odd extension's sign
+        eigo.resize((size_t)NBASIS * N);
+        for (int i = 0; i < N; ++i) {
+            const int g = i % p->G, e = i / p->G, j = plan_j(g, e, p->R, p->M, p->G);
+            const double sg = e % p->R < p->R / 2 ? 1.0 : -1.0;
+            for (int b = 0; b < NBASIS; ++b) eigo[(size_t)b * N + i] = Prec<T>::make_r(sg * c->basis_host[(size_t)b * N + j]);
+        }
+    }
     if (p) {
         auto root = [&](long k, long n) {   // exp(-2 pi i k / n)
             const double a = -2.0 * PI * (double)(k % n) / (double)n;
@@ -346,7 +355,8 @@ qtraj_status build_set(const qtraj_ctx *c, qtraj_ctx::TabSet &t, const Plan *p, 
     const size_t n = (size_t)2 * LTAB * N;
     if (cudaMalloc(&t.statV, sizeof(PS) * n) != cudaSuccess || (full && cudaMalloc(&t.statV2, sizeof(PS) * n) != cudaSuccess) ||
         (p && (cudaMalloc(&t.dirs, sizeof(typename Prec<T>::D) * dirs.size()) != cudaSuccess ||
-               cudaMalloc(&t.parts, sizeof(PC) * parts.size()) != cudaSuccess))) {
+               cudaMalloc(&t.parts, sizeof(PC) * parts.size()) != cudaSuccess ||
+               (full && cudaMalloc(&t.eigo, sizeof(eigo[0]) * eigo.size()) != cudaSuccess)))) {
         cudaGetLastError();
         return fail(QTRAJ_ENOMEM, "cudaMalloc of the tables (%zu bytes)", (full ? 2 : 1) * sizeof(PS) * n);
     }
@@ -360,6 +370,8 @@ qtraj_status build_set(const qtraj_ctx *c, qtraj_ctx::TabSet &t, const Plan *p, 
         void *w = sizeof(T) == 8 ? t.dirs : t.statV;
         e = cudaMemcpyAsync(w, dirs.data(), sizeof(Z) * dirs.size(), cudaMemcpyHostToDevice, s);
         if (e == cudaSuccess) e = cudaMemcpyAsync(t.parts, parts.data(), sizeof(PC) * parts.size(), cudaMemcpyHostToDevice, s);
+        if (e == cudaSuccess && full)
+            e = cudaMemcpyAsync(t.eigo, eigo.data(), sizeof(eigo[0]) * eigo.size(), cudaMemcpyHostToDevice, s);
         if (sizeof(T) == 4)
             find_directions<<<((int)dirs.size() + 7) / 8, 256, 0, s>>>((const Z *)w, (Prec<float>::D *)t.dirs, (int)dirs.size());
     }
@@ -504,6 +516,7 @@ template <typename T> Tables<T> tables(const qtraj_ctx *c, bool plain = false)
     t.TM = t.KF + ts.tm;
     t.TI = t.KF + ts.ti;
     t.TS = t.TH + ts.ts;
+    t.eigo = (const typename Prec<T>::Rl *)ts.eigo;
     t.statV = (const typename Prec<T>::S *)ts.statV;
     t.statV2 = (const typename Prec<T>::S *)ts.statV2;
     t.eig = c->eig;

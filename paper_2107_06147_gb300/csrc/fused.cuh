@@ -124,6 +124,12 @@ template <int G> __device__ __forceinline__ unsigned lane_mask()
     return G >= 32 ? 0xffffffffu : ((1u << G) - 1u);
 }
 
+template <int G> __device__ __forceinline__ void traj_sync()
+{
+    if constexpr (G > 32) __syncthreads();
+    else __syncwarp(lane_mask<G>());
+}
+
 // combines per-warp totals (equal in every lane of a warp) across the G threads of a trajectory in a
 // fixed order; red holds >= G/32 doubles
 template <int G> __device__ __forceinline__ double cross_warp(double v, double *red)
@@ -152,30 +158,78 @@ template <int G> __device__ __forceinline__ double slot_sum(double v, double *re
     return cross_warp<G>(v, red);
 }
 
-// the same for K values at once, with two barriers in all; red holds >= K G/32 doubles
-template <int G, int K> __device__ __forceinline__ void slot_sums(double (&v)[K], double *red)
+// Eight sums over the G threads of a trajectory, left in fin[0..8) for the threads of its first warp.  The warp sums
+// by halving -- each lane passes half of its values on and keeps the sums of the other half, 9 additions instead of
+// 40 -- and the first eight lanes add the warps' sums: an FP64 addition takes a warp 64 cycles.  red holds >= 8 G/32
+// doubles.
+template <int G> __device__ __forceinline__ void slot_sums8(double (&v)[8], double *red, double *fin)
 {
-    constexpr int W = G < 32 ? G : 32;
+    constexpr int W = G < 32 ? G : 32, NW = G < 32 ? 1 : G / 32;
     const unsigned mask = lane_mask<G>();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int at = 0;   // the value this lane is left with
+    if constexpr (W == 32) {
 #pragma unroll
-    for (int i = 0; i < K; ++i) {
+        for (int k = 4, off = 16; k > 0; k >>= 1, off >>= 1) {
+            const bool up = lane & off;
 #pragma unroll
-        for (int off = W / 2; off > 0; off >>= 1) v[i] += __shfl_xor_sync(mask, v[i], off, W);
-        if constexpr (G <= 32) v[i] = __shfl_sync(mask, v[i], 0, W);
-        else if ((threadIdx.x & 31) == 0) red[i * (G / 32) + (threadIdx.x >> 5)] = v[i];
-    }
-    if constexpr (G > 32) {
-        __syncthreads();
-#pragma unroll
-        for (int i = 0; i < K; ++i) {
-            double s = 0.0;
-#pragma unroll
-            for (int w = 0; w < G / 32; ++w) s += red[i * (G / 32) + w];
-            v[i] = s;
+            for (int i = 0; i < k; ++i) {
+                const double mine = up ? v[i + k] : v[i], his = up ? v[i] : v[i + k];
+                v[i] = mine + __shfl_xor_sync(mask, his, off, W);
+            }
+            at += up ? k : 0;
         }
-        __syncthreads();
+#pragma unroll
+        for (int off = 2; off > 0; off >>= 1) v[0] += __shfl_xor_sync(mask, v[0], off, W);
+        if ((lane & 3) == 0) red[at * NW + warp] = v[0];
+    } else {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+#pragma unroll
+            for (int off = W / 2; off > 0; off >>= 1) v[i] += __shfl_xor_sync(mask, v[i], off, W);
+            if (lane == 0) red[i] = v[i];
+        }
+    }
+    traj_sync<G>();
+    if (warp == 0) {
+        for (int i = lane; i < 8; i += W) {
+            double t = 0.0;
+            for (int w = 0; w < NW; ++w) t += red[i * NW + w];
+            fin[i] = t;
+        }
+        __syncwarp(mask);
     }
 }
+
+// A sum of products f u with a constant real f = h + l and FP32 complex u, both parts at once in packed FP32x2
+// instructions: products and partial sums in error-free parts (the Dot2 scheme of Ogita, Rump and Oishi), some 2^-46
+// of the terms' magnitudes.
+struct Dot2 {
+    float2 s = make_float2(0.f, 0.f), c = make_float2(0.f, 0.f);
+    static __device__ __forceinline__ float2 neg(float2 a) { return make_float2(-a.x, -a.y); }
+    __device__ __forceinline__ void add(float2 f, float2 u)   // f u, componentwise
+    {
+        const float2 p = __fmul2_rn(f, u), r = __ffma2_rn(f, u, neg(p));
+        const float2 t = __fadd2_rn(s, p), b = __fadd2_rn(t, neg(s));
+        const float2 e = __fadd2_rn(__fadd2_rn(s, neg(__fadd2_rn(t, neg(b)))), __fadd2_rn(p, neg(b)));
+        c = __fadd2_rn(c, __fadd2_rn(e, r));
+        s = t;
+    }
+    __device__ __forceinline__ void add(Prec<float>::Rl f, float2 u)
+    {
+        add(make_float2(f.h, f.h), u);
+        c = __ffma2_rn(make_float2(f.l, f.l), u, c);
+    }
+    __device__ __forceinline__ double x() const { return (double)s.x + (double)c.x; }
+    __device__ __forceinline__ double y() const { return (double)s.y + (double)c.y; }
+};
+struct Dot1 {   // the FP64 form
+    double s = 0.0, t = 0.0;
+    __device__ __forceinline__ void add(double f, cpx<double> u) { s = fma(f, u.x, s); t = fma(f, u.y, t); }
+    __device__ __forceinline__ void sq(cpx<double> u) { s = fma(u.x, u.x, s); t = fma(u.y, u.y, t); }
+    __device__ __forceinline__ double x() const { return s; }
+    __device__ __forceinline__ double y() const { return t; }
+};
 
 // squared norm over the G threads of a trajectory; FP32 forms reduce in double-float all the way and
 // convert once, so no FP64 instruction is needed per thread beyond the final conversion
@@ -641,12 +695,6 @@ template <typename T, int RR, bool HL = false> struct DFTI {
 // ------------------------------------------------------------------------------------------------
 // the sine transform
 // ------------------------------------------------------------------------------------------------
-template <int G> __device__ __forceinline__ void traj_sync()
-{
-    if constexpr (G > 32) __syncthreads();
-    else __syncwarp(lane_mask<G>());
-}
-
 template <typename T, int N, int V> struct Sine {
     using P = FusedPlan<T, N, V>;
     using PR = Prec<T>;
@@ -974,10 +1022,12 @@ template <typename T, int N, int V> struct Pointwise {
     // exact j^2 (N <= 4096; rounded once above), so no rounding that repeats identically every step enters.
     // exp(2 er_a r^2) = mag exp((er_a - er_b) r^2), the second factor 1 + z with |z| <~ 1e-4 (the temperature's
     // change over one step): FP32 keeps the first order.
+    // The first half-step of a trajectory and the last of its last step are the same with the half-step rows and
+    // only one half-step's coefficients (last: the sum is |x_new|^2).
     // PHASE = false: gamma_hat = 0, B = 0 exactly, the phase series is skipped (its value would be 0).
     template <bool PHASE>
-    static __device__ __forceinline__ void factor_regs(cpx<T> *x, const SC *row, int g, T A, T B, T D, SqAcc<T> &acc,
-                                                       SqAcc<T> &acc2)
+    static __device__ __forceinline__ void factor_regs(cpx<T> *x, const SC *row, int g, T A, T B, T D, bool last,
+                                                       SqAcc<T> &acc, SqAcc<T> &acc2)
     {
         const T Bpi = (T)3.14159265358979323846 * B;
         const T qlim = fmax(-2 * A, fabs(Bpi));   // a >= -1/2 and |t| <= 1 where qlim j^2 <= 1
@@ -1020,8 +1070,10 @@ template <typename T, int N, int V> struct Pointwise {
                         else Dyn<float>::far2(a2, t2, &fr, &fi, &em);
                         fr = em;
                     }
-                    const float2 z = __fmul2_rn(make_float2(D, D), j2);
-                    const float2 mag = __fadd2_rn(make_float2(1.f, 1.f), em), wt = __ffma2_rn(mag, z, mag);
+                    const float2 mag = __fadd2_rn(make_float2(1.f, 1.f), em);
+                    float2 z = __fmul2_rn(make_float2(D, D), j2);
+                    z = make_float2(last ? em.x : z.x, last ? em.y : z.y);   // (last: |x_new|^2 = mag^2 |x_old|^2)
+                    const float2 wt = __ffma2_rn(mag, z, mag);
                     acc.add_w(x0, wt.x);
                     acc2.add_w(x1, wt.y);
                     const cpx<T> w0 = PR::mul_s(x0, mk(st.x, st.y)), w1 = PR::mul_s(x1, mk(st.z, st.w));
@@ -1037,9 +1089,10 @@ template <typename T, int N, int V> struct Pointwise {
                             u.e = Dyn<double>::template cexp<PHASE>(A * j2, Bpi * j2, &u.w);
                             u.w *= Dyn<double>::near1(D * j2);
                         }
-                        (h ? acc2 : acc).add_w(xe, u.w);
                         const cpx<T> w = PR::mul_s(xe, PR::ld_s(row + (2 * pr + h) * G + g));
-                        xe = PHASE ? w * u.e : scale(w, u.e.x);
+                        const cpx<T> xn = PHASE ? w * u.e : scale(w, u.e.x);
+                        (h ? acc2 : acc).add_w(mk(last ? xn.x : xe.x, last ? xn.y : xe.y), last ? (T)1 : u.w);
+                        xe = xn;
                         if (RUN && m + 1 < H) u.template step<PHASE>(qe, qw);
                     }
                 }
@@ -1309,7 +1362,7 @@ __device__ int fetch_trajectory(const Tables<T> &tb, const LaunchArgs &a)
     }
 }
 
-constexpr int fused_red = 7;   // sums reduced at once (slot_sums)
+constexpr int fused_red = 8;   // sums reduced at once (slot_sums8)
 
 // Occupancy target of a kernel variant: variant 0 asks for 512 resident threads per SM in FP32
 // (<= 128 registers); variant 1 asks for 640 (<= 102 registers, at the price of spills), variants 2 and 3
@@ -1334,7 +1387,7 @@ __global__ void __launch_bounds__(FusedPlan<T, N, V>::G, (FusedBounds<T, N, V>::
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cpx<T> *buf = reinterpret_cast<cpx<T> *>(smem_raw);
     double *red = reinterpret_cast<double *>(buf + P::BUF);         // reductions of the rare paths
-    NS2 *redh = reinterpret_cast<NS2 *>(red + RED * (G / 32 + 1));  // the step's norm
+    NS2 *redh = reinterpret_cast<NS2 *>(red + RED * (G / 32 + 1) + 8);  // the step's norm
     __shared__ int s_traj;
 
     const int g = threadIdx.x;
@@ -1365,17 +1418,11 @@ __global__ void __launch_bounds__(FusedPlan<T, N, V>::G, (FusedBounds<T, N, V>::
         int l = tb.spec_l[spec], c = tb.spec_color[spec];
         {
             const double *ic = tb.ic + (size_t)spec * N * (tb.ic_cplx ? 2 : 1);
-#pragma unroll 4
+#pragma unroll
             for (int e = 0; e < E; ++e) {
                 const int j = PW::jof(g, e);
-                T re, im = (T)0;
-                if (tb.ic_cplx) {
-                    re = (T)ic[2 * j];
-                    im = (T)ic[2 * j + 1];
-                } else {
-                    re = (T)ic[j];
-                }
-                buf[e * G + g] = PW::odd_half(e) ? mk(-re, -im) : mk(re, im);
+                const T re = tb.ic_cplx ? (T)ic[2 * j] : (T)ic[j], im = tb.ic_cplx ? (T)ic[2 * j + 1] : (T)0;
+                x[e] = PW::odd_half(e) ? mk(-re, -im) : mk(re, im);
             }
         }
         uint32_t kdraw = 0;
@@ -1403,39 +1450,35 @@ __global__ void __launch_bounds__(FusedPlan<T, N, V>::G, (FusedBounds<T, N, V>::
             return mp->kind == 1 ? table_T3_far<T>(tb.prof + 2 * (size_t)mp->tab_off, mp->tab_len, tau, &seg)
                                  : (T)mp->A / tau;
         };
-        T T3b = T3_of(0);
-        T K3b = kappa_T3<T>(mp->kfit, T3b);   // kappa_hat(T) T^3 when kappa_hat follows a lattice fit
+        T T3b = (T)0, K3b = (T)0;   // K3: kappa_hat(T) T^3 when kappa_hat follows a lattice fit
         KsuT<T> kb{};
-        if constexpr (KSU) kb = ksu_at<T>(tb, T3b);
-        if (ns > 0) {
-            if constexpr (KSU) PW::factor_ksu(buf, tb, g, l, 0, kb, kb, red);
-            else PW::factor(buf, tb, g, c, l, 0, (T)mp->erj[c] * K3b, (T)mp->eij[c] * T3b, (T)0, red);
-            PW::to_regs(x, buf, g);
-            traj_sync<G>();   // the copies are read before the first pass writes its sequences
-        }
+        bool in_smem = false;   // the state is in the shared-memory copy (else in the registers)
 
-        for (int n = 0; n < ns; ++n) {
+        // step -1 is the first half-step alone, so that the factor's code is there once
+        for (int n = ns > 0 ? -1 : 0; n < ns; ++n) {
             const T T3a = T3b, K3a = K3b;
-            const bool last = (n + 1 == ns);
+            const bool start = n < 0, last = n + 1 == ns;
             T3b = T3_of(n + 1);
             K3b = kappa_T3<T>(mp->kfit, T3b);
+            in_smem = false;
+            if (!start) {
 #pragma unroll 1
-            for (int h = 0; h < 2; ++h) {
-                K::first(x, buf, tb.TA, tb.TH, g, pb, pm);
-                traj_sync<G>();
-                K::mid(x, buf, tb.TM, tb.TI, tb.TS, g);
-                traj_sync<G>();
-                K::last(x, buf, tb.TM, g);
-                if (h == 0) {
-                    K::kinetic(x, tb.KF, g);
+                for (int h = 0; h < 2; ++h) {
+                    K::first(x, buf, tb.TA, tb.TH, g, pb, pm);
                     traj_sync<G>();
+                    K::mid(x, buf, tb.TM, tb.TI, tb.TS, g);
+                    traj_sync<G>();
+                    K::last(x, buf, tb.TM, g);
+                    if (h == 0) {
+                        K::kinetic(x, tb.KF, g);
+                        traj_sync<G>();
+                    }
                 }
             }
             executed = n + 1;
             const T erj = (T)mp->erj[c], eij = (T)mp->eij[c];
-            bool in_smem = false;   // the state is in the shared-memory copy (else in the registers)
             if constexpr (TRACED) {   // per-step summary rows
-                if (traced && ((n + 1) % a.trace_every == 0 || last) && nrec < a.trace_cap) {
+                if (!start && traced && ((n + 1) % a.trace_every == 0 || last) && nrec < a.trace_cap) {
                     traj_sync<G>();
                     PW::to_smem(x, buf, g);
                     PW::trace_row(buf, tb, g, c, l, erj * K3a, eij * T3a, red,
@@ -1443,28 +1486,36 @@ __global__ void __launch_bounds__(FusedPlan<T, N, V>::G, (FusedBounds<T, N, V>::
                     ++nrec;
                 }
             }
-            const T Tsum = last ? T3a : T3a + T3b, Ksum = last ? K3a : K3a + K3b;
-            const T cA = erj * Ksum, cB = eij * Tsum, cD = last ? (T)0 : erj * (K3a - K3b);
+            const T Tsum = last ? T3a : T3a + T3b, Ksum = last ? K3a : K3a + K3b;   // (step -1: T3a = K3a = 0)
+            const T cA = erj * Ksum, cB = eij * Tsum, cD = start || last ? (T)0 : erj * (K3a - K3b);
+            const int mode = start ? 0 : last ? 2 : 1;
             NS2 n2s;   // norm^2 / dr
             // (phases beyond 1e5: far2's reduction would lose them)
-            if (KSU || last || l >= LTAB || !(fabs(cB) * (T)N * (T)N < (T)3e4)) {
+            if (KSU || l >= LTAB || !(fabs(cB) * (T)N * (T)N < (T)3e4)) {
                 traj_sync<G>();   // all have read the transform's output
                 PW::to_smem(x, buf, g);
                 in_smem = true;
                 if constexpr (KSU) {
                     const KsuT<T> ka = kb;
                     kb = ksu_at<T>(tb, T3b);
-                    n2s = PW::factor_ksu(buf, tb, g, l, last ? 2 : 1, ka, kb, red);
+                    n2s = PW::factor_ksu(buf, tb, g, l, mode, ka, kb, red);
                 } else {
-                    n2s = PW::factor(buf, tb, g, c, l, last ? 2 : 1, cA, cB, cD, red);
+                    n2s = PW::factor(buf, tb, g, c, l, mode, cA, cB, cD, red);
                 }
             } else {
                 SqAcc<T> acc, acc2;
-                const typename Prec<T>::S *row = tb.statV2 + ((size_t)c * LTAB + l) * N;
-                if (cB == (T)0) PW::template factor_regs<false>(x, row, g, cA, cB, cD, acc, acc2);
-                else PW::template factor_regs<true>(x, row, g, cA, cB, cD, acc, acc2);
+                const typename Prec<T>::S *row = (mode == 1 ? tb.statV2 : tb.statV) + ((size_t)c * LTAB + l) * N;
+                if (cB == (T)0) PW::template factor_regs<false>(x, row, g, cA, cB, cD, last, acc, acc2);
+                else PW::template factor_regs<true>(x, row, g, cA, cB, cD, last, acc, acc2);
                 acc.merge(acc2);
                 n2s = step_norm<T, G>(acc, redh);   // synchronises: all have read the transform's output
+            }
+            if (start) {
+                if (in_smem) {
+                    PW::to_regs(x, buf, g);
+                    traj_sync<G>();   // the copies are read before the first pass writes its sequences
+                }
+                continue;
             }
             bool stop = false;
             if (!thr.finite(n2s)) {
@@ -1518,54 +1569,52 @@ __global__ void __launch_bounds__(FusedPlan<T, N, V>::G, (FusedBounds<T, N, V>::
                     }
                 }
             }
-            if (stop) {
-                if (!in_smem) PW::to_smem(x, buf, g);
-                break;
-            }
+            if (stop) break;
             if (in_smem && !last) {
                 PW::to_regs(x, buf, g);
                 traj_sync<G>();
             }
         }
 
-        // observables (FP64) from the shared-memory copy, the norm and the overlaps of the state's l in one pass:
-        // the conversions and sums run on the narrow FP64 pipe (160 of its instructions a warp at 16 values a
-        // thread and l = 0, 256 with a pass for each sum)
-        double n2, ovr[NBASIS] = {0, 0, 0, 0, 0, 0}, ovi[NBASIS] = {0, 0, 0, 0, 0, 0};
-        const int basis_l[NBASIS] = {0, 0, 1, 0, 1, 2};
-        auto observe = [&](auto nb, int s0, int s1, int s2) {
-            constexpr int NB = decltype(nb)::value;
-            const double *phi[3] = {tb.eig + (size_t)s0 * N, tb.eig + (size_t)s1 * N, tb.eig + (size_t)s2 * N};
-            double v[1 + 2 * NB];
+        // (all have read the transform's output: step_norm, or the sync before the copy)
+        if (!in_smem) PW::to_smem(x, buf, g);
+
+        // the norm and the overlaps of the state's l in one pass over the shared-memory copy, in FP64 or (FP32) in
+        // error-free parts: the sums ran on the FP64 pipe before, 160 of its instructions a warp of 16 values a thread
+        double *fin = red + 8 * (G / 32 + 1);   // norm^2 / dr, then (re, im) / dr of each overlap
+        const int nb = ended || c != 0 || l > 2 ? 0 : 3 - l;            // basis states of this l: 1S 2S 3S, 1P 2P, 1D
+        auto state_of = [&](int i) { return l == 0 ? (i == 2 ? 3 : i) : l == 1 ? 2 + 2 * i : 5; };
+        auto observe = [&](auto n) {
+            constexpr int NB = decltype(n)::value;
+            using Dot = typename std::conditional<sizeof(T) == 4, Dot2, Dot1>::type;
+            using RL = typename Prec<T>::Rl;
+            Dot norm, dot[NB > 0 ? NB : 1];
+            const RL *phi[NB > 0 ? NB : 1];
 #pragma unroll
-            for (int i = 0; i < 1 + 2 * NB; ++i) v[i] = 0.0;
+            for (int i = 0; i < NB; ++i) phi[i] = tb.eigo + (size_t)state_of(i) * N + g;
 #pragma unroll 4
             for (int e = 0; e < E; ++e) {
                 const cpx<T> u = buf[e * G + g];
-                const double re = (double)u.x, im = (double)u.y;
-                v[0] = fma(re, re, fma(im, im, v[0]));
-                const int j = PW::jof(g, e);
-                const bool neg = PW::odd_half(e);
+                if constexpr (sizeof(T) == 4) norm.add(make_float2(u.x, u.y), make_float2(u.x, u.y));
+                else norm.sq(u);
 #pragma unroll
                 for (int i = 0; i < NB; ++i) {
-                    const double f = phi[i][j], fs = neg ? -f : f;
-                    v[1 + 2 * i] = fma(fs, re, v[1 + 2 * i]);
-                    v[2 + 2 * i] = fma(fs, im, v[2 + 2 * i]);
+                    if constexpr (sizeof(T) == 4) dot[i].add(Prec<T>::ldr(phi[i] + e * G), make_float2(u.x, u.y));
+                    else dot[i].add(__ldg(phi[i] + e * G), u);
                 }
             }
-            slot_sums<G>(v, red);
-            n2 = v[0] * dr;
-            const int sel[3] = {s0, s1, s2};
+            double v[8] = {norm.x() + norm.y(), 0, 0, 0, 0, 0, 0, 0};
 #pragma unroll
             for (int i = 0; i < NB; ++i) {
-                ovr[sel[i]] = v[1 + 2 * i] * dr;
-                ovi[sel[i]] = v[2 + 2 * i] * dr;
+                v[1 + 2 * i] = dot[i].x();
+                v[2 + 2 * i] = dot[i].y();
             }
+            slot_sums8<G>(v, red, fin);
         };
-        if (ended || c != 0 || l > 2) observe(std::integral_constant<int, 0>{}, 0, 0, 0);
-        else if (l == 0) observe(std::integral_constant<int, 3>{}, 0, 1, 3);
-        else if (l == 1) observe(std::integral_constant<int, 2>{}, 2, 4, 0);
-        else observe(std::integral_constant<int, 1>{}, 5, 0, 0);
+        if (nb == 0) observe(std::integral_constant<int, 0>{});
+        else if (nb == 3) observe(std::integral_constant<int, 3>{});
+        else if (nb == 2) observe(std::integral_constant<int, 2>{});
+        else observe(std::integral_constant<int, 1>{});
         if (a.states && !grp) {
             double *st = a.states + (size_t)t * N * 2;
 #pragma unroll 4
@@ -1577,49 +1626,48 @@ __global__ void __launch_bounds__(FusedPlan<T, N, V>::G, (FusedBounds<T, N, V>::
                 st[2 * j + 1] = sg * (double)v.y;
             }
         }
-        if (g == 0) {
-            qtraj_obs o;
-            for (int s = 0; s < NBASIS; ++s) {
-                o.ov_re[s] = ovr[s];
-                o.ov_im[s] = ovi[s];
-                double sv = 0.0;
-                if (!ended && c == 0 && basis_l[s] == l) {
-                    // with jumps the estimator takes the normalised state; without (KSU) the norm lost
-                    // to V_I is the dissociation, and the overlap is taken unnormalised
-                    const double prob = (ovr[s] * ovr[s] + ovi[s] * ovi[s]) / (KSU ? 1.0 : n2);
-                    if (tb.ov0_zero[spec * NBASIS + s]) sv = prob;
-                    else {
+        // the record: a lane of the first warp per basis state, the rest by thread 0
+        if (g < 32) {
+            qtraj_obs *o = grp ? a.gobs + t : a.obs + t;
+            const double n2 = fin[0] * dr;
+            for (int s = g; s < NBASIS; s += G < 32 ? G : 32) {
+                const int sl = s == 2 || s == 4 ? 1 : s == 5 ? 2 : 0, i = s < 3 ? (s == 2 ? 0 : s) : s == 3 ? 2 : s == 4 ? 1 : 0;
+                double re = 0.0, im = 0.0, sv = 0.0;
+                if (nb > 0 && sl == l && !rmax_hit) {
+                    re = fin[1 + 2 * i] * dr;
+                    im = fin[2 + 2 * i] * dr;
+                    // with jumps the estimator takes the normalised state; without (KSU) the norm lost to V_I is
+                    // the dissociation, and the overlap is taken unnormalised
+                    sv = (re * re + im * im) / (KSU ? 1.0 : n2);
+                    if (!tb.ov0_zero[spec * NBASIS + s]) {
                         const double a0 = tb.ov0[(spec * NBASIS + s) * 2], b0 = tb.ov0[(spec * NBASIS + s) * 2 + 1];
-                        sv = prob / (a0 * a0 + b0 * b0);
+                        sv /= a0 * a0 + b0 * b0;
                     }
                 }
-                o.surv[s] = sv;
+                o->surv[s] = sv;
+                o->ov_re[s] = re;
+                o->ov_im[s] = im;
             }
-            o.norm2 = n2;
-            o.r0 = nojump ? 0.0 : draws(dp->seed, 0u).r;
-            o.l = l;
-            o.color = c;
-            o.n_jumps = nj;
-            o.n_steps_exec = executed;
-            o.flags = flags;
-            o.first_jump_step = fj;
-            o.last_jump_step = lj;
-            o.jump_digest = digest;
-            if (rmax_hit) {   // the r_max record, with the steps that found r0 >= p_NoJump
-                for (int s = 0; s < NBASIS; ++s) { o.surv[s] = 0; o.ov_re[s] = 0; o.ov_im[s] = 0; }
-                o.norm2 = 1.0;
-                o.l = tb.spec_l[spec];
-                o.color = tb.spec_color[spec];
-                o.flags = flags | QTRAJ_F_RMAX;
+            if (grp) __threadfence();         // the record before the flag that publishes it
+            __syncwarp(lane_mask<G>());
+            if (g == 0) {
+                o->norm2 = rmax_hit ? 1.0 : n2;
+                o->r0 = nojump ? 0.0 : draws(dp->seed, 0u).r;
+                // (rmax_hit: the r_max record, with the steps that found r0 >= p_NoJump)
+                o->l = rmax_hit ? tb.spec_l[spec] : l;
+                o->color = rmax_hit ? tb.spec_color[spec] : c;
+                o->n_jumps = nj;
+                o->n_steps_exec = executed;
+                o->flags = rmax_hit ? flags | QTRAJ_F_RMAX : flags;
+                o->first_jump_step = fj;
+                o->last_jump_step = lj;
+                o->jump_digest = digest;
+                if (grp) {
+                    __threadfence();
+                    atomicExch(a.gready + t, 1);
+                }
+                if (traced) a.trace_cnt[t] = nrec;
             }
-            if (grp) {
-                a.gobs[t] = o;
-                __threadfence();              // the record before the flag that publishes it
-                atomicExch(a.gready + t, 1);
-            } else {
-                a.obs[t] = o;
-            }
-            if (traced) a.trace_cnt[t] = nrec;
         }
         __syncthreads();
     }
@@ -1629,7 +1677,7 @@ __global__ void __launch_bounds__(FusedPlan<T, N, V>::G, (FusedBounds<T, N, V>::
 template <typename T, int N, int V> constexpr int fused_smem_bytes()
 {
     using P = FusedPlan<T, N, V>;
-    return P::BUF * (int)sizeof(cpx<T>) + (P::G / 32 + 1) * (fused_red + 1) * 8;
+    return P::BUF * (int)sizeof(cpx<T>) + (P::G / 32 + 1) * (fused_red + 1) * 8 + 64;
 }
 
 // Launches a trajectory kernel as one persistent wave (SMs x resident CTAs, at most max_ctas when

@@ -456,6 +456,7 @@ template <typename T> struct Tables {
     const typename Prec<T>::S *statV2; // [2][LTAB][N] the same over a full step, exp(-i (...) dt)
                                        // (both in natural order for the FP32 KSU kernel)
     const double *eig;     // [NBASIS][N] Coulomb basis, discretely normalised
+    const typename Prec<T>::Rl *eigo;   // the same in the order e G + g of the fused kernel's values, with their signs
     const double *ic;      // initial states, discretely normalised: [n_spec][N] real, or
                            // [n_spec][N][2] (re, im) when ic_cplx (after a vacuum evolution)
     const double *ov0;     // [n_spec][NBASIS][2] initial overlaps
