@@ -299,7 +299,7 @@ __global__ void find_directions(const cpx<double> *w, Prec<float>::D *out, int n
 }
 
 // The tables in the order of plan p: the transform's and the kinetic factors, and the static potential rows of a
-// half and (full) a whole step; p = nullptr: only the rows, in natural order.
+// half and (full) a whole step with the overlap basis; p = nullptr: only the rows and the basis, in natural order.
 template <typename T>
 qtraj_status build_set(const qtraj_ctx *c, qtraj_ctx::TabSet &t, const Plan *p, const double *coul, bool full,
                        const std::vector<std::pair<double, double>> &kt)
@@ -311,11 +311,11 @@ qtraj_status build_set(const qtraj_ctx *c, qtraj_ctx::TabSet &t, const Plan *p, 
     std::vector<Z> dirs;
     std::vector<PC> parts;
     std::vector<typename Prec<T>::Rl> eigo;
-    if (p && full) {   // the overlap basis in the order of the values, with the odd extension's sign
+    if (full) {   // the overlap basis in the order of the values, with the odd extension's sign
         eigo.resize((size_t)NBASIS * N);
         for (int i = 0; i < N; ++i) {
-            const int g = i % p->G, e = i / p->G, j = plan_j(g, e, p->R, p->M, p->G);
-            const double sg = e % p->R < p->R / 2 ? 1.0 : -1.0;
+            const int g = p ? i % p->G : 0, e = p ? i / p->G : 0, j = p ? plan_j(g, e, p->R, p->M, p->G) : i;
+            const double sg = !p || e % p->R < p->R / 2 ? 1.0 : -1.0;
             for (int b = 0; b < NBASIS; ++b) eigo[(size_t)b * N + i] = Prec<T>::make_r(sg * c->basis_host[(size_t)b * N + j]);
         }
     }
@@ -355,8 +355,8 @@ qtraj_status build_set(const qtraj_ctx *c, qtraj_ctx::TabSet &t, const Plan *p, 
     const size_t n = (size_t)2 * LTAB * N;
     if (cudaMalloc(&t.statV, sizeof(PS) * n) != cudaSuccess || (full && cudaMalloc(&t.statV2, sizeof(PS) * n) != cudaSuccess) ||
         (p && (cudaMalloc(&t.dirs, sizeof(typename Prec<T>::D) * dirs.size()) != cudaSuccess ||
-               cudaMalloc(&t.parts, sizeof(PC) * parts.size()) != cudaSuccess ||
-               (full && cudaMalloc(&t.eigo, sizeof(eigo[0]) * eigo.size()) != cudaSuccess)))) {
+               cudaMalloc(&t.parts, sizeof(PC) * parts.size()) != cudaSuccess)) ||
+        (full && cudaMalloc(&t.eigo, sizeof(eigo[0]) * eigo.size()) != cudaSuccess)) {
         cudaGetLastError();
         return fail(QTRAJ_ENOMEM, "cudaMalloc of the tables (%zu bytes)", (full ? 2 : 1) * sizeof(PS) * n);
     }
@@ -370,11 +370,11 @@ qtraj_status build_set(const qtraj_ctx *c, qtraj_ctx::TabSet &t, const Plan *p, 
         void *w = sizeof(T) == 8 ? t.dirs : t.statV;
         e = cudaMemcpyAsync(w, dirs.data(), sizeof(Z) * dirs.size(), cudaMemcpyHostToDevice, s);
         if (e == cudaSuccess) e = cudaMemcpyAsync(t.parts, parts.data(), sizeof(PC) * parts.size(), cudaMemcpyHostToDevice, s);
-        if (e == cudaSuccess && full)
-            e = cudaMemcpyAsync(t.eigo, eigo.data(), sizeof(eigo[0]) * eigo.size(), cudaMemcpyHostToDevice, s);
         if (sizeof(T) == 4)
             find_directions<<<((int)dirs.size() + 7) / 8, 256, 0, s>>>((const Z *)w, (Prec<float>::D *)t.dirs, (int)dirs.size());
     }
+    if (e == cudaSuccess && full)
+        e = cudaMemcpyAsync(t.eigo, eigo.data(), sizeof(eigo[0]) * eigo.size(), cudaMemcpyHostToDevice, s);
     const int blocks = (int)std::min<size_t>((n + 255) / 256, 4096);
     for (int h = 0; h < (full ? 2 : 1); ++h)
         stat_rows<T><<<blocks, 256, 0, s>>>((PS *)(h ? t.statV2 : t.statV), N, c->dr, c->M, c->dt, coul[0], coul[1],

@@ -40,6 +40,11 @@ template <int N> struct NftPlan {
     static constexpr int TW1 = R * M1;
     static constexpr int TW2 = M2 > 1 ? R * M1 * M2 : 0;
     static_assert(N == R * M1 * M2 * R, "plan");
+    // shared memory without the cached potential: state, twiddles, carries and reductions
+    static constexpr int SMEM = BUF * 8 + (TW1 + TW2) * 16 + (G / 32 + 1) * (16 + 64) + 64;
+    static constexpr int MIN_BLOCKS = 512 / G > 32 ? 32 : (512 / G > 0 ? 512 / G : 1);   // 512 threads per SM
+    // the potential at T_{n+1} is cached where that costs no resident CTA (N <= 2048)
+    static constexpr bool CACHE = (SMEM + N * 8) * MIN_BLOCKS <= 220 * 1024;
 };
 
 
@@ -304,13 +309,15 @@ template <int N> struct NftPointwise {
     // The dynamic exponent of the half-step at temperature T is (V_I - i (V_R + a/r)) dt/2 at each point, evaluated
     // per point and applied as w + w f1 (fused.cuh); ka, kb are the per-step scalars of T_n (the closing half-step)
     // and T_{n+1} (the opening one).
+    // CACHE: the potential at T_{n+1} is kept in shared memory (vc, thread-private places) for the next step's T_n.
+    template <bool CACHE>
     static __device__ typename NormSum<T>::type factor_ksu(cpx<T> *buf, const Tables<T> &tb, int g, int l, int mode,
-                                                           const KsuT<T> &ka, const KsuT<T> &kb, double *red)
+                                                           const KsuT<T> &ka, const KsuT<T> &kb, float2 *vc, double *red)
     {
         SqAcc<T> acc, acc_odd;
         const SC *tab = (mode == 1) ? tb.statV2 : tb.statV;
         const T hdt = (T)0.5 * tb.ksu_dt;
-#pragma unroll 1
+#pragma unroll 2
         for (int k = g; k < N / 2; k += G) {
 #pragma unroll
             for (int par = 0; par < 2; ++par) {
@@ -320,8 +327,20 @@ template <int N> struct NftPointwise {
                 T A = (T)0, t = (T)0;
                 if (j > 0) {
                     T vda = (T)0, via = (T)0, vdb = (T)0, vib = (T)0;
-                    if (mode != 0) ksu_point<T>(tb, ka, fj, vda, via);
-                    if (mode != 2) ksu_point<T>(tb, kb, fj, vdb, vib);
+                    if constexpr (CACHE) {
+                        float2 *q = vc + par * (N / 2) + k;
+                        if (mode != 0) {
+                            vda = q->x;
+                            via = q->y;
+                        }
+                        if (mode != 2) {
+                            ksu_point<T>(tb, kb, fj, vdb, vib);
+                            *q = make_float2(vdb, vib);
+                        }
+                    } else {
+                        if (mode != 0) ksu_point<T>(tb, ka, fj, vda, via);
+                        if (mode != 2) ksu_point<T>(tb, kb, fj, vdb, vib);
+                    }
                     A = (via + vib) * hdt;
                     t = -(vda + vdb) * hdt;
                 }
@@ -342,13 +361,8 @@ template <int N> struct NftPointwise {
     }
 };
 
-template <int N> struct KsuBounds {
-    static constexpr int G = NftPlan<N>::G;
-    static constexpr int MIN_BLOCKS = 512 / G > 32 ? 32 : (512 / G > 0 ? 512 / G : 1);   // 512 threads per SM
-};
-
 template <int N>
-__global__ void __launch_bounds__(NftPlan<N>::G, (KsuBounds<N>::MIN_BLOCKS)) ksu32_kernel(Tables<float> tb, LaunchArgs a)
+__global__ void __launch_bounds__(NftPlan<N>::G, (NftPlan<N>::MIN_BLOCKS)) ksu32_kernel(Tables<float> tb, LaunchArgs a)
 {
     using T = float;
     using K = NftSine<N>;
@@ -361,7 +375,8 @@ __global__ void __launch_bounds__(NftPlan<N>::G, (KsuBounds<N>::MIN_BLOCKS)) ksu
     C *tw1 = reinterpret_cast<C *>(buf + P::BUF);
     C *tw2 = tw1 + P::TW1;
     Carry *wtot = reinterpret_cast<Carry *>(tw2 + P::TW2);
-    double *red = reinterpret_cast<double *>(wtot + (G / 32 + 1));
+    double *red = reinterpret_cast<double *>(wtot + (G / 32 + 1)), *fin = red + 8 * (G / 32 + 1);
+    float2 *vc = reinterpret_cast<float2 *>(fin + 8);
     __shared__ int s_traj;
     // middle-pass twiddles, row m of a table holding W^(m k) for every k (tw1: [M1][R] of W_{R M1},
     // tw2: [M2][R M1] of W_{R M1 M2}, the second only with a second middle pass), built once per CTA
@@ -403,7 +418,7 @@ __global__ void __launch_bounds__(NftPlan<N>::G, (KsuBounds<N>::MIN_BLOCKS)) ksu
         KsuT<T> kb = ksu_at<T>(tb, T3b);
         if (ns > 0) {
             __syncthreads();
-            PW::factor_ksu(buf, tb, g, l, 0, kb, kb, red);
+            PW::template factor_ksu<P::CACHE>(buf, tb, g, l, 0, kb, kb, vc, red);
         }
         for (int n = 0; n < ns; ++n) {
             const bool last = (n + 1 == ns);
@@ -414,7 +429,7 @@ __global__ void __launch_bounds__(NftPlan<N>::G, (KsuBounds<N>::MIN_BLOCKS)) ksu
             executed = n + 1;
             const KsuT<T> ka = kb;
             kb = ksu_at<T>(tb, T3b);
-            const typename NormSum<T>::type n2s = PW::factor_ksu(buf, tb, g, l, last ? 2 : 1, ka, kb, red);
+            const typename NormSum<T>::type n2s = PW::template factor_ksu<P::CACHE>(buf, tb, g, l, last ? 2 : 1, ka, kb, vc, red);
             if (!thr.finite(n2s)) {
                 flags |= QTRAJ_F_NONFINITE;
                 ended = 1;
@@ -424,31 +439,27 @@ __global__ void __launch_bounds__(NftPlan<N>::G, (KsuBounds<N>::MIN_BLOCKS)) ksu
         }
         __syncthreads();
 
-        // observables (FP64); without jumps the norm lost to V_I is the dissociation, and the overlap is
-        // taken unnormalised
-        double acc = 0.0;
-        for (int k = g; k < N / 2; k += G) {
-            const cpx<T> a0 = buf[K::even_pos(k)], a1 = buf[K::odd_pos(k)];
-            acc += (double)a0.x * a0.x + (double)a0.y * a0.y + (double)a1.x * a1.x + (double)a1.y * a1.y;
-        }
-        const double n2 = slot_sum<G>(acc, red) * dr;
-        double ovr[NBASIS], ovi[NBASIS];
-        const int basis_l[NBASIS] = {0, 0, 1, 0, 1, 2};
-#pragma unroll
-        for (int s = 0; s < NBASIS; ++s) {
-            ovr[s] = 0.0;
-            ovi[s] = 0.0;
-            if (ended || basis_l[s] != l) continue;
-            const double *phi = tb.eig + (size_t)s * N;
-            double pr = 0.0, pi = 0.0;
+        // the norm and the overlaps as fused.cuh's read-out; without jumps the norm lost to V_I is the dissociation, and
+        // the overlap is taken unnormalised
+        const int nb = ended || l > 2 ? 0 : 3 - l;
+        auto state_of = [&](int i) { return l == 0 ? (i == 2 ? 3 : i) : l == 1 ? 2 + 2 * i : 5; };
+        {
+            Dot2 norm, dot[3];
             for (int k = g; k < N / 2; k += G) {
                 const cpx<T> a0 = buf[K::even_pos(k)], a1 = buf[K::odd_pos(k)];
-                const double f0 = phi[2 * k], f1 = phi[2 * k + 1];
-                pr += f0 * (double)a0.x + f1 * (double)a1.x;
-                pi += f0 * (double)a0.y + f1 * (double)a1.y;
+                const float2 u0 = make_float2(a0.x, a0.y), u1 = make_float2(a1.x, a1.y);
+                norm.add(u0, u0);
+                norm.add(u1, u1);
+#pragma unroll
+                for (int i = 0; i < 3; ++i)
+                    if (i < nb) {
+                        const float4 f = __ldg(reinterpret_cast<const float4 *>(tb.eigo + (size_t)state_of(i) * N) + k);
+                        dot[i].add(Prec<float>::Rl{f.x, f.y}, u0);
+                        dot[i].add(Prec<float>::Rl{f.z, f.w}, u1);
+                    }
             }
-            ovr[s] = slot_sum<G>(pr, red) * dr;
-            ovi[s] = slot_sum<G>(pi, red) * dr;
+            double v[8] = {norm.x() + norm.y(), dot[0].x(), dot[0].y(), dot[1].x(), dot[1].y(), dot[2].x(), dot[2].y(), 0};
+            slot_sums8<G>(v, red, fin);
         }
         if (a.states) {
             double *st = a.states + (size_t)t * N * 2;
@@ -460,34 +471,36 @@ __global__ void __launch_bounds__(NftPlan<N>::G, (KsuBounds<N>::MIN_BLOCKS)) ksu
                 st[4 * k + 3] = (double)a1.y;
             }
         }
-        if (g == 0) {
-            qtraj_obs o;
-            const int sp = d.spec;
-            for (int s = 0; s < NBASIS; ++s) {
-                o.ov_re[s] = ovr[s];
-                o.ov_im[s] = ovi[s];
-                double sv = 0.0;
-                if (!ended && basis_l[s] == l) {
-                    const double prob = ovr[s] * ovr[s] + ovi[s] * ovi[s];
-                    if (tb.ov0_zero[sp * NBASIS + s]) sv = prob;
-                    else {
-                        const double a0 = tb.ov0[(sp * NBASIS + s) * 2], b0 = tb.ov0[(sp * NBASIS + s) * 2 + 1];
-                        sv = prob / (a0 * a0 + b0 * b0);
+        if (g < 32) {
+            qtraj_obs *o = a.obs + t;
+            for (int q = g; q < NBASIS; q += G < 32 ? G : 32) {
+                const int ql = q == 2 || q == 4 ? 1 : q == 5 ? 2 : 0, i = q < 3 ? (q == 2 ? 0 : q) : q == 3 ? 2 : q == 4 ? 1 : 0;
+                double re = 0.0, im = 0.0, sv = 0.0;
+                if (nb > 0 && ql == l) {
+                    re = fin[1 + 2 * i] * dr;
+                    im = fin[2 + 2 * i] * dr;
+                    sv = re * re + im * im;
+                    if (!tb.ov0_zero[d.spec * NBASIS + q]) {
+                        const double a0 = tb.ov0[(d.spec * NBASIS + q) * 2], b0 = tb.ov0[(d.spec * NBASIS + q) * 2 + 1];
+                        sv /= a0 * a0 + b0 * b0;
                     }
                 }
-                o.surv[s] = sv;
+                o->surv[q] = sv;
+                o->ov_re[q] = re;
+                o->ov_im[q] = im;
             }
-            o.norm2 = n2;
-            o.r0 = 0.0;
-            o.l = l;
-            o.color = 0;
-            o.n_jumps = 0;
-            o.n_steps_exec = executed;
-            o.flags = flags;
-            o.first_jump_step = -1;
-            o.last_jump_step = -1;
-            o.jump_digest = DIGEST_BASIS;
-            a.obs[t] = o;
+            if (g == 0) {
+                o->norm2 = fin[0] * dr;
+                o->r0 = 0.0;
+                o->l = l;
+                o->color = 0;
+                o->n_jumps = 0;
+                o->n_steps_exec = executed;
+                o->flags = flags;
+                o->first_jump_step = -1;
+                o->last_jump_step = -1;
+                o->jump_digest = DIGEST_BASIS;
+            }
         }
         __syncthreads();
     }
@@ -499,8 +512,7 @@ cudaError_t ksu32_go(const Tables<float> &tb, const LaunchArgs &a, int sm_count,
                      FusedInfo *info, bool query_only)
 {
     using P = NftPlan<N>;
-    constexpr int smem = P::BUF * (int)sizeof(cpx<float>) + (P::TW1 + P::TW2) * (int)sizeof(typename Prec<float>::C) +
-                         (P::G / 32 + 1) * (int)sizeof(Carry) + (P::G / 32 + 1) * 8 + 16;
+    constexpr int smem = P::SMEM + (P::CACHE ? N * 8 : 0);
     return launch_wave(ksu32_kernel<N>, P::G, P::R, smem, tb, a, sm_count, max_ctas, s, info, query_only);
 }
 
