@@ -1529,7 +1529,7 @@ extern "C" qtraj_status qtraj_evolve_static(qtraj_ctx *c, int batch, const qtraj
     ma.gtrajs = ds->gtrajs;
     ma.n_groups = n_groups;
     ma.gobs = ds->gobs;
-    ma.gready = ds->gready;
+    ma.gready = n_groups > 0 ? ds->gready : nullptr;   // (without groups the flags are an earlier call's)
     FusedInfo fi;
     auto point = [&](auto tb) {
         tb.ic = ds->ic;

@@ -100,3 +100,31 @@ def test_fp32_large_phases_conserve_the_norm(q, gamma):  # noqa: F811
     e.close()
     assert (o["n_steps_exec"] > 10).all()
     assert (np.abs(o["norm2"] - 1) <= fp32_bound(64, o["n_steps_exec"])).all(), o["norm2"]
+
+
+def test_static_entry_takes_no_flags_of_an_earlier_call(q):  # noqa: F811
+    """A KSU call of qtraj_evolve_static (no groups, use_rmin on by default) after an OQS call whose groups published
+    their no-jump records in the shared scratch: the records are the KSU evolution's, as through a workspace."""
+    import ctypes as C
+    import torch
+    spec, med = q.init_spec("gauss", 0.8, 1, 0, 0), q.medium(0.425, 0.6, 0.4, 0.5, 0.0)
+    seeds = np.arange(4, dtype=np.uint64)
+
+    def static(e):
+        out = torch.zeros(4 * q.OBS_DTYPE.itemsize, dtype=torch.uint8, device="cuda")
+        st = e.lib.qtraj_evolve_static(e.ctx, 4, (q.InitSpec * 1)(spec), 1, None, (q.Medium * 1)(med), 1, None,
+                                       seeds.ctypes.data_as(C.POINTER(C.c_uint64)), C.c_void_p(out.data_ptr()),
+                                       C.c_void_p(torch.cuda.current_stream().cuda_stream))
+        assert st == 0, e.lib.qtraj_last_error(e.ctx)
+        return out.cpu().numpy().view(q.OBS_DTYPE)
+
+    oqs = q.Engine(q.Config(N=64, L=5.0, dt=0.001, precision=q.FP64))
+    static(oqs)
+    ksu = q.Engine(q.Config(N=64, L=5.0, dt=0.001, precision=q.FP64, potential=1))
+    a = static(ksu)
+    ksu.init([spec], 4)
+    ksu.evolve([med], seeds)
+    b = ksu.observables()
+    assert (a["n_steps_exec"] > 0).all() and np.array_equal(a["norm2"], b["norm2"]) and np.array_equal(a["surv"], b["surv"])
+    oqs.close()
+    ksu.close()
