@@ -42,10 +42,11 @@ UNIT = "traj-steps/s"
 N_GRID, L_BOX, DT = 4096, 40.0, 0.001
 # DRAM traffic of fused_kernel<float, 4096, 0> from two ncu captures of the current kernel source
 # (608 trajectories through 300 and through 1000 steps; dram__bytes_read.sum + dram__bytes_write.sum):
-# a launch costs a fixed part (the first touch of the tables) plus a part per trajectory-step (the
-# per-step tables that fall out of L2).  None until the kernel has been captured again after a change.
-PROFILED_DRAM_FIXED_BYTES = 1.107e6
-PROFILED_DRAM_BYTES_PER_TRAJ_STEP = 2.63
+# 1.389 MB and 0.809 MB, and 0.847 MB for 9216 trajectories through 16 steps, so a launch costs the first
+# touch of the tables, and a part per trajectory-step is not resolved: the tables stay in L2.  None until
+# the kernel has been captured again after a change.
+PROFILED_DRAM_FIXED_BYTES = 1.389e6
+PROFILED_DRAM_BYTES_PER_TRAJ_STEP = 0.0
 N_STEPS_FULL = 11899          # ceil((tau_f - tau0) / (hbar c dt)) for the Bjorken medium 0.425 -> 0.25 GeV at tau0 = 0.6 fm/c
 
 
@@ -116,9 +117,10 @@ def fp32_peak_tflops(sm_count, mhz=2070.0):
 
 
 def algorithmic_flops_per_step(N):
-    """FP32 flops of one trajectory-step of the method as implemented: two sine transforms, each an
-    N-point complex FFT (5 N log2 N) plus pre/post-processing and the odd-coefficient prefix sum
-    (12 N), the kinetic factor (6 N), two space half-steps (12 N each) and the norm (4 N)."""
+    """FP32 flops of one trajectory-step by the cheapest usual method: two sine transforms, each through
+    an N-point complex FFT (5 N log2 N) with pre/post-processing and an odd-coefficient prefix sum
+    (12 N), the kinetic factor (6 N), two space half-steps (12 N each) and the norm (4 N).  (The kernels
+    take the independent half of a 2N-point FFT of the odd extension, which is as many operations.)"""
     lg = int(np.log2(N))
     return 2 * (5 * N * lg + 12 * N) + 6 * N + 2 * 12 * N + 4 * N
 

@@ -40,7 +40,8 @@ typedef enum {
     QTRAJ_EBUSY = 6       /* the context has queued work that this call would overwrite */
 } qtraj_status;
 
-/* arithmetic of the step: the norm, the waiting-time comparison and the overlaps are FP64 in all */
+/* arithmetic of the step.  FP32: the waiting-time comparison is in double-float, the final norm and the overlaps are
+ * sums of FP32 products in error-free parts (2^-46 of the terms), reported as FP64 */
 typedef enum { QTRAJ_FP64 = 0, QTRAJ_FP32 = 1 } qtraj_precision;
 
 /* QTRAJ_FUSED: one persistent kernel; every trajectory stays in shared memory/registers for its
@@ -62,8 +63,8 @@ typedef struct {
     int form;        /* qtraj_form */
     int save_states; /* 1: keep every final u(r) (FP64) in the workspace for qtraj_states()     */
     int variant;     /* fused kernel variant (FP32, N in {2048, 4096}; elsewhere the same as 0):
-                        0 = radix 16, 512 resident threads per SM (384 at N = 4096); 1 = radix 16,
-                        640; 2 = radix 8, 768; 3 = radix 8, 1024                                   */
+                        0 = radix 16, 512 resident threads per SM; 1 = radix 16, 640; 2 = radix 8, 768;
+                        3 = radix 8, 1024                                                          */
     double t_vacuum; /* >= 0, GeV^-1: vacuum evolution of every initial state before the medium
                         (Table 1: tmed - t0; Sec. 3.5 item 3): round(t_vacuum / dt) Strang steps
                         at T = 0 (Coulomb + centrifugal potential of the state's colour, no
@@ -259,8 +260,8 @@ qtraj_status qtraj_kernel_info_get(const qtraj_ctx *ctx, qtraj_kernel_info *out)
 /* Measurement of the radix-16 DFT blocks of the sine transforms (Sec. 3.3; the paper's transforms
  * are FFTW calls and have no tensor-core form): one CTA per batch of 256 columns of 16 complex FP32
  * points, resident in shared memory, applies `passes` times y = (F/4) x to every column, F the
- * 16-point DFT matrix exp(-2 pi i m'm/16) ((F/4)^4 = I).  method 0: CUDA cores (the fused kernel's
- * DFT16, constants in hi+lo, then times 1/4).  Tensor cores, mma.sync -> FP32 with the matrix in PA
+ * 16-point DFT matrix exp(-2 pi i m'm/16) ((F/4)^4 = I).  method 0: CUDA cores (radix 4 x 4 as in
+ * the kernels, constants in hi+lo, then times 1/4).  Tensor cores, mma.sync -> FP32 with the matrix in PA
  * parts, each value in PB parts and the products of part orders j + k <= MAXORD: 1 BF16X3 (BF16,
  * PA = PB = 2, 3 products); 2 BF16X9 (BF16, PA = 4, PB = 3, 9 products); 3 FP16X3 (FP16, PA = PB = 2,
  * 3 products); 4 FP16X5 (FP16, PA = 3, PB = 2, 5 products); the FP16 forms scale each column by a

@@ -1,7 +1,7 @@
 """In-project autotuner for the fused kernel's launch variant.
 
 For a grid size N and precision, every variant the library offers (512 or 640 resident threads
-per SM at the size's own radix -- 8 up to N = 2048, 16 above -- and radix 8 with 768 or 1024) is
+per SM at the size's own plan, radix 16 at N = 2048 and 4096, and radix 8 with 768 or 1024) is
 timed on one full wave of trajectories of
 the benchmark medium through its first `steps` steps, and the fastest is recorded, with all measured
 rates and the kernel geometry, in a JSON cache (`_lib/autotune.json` in the package, or the path in

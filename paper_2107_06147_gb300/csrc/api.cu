@@ -1,6 +1,6 @@
 // api.cu -- the C ABI of libqtraj (include/qtraj.h): context, read-only tables, workspace layout,
-// and the orchestration of an evolve (no-jump runs of every (initial state, medium) group first,
-// then all trajectories).  All host-side tables are built in FP64.
+// and the orchestration of an evolve (fused form: one launch, whose first work items are the no-jump runs of
+// the (initial state, medium) groups; plain form: those runs first).  All host-side tables are built in FP64.
 #include <algorithm>
 #include <cmath>
 #include <cstdarg>

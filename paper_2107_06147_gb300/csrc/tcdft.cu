@@ -6,7 +6,7 @@
 // matrix exp(-2 pi i m'm/16).  F/4 is a quarter of a unitary matrix times 4, so |y| = |x| and four
 // passes give x back exactly in exact arithmetic.
 //
-//   method 0  CUDA cores: the fused kernel's DFT16 (radix 4 x 4, constants in hi+lo), then x 1/4;
+//   method 0  CUDA cores: a DFT16 as in the kernels (radix 4 x 4, constants in hi+lo), then x 1/4;
 //             one column per thread.
 //   tensor-core forms: mma.sync m16n8k16 -> FP32 on the real form [Re -Im; Im Re] of F/4.  The matrix
 //   is split into PA parts and the data into PB parts of the operand type, and the products A_j B_k
