@@ -310,6 +310,10 @@ template <int N> struct NftPointwise {
     // per point and applied as w + w f1 (fused.cuh); ka, kb are the per-step scalars of T_n (the closing half-step)
     // and T_{n+1} (the opening one).
     // CACHE: the potential at T_{n+1} is kept in shared memory (vc, thread-private places) for the next step's T_n.
+    // (Of the even points alone it fits at N = 4096 too, but the L1 that this takes made the step 20% slower.)
+    // The loop is not unrolled: with two pairs of points in flight the code outgrows the instruction cache once the CTAs
+    // have drifted apart (N = 4096 through 2404 steps: 1.15e7 trajectory-steps/s unrolled, 1.25e7 not; 1.21e7 before the
+    // norm's weight was left out; N = 1024: 5.95e7, 6.54e7, 4.87e7).
     template <bool CACHE>
     static __device__ typename NormSum<T>::type factor_ksu(cpx<T> *buf, const Tables<T> &tb, int g, int l, int mode,
                                                            const KsuT<T> &ka, const KsuT<T> &kb, float2 *vc, double *red)
@@ -317,7 +321,7 @@ template <int N> struct NftPointwise {
         SqAcc<T> acc, acc_odd;
         const SC *tab = (mode == 1) ? tb.statV2 : tb.statV;
         const T hdt = (T)0.5 * tb.ksu_dt;
-#pragma unroll 2
+#pragma unroll 1
         for (int k = g; k < N / 2; k += G) {
 #pragma unroll
             for (int par = 0; par < 2; ++par) {
