@@ -107,7 +107,7 @@ struct qtraj_ctx {
         void *dirs = nullptr, *parts = nullptr;                           // KF | TA | TM | TI and TH | TS
         size_t ta = 0, tm = 0, ti = 0, ts = 0;                            // where these begin
         void *statV = nullptr, *statV2 = nullptr, *eigo = nullptr;
-        void **all[5] = {&dirs, &parts, &statV, &statV2, &eigo};
+        void *base = nullptr;                                             // the allocation that holds them all
     } fused, plain;
     double *eig = nullptr;
     double *ic = nullptr, *ov0 = nullptr;
@@ -250,6 +250,17 @@ __global__ void stat_rows(typename Prec<T>::S *out, int N, double dr, double M, 
     }
 }
 
+// the overlap basis in the order of the values, with the odd extension's sign (R = 0: natural order)
+template <typename T>
+__global__ void basis_rows(typename Prec<T>::Rl *out, const double *eig, int N, int R, int PM, int G)
+{
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x) {
+        const int e = i / G, j = R > 0 ? plan_j(i % G, e, R, PM, G) : i;
+        const double sg = R == 0 || e % R < R / 2 ? 1.0 : -1.0;
+        for (int b = 0; b < NBASIS; ++b) out[(size_t)b * N + i] = Prec<T>::make_r(sg * eig[(size_t)b * N + j]);
+    }
+}
+
 // host array -> new device array
 template <typename V> qtraj_status upload(void **out, const std::vector<V> &v)
 {
@@ -300,25 +311,20 @@ __global__ void find_directions(const cpx<double> *w, Prec<float>::D *out, int n
 
 // The tables in the order of plan p: the transform's and the kinetic factors, and the static potential rows of a
 // half and (full) a whole step with the overlap basis; p = nullptr: only the rows and the basis, in natural order.
+// One allocation, and the basis reordered on the device from its copy there (uploaded on stream s before): five
+// allocations and a host loop over the basis made a context 10% slower to build.
 template <typename T>
 qtraj_status build_set(const qtraj_ctx *c, qtraj_ctx::TabSet &t, const Plan *p, const double *coul, bool full,
-                       const std::vector<std::pair<double, double>> &kt)
+                       const std::vector<std::pair<double, double>> &kt, cudaStream_t s)
 {
     using PC = typename Prec<T>::C;
+    using PD = typename Prec<T>::D;
     using PS = typename Prec<T>::S;
+    using PR = typename Prec<T>::Rl;
     using Z = cpx<double>;
     const int N = c->N;
     std::vector<Z> dirs;
     std::vector<PC> parts;
-    std::vector<typename Prec<T>::Rl> eigo;
-    if (full) {   // the overlap basis in the order of the values, with the odd extension's sign
-        eigo.resize((size_t)NBASIS * N);
-        for (int i = 0; i < N; ++i) {
-            const int g = p ? i % p->G : 0, e = p ? i / p->G : 0, j = p ? plan_j(g, e, p->R, p->M, p->G) : i;
-            const double sg = !p || e % p->R < p->R / 2 ? 1.0 : -1.0;
-            for (int b = 0; b < NBASIS; ++b) eigo[(size_t)b * N + i] = Prec<T>::make_r(sg * c->basis_host[(size_t)b * N + j]);
-        }
-    }
     if (p) {
         auto root = [&](long k, long n) {   // exp(-2 pi i k / n)
             const double a = -2.0 * PI * (double)(k % n) / (double)n;
@@ -353,16 +359,24 @@ qtraj_status build_set(const qtraj_ctx *c, qtraj_ctx::TabSet &t, const Plan *p, 
         for (int k = 1; k < H; ++k) parts[t.ts + k] = Prec<T>::make(0.5 / std::sin(PI * k / p->R), 0.5 / std::tan(PI * k / p->R));
     }
     const size_t n = (size_t)2 * LTAB * N;
-    if (cudaMalloc(&t.statV, sizeof(PS) * n) != cudaSuccess || (full && cudaMalloc(&t.statV2, sizeof(PS) * n) != cudaSuccess) ||
-        (p && (cudaMalloc(&t.dirs, sizeof(typename Prec<T>::D) * dirs.size()) != cudaSuccess ||
-               cudaMalloc(&t.parts, sizeof(PC) * parts.size()) != cudaSuccess)) ||
-        (full && cudaMalloc(&t.eigo, sizeof(eigo[0]) * eigo.size()) != cudaSuccess)) {
+    size_t o = 0;
+    auto part = [&](size_t bytes) {
+        const size_t at = o;
+        o = align256(o + bytes);
+        return at;
+    };
+    const size_t o_s1 = part(sizeof(PS) * n), o_s2 = part(full ? sizeof(PS) * n : 0), o_d = part(sizeof(PD) * dirs.size()),
+                 o_p = part(sizeof(PC) * parts.size()), o_e = part(full ? sizeof(PR) * NBASIS * (size_t)N : 0);
+    if (cudaMalloc(&t.base, o) != cudaSuccess) {
         cudaGetLastError();
-        return fail(QTRAJ_ENOMEM, "cudaMalloc of the tables (%zu bytes)", (full ? 2 : 1) * sizeof(PS) * n);
+        return fail(QTRAJ_ENOMEM, "cudaMalloc of the tables (%zu bytes)", o);
     }
-    // a private non-blocking stream: building a context waits for nothing else on the device
-    cudaStream_t s = nullptr;
-    CK(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
+    char *base = (char *)t.base;
+    t.statV = base + o_s1;
+    if (full) t.statV2 = base + o_s2;
+    if (p) t.dirs = base + o_d;
+    if (p) t.parts = base + o_p;
+    if (full) t.eigo = base + o_e;
     cudaError_t e = cudaSuccess;
     if (p) {
         // (the constants in 64 bits pass through the memory of the rows, which are filled after them)
@@ -373,21 +387,20 @@ qtraj_status build_set(const qtraj_ctx *c, qtraj_ctx::TabSet &t, const Plan *p, 
         if (sizeof(T) == 4)
             find_directions<<<((int)dirs.size() + 7) / 8, 256, 0, s>>>((const Z *)w, (Prec<float>::D *)t.dirs, (int)dirs.size());
     }
-    if (e == cudaSuccess && full)
-        e = cudaMemcpyAsync(t.eigo, eigo.data(), sizeof(eigo[0]) * eigo.size(), cudaMemcpyHostToDevice, s);
+    if (full)
+        basis_rows<T><<<(N + 255) / 256, 256, 0, s>>>((PR *)t.eigo, c->eig, N, p ? p->R : 0, p ? p->M : 0, p ? p->G : 1);
     const int blocks = (int)std::min<size_t>((n + 255) / 256, 4096);
     for (int h = 0; h < (full ? 2 : 1); ++h)
         stat_rows<T><<<blocks, 256, 0, s>>>((PS *)(h ? t.statV2 : t.statV), N, c->dr, c->M, c->dt, coul[0], coul[1],
                                             h ? 2.0 : 1.0, p ? p->R : 0, p ? p->M : 0, p ? p->G : 1);
     if (e == cudaSuccess) e = cudaGetLastError();
-    const cudaError_t e2 = cudaStreamSynchronize(s);
+    const cudaError_t e2 = cudaStreamSynchronize(s);   // (the host arrays end here)
     if (e == cudaSuccess) e = e2;
-    cudaStreamDestroy(s);
     CK(e);
     return QTRAJ_OK;
 }
 
-template <typename T> qtraj_status build_tables(qtraj_ctx *c)
+template <typename T> qtraj_status build_tables(qtraj_ctx *c, cudaStream_t s)
 {
     using PC = typename Prec<T>::C;
     using PR = typename Prec<T>::Rl;
@@ -487,15 +500,15 @@ template <typename T> qtraj_status build_tables(qtraj_ctx *c)
         if ((st = upload(&c->W, W)) != QTRAJ_OK || (st = upload(&c->KT, KT)) != QTRAJ_OK ||
             (st = upload(&c->sinpre, sp)) != QTRAJ_OK || (st = upload(&c->WL, WL)) != QTRAJ_OK)
             return st;
-        return build_set<T>(c, c->fused, nullptr, coul, true, kt);
+        return build_set<T>(c, c->fused, nullptr, coul, true, kt, s);
     }
     // a plain context runs the fused kernel only for the vacuum evolution of its initial states
     const int variant = c->p.potential == 1 ? 0 : c->p.variant;
     const Plan pf = make_plan(N, sizeof(T) == 8, variant >= 2 ? PLAN_RAD8 : PLAN_FUSED), pp = make_plan(N, true, PLAN_PLAIN);
     qtraj_status st = QTRAJ_OK;
     if (c->p.form != QTRAJ_PLAIN || c->p.t_vacuum > 0)
-        if ((st = build_set<T>(c, c->fused, &pf, coul, true, kt)) != QTRAJ_OK) return st;
-    if (c->p.form == QTRAJ_PLAIN) st = build_set<T>(c, c->plain, &pp, coul, false, kt);
+        if ((st = build_set<T>(c, c->fused, &pf, coul, true, kt, s)) != QTRAJ_OK) return st;
+    if (c->p.form == QTRAJ_PLAIN) st = build_set<T>(c, c->plain, &pp, coul, false, kt, s);
     return st;
 }
 
@@ -838,12 +851,18 @@ qtraj_status qtraj_create(int N, double L, double dt, double M, const qtraj_para
     if (cudaGetDevice(&c->device) != cudaSuccess) return bail(fail(QTRAJ_ECUDA, "no CUDA device"));
     if (cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess)
         return bail(fail(QTRAJ_ECUDA, "cannot query the SM count"));
-    st = p.precision == QTRAJ_FP32 ? build_tables<float>(c) : build_tables<double>(c);
+    const size_t b_eig = sizeof(double) * c->basis_host.size();
+    if (cudaMalloc(&c->eig, b_eig) != cudaSuccess) return bail(fail(QTRAJ_ENOMEM, "cudaMalloc"));
+    // a private non-blocking stream: building a context waits for nothing else on the device
+    cudaStream_t s = nullptr;
+    if (cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) != cudaSuccess)
+        return bail(fail(QTRAJ_ECUDA, "cudaStreamCreate failed"));
+    const cudaError_t up = cudaMemcpyAsync(c->eig, c->basis_host.data(), b_eig, cudaMemcpyHostToDevice, s);
+    if (up != cudaSuccess) st = fail(QTRAJ_ECUDA, "upload of the Coulomb basis failed");
+    else st = p.precision == QTRAJ_FP32 ? build_tables<float>(c, s) : build_tables<double>(c, s);
+    cudaStreamSynchronize(s);
+    cudaStreamDestroy(s);
     if (st != QTRAJ_OK) return bail(st);
-    const std::vector<double> &eig = c->basis_host;
-    if (cudaMalloc(&c->eig, sizeof(double) * eig.size()) != cudaSuccess) return bail(fail(QTRAJ_ENOMEM, "cudaMalloc"));
-    if (cudaMemcpy(c->eig, eig.data(), sizeof(double) * eig.size(), cudaMemcpyHostToDevice) != cudaSuccess)
-        return bail(fail(QTRAJ_ECUDA, "upload of the Coulomb basis failed"));
     if (cudaEventCreateWithFlags(&c->ev_stage, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreate(&c->ev0) != cudaSuccess || cudaEventCreate(&c->ev1) != cudaSuccess ||
         cudaEventCreate(&c->ev2) != cudaSuccess)
@@ -860,8 +879,8 @@ void qtraj_destroy(qtraj_ctx *c)
     free_ptr(c->WL);
     free_ptr(c->KT);
     free_ptr(c->sinpre);
-    for (qtraj_ctx::TabSet *t : {&c->fused, &c->plain})
-        for (void **p : t->all) free_ptr(*p);
+    free_ptr(c->fused.base);
+    free_ptr(c->plain.base);
     free_ptr(c->phi_tab);
     free_typed(c->eig);
     free_typed(c->ic);

@@ -77,7 +77,7 @@ template <> struct Prec<double> {
     using C = cpx<double>; // complex constant
     using Rl = double;     // real constant
     static __host__ C make(double re, double im) { return {re, im}; }
-    static __host__ Rl make_r(double v) { return v; }
+    static __host__ __device__ Rl make_r(double v) { return v; }
     static __device__ __forceinline__ cpx<double> mul(cpx<double> x, C w) { return x * w; }
     static __device__ __forceinline__ C conj(C w) { return {w.x, -w.y}; }
     using D = C;           // (FP32: a direction, below)
@@ -104,7 +104,7 @@ template <> struct Prec<float> {
         const float rh = (float)re, ih = (float)im;
         return {rh, ih, (float)(re - (double)rh), (float)(im - (double)ih)};
     }
-    static __host__ Rl make_r(double v)
+    static __host__ __device__ Rl make_r(double v)
     {
         const float h = (float)v;
         return {h, (float)(v - (double)h)};
