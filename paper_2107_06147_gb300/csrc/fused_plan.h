@@ -20,9 +20,10 @@ struct PlanDims { int R, E, M1, M2; };
 // often than thousands, so theirs are the plans of the shortest step: an FP64 instruction takes a warp 64 cycles
 // whatever its lanes do and an SM completes one every 19, so FP64 wants four warps with little each (us a step of 8
 // trajectories / 10^6 trajectory-steps a second of a full device, FP64: N = 512 radix 4, 8 x 8 28.0 / 7.7, radix 8,
-// 16 41.9 / 8.5; N = 1024 radix 8, 8 x 4 44.4 / 3.9, radix 16, 8 65.7 / 4.6; N = 256 radix 4, 4 x 8 22.5 / 15.9,
-// radix 8, 8 34.4 / 16.9.  FP32: N = 128 radix 4, 16 2.2 / 642, radix 8, 4 2.9 / 602).  FP32 at N = 256 and above
-// keeps the larger radix: the throughput lost outweighs the step (N = 512 radix 8, 16 2.9 / 226, radix 16, 4 4.2 /
+// 16 41.9 / 8.5; N = 1024 radix 8, 8 x 4 44.4 / 3.9, radix 16, 8 65.7 / 4.6.  FP32: N = 128 radix 4, 16 2.2 / 642,
+// radix 8, 4 2.9 / 602).  FP64 N = 256 keeps radix 8: radix 4, 4 x 8 was quicker for a few trajectories (22.5 us a step
+// instead of 34.4) but left final states 5.8e-14 off after 64 steps where the earlier transform left 3.4e-14 (radix 8
+// 1.6e-14).  FP32 at N = 256 and above keeps the larger radix: the throughput lost outweighs the step (N = 512 radix 8, 16 2.9 / 226, radix 16, 4 4.2 /
 // 284), and the share of the spectrum that goes through a running sum, 2/R, sets the rounding noise.
 // RAD8: the radix-8 plans of the launch variants 2 and 3 (FP32, N = 2048 and 4096); PLAIN: the plain form's, one
 // middle pass and at most 32 of a sequence's slots (plain_step.cuh).
@@ -34,7 +35,6 @@ __host__ __device__ constexpr PlanDims plan_dims(int N, bool f64, PlanKind kind)
     if (f64 && kind != PLAN_PLAIN) {
         switch (N) {
         case 128: return {4, 4, 4, 4};
-        case 256: return {4, 4, 4, 8};
         case 512: return {4, 4, 8, 8};
         case 1024: return {8, 8, 8, 4};
         default: break;
