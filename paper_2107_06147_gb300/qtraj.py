@@ -298,7 +298,8 @@ class Engine:
 
     def evolve(self, media, seeds, medium_idx=None, batch: int | None = None, stream=None):
         batch = len(seeds) if batch is None else batch
-        arr = media if isinstance(media, C.Array) else (Medium * len(media))(*media)   # a list, or laid out once
+        # an array of Medium as it is, anything else (a list, an array of a larger structure) converted
+        arr = media if isinstance(media, C.Array) and media._type_ is Medium else (Medium * len(media))(*media)
         self._seeds = np.ascontiguousarray(seeds, dtype=np.uint64)
         idx = None
         if medium_idx is not None:
