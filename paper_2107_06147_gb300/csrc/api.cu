@@ -133,9 +133,15 @@ struct qtraj_ctx {
     size_t off_trajs = 0, off_obs = 0, off_gtrajs = 0, off_gobs = 0, off_gready = 0, off_ctr = 0, off_states = 0,
            off_plain = 0;
     // host staging and timing
-    void *h_stage = nullptr;
-    size_t h_stage_bytes = 0;
-    cudaEvent_t ev_stage = nullptr, ev0 = nullptr, ev1 = nullptr, ev2 = nullptr;
+    // Staging buffers: an upload is queued behind the kernel before it, so that a call that waited for the previous
+    // call's upload would wait for that kernel; it takes the other buffer instead, which is made when first needed
+    struct Stage {
+        void *host = nullptr;
+        size_t bytes = 0;
+        cudaEvent_t ev = nullptr;   // its last upload
+    } stage[2];
+    int stage_at = 0;
+    cudaEvent_t ev0 = nullptr, ev1 = nullptr, ev2 = nullptr;
     bool evolved = false;
     int last_batch = 0, last_groups = 0, last_n_media = 0, launches = 0;
     std::vector<int> group_pair;
@@ -649,6 +655,17 @@ const char *medium_check(const qtraj_medium &q, const double *prof = nullptr, in
     return nullptr;
 }
 
+// a larger staging buffer in the place of one that no upload reads any more
+cudaError_t grow_stage(qtraj_ctx::Stage &st, size_t bytes)
+{
+    if (st.host) cudaFreeHost(st.host);
+    st.host = nullptr;
+    st.bytes = 0;
+    const cudaError_t e = cudaMallocHost(&st.host, bytes);
+    if (e == cudaSuccess) st.bytes = bytes;
+    return e;
+}
+
 // the device record of a medium on a context's grid
 MediumDev encode_medium(const qtraj_ctx *c, const qtraj_medium &q)
 {
@@ -863,7 +880,8 @@ qtraj_status qtraj_create(int N, double L, double dt, double M, const qtraj_para
     cudaStreamSynchronize(s);
     cudaStreamDestroy(s);
     if (st != QTRAJ_OK) return bail(st);
-    if (cudaEventCreateWithFlags(&c->ev_stage, cudaEventDisableTiming) != cudaSuccess ||
+    if (cudaEventCreateWithFlags(&c->stage[0].ev, cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&c->stage[1].ev, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreate(&c->ev0) != cudaSuccess || cudaEventCreate(&c->ev1) != cudaSuccess ||
         cudaEventCreate(&c->ev2) != cudaSuccess)
         return bail(fail(QTRAJ_ECUDA, "cudaEventCreate failed"));
@@ -890,8 +908,10 @@ void qtraj_destroy(qtraj_ctx *c)
     free_typed(c->spec_color);
     free_typed(c->prof);
     free_typed(c->media);
-    if (c->h_stage) cudaFreeHost(c->h_stage);
-    if (c->ev_stage) cudaEventDestroy(c->ev_stage);
+    for (auto &st : c->stage) {
+        if (st.host) cudaFreeHost(st.host);
+        if (st.ev) cudaEventDestroy(st.ev);
+    }
     if (c->ev0) cudaEventDestroy(c->ev0);
     if (c->ev1) cudaEventDestroy(c->ev1);
     if (c->ev2) cudaEventDestroy(c->ev2);
@@ -1075,21 +1095,23 @@ qtraj_status qtraj_evolve(qtraj_ctx *c, int batch, const qtraj_medium *media, in
     cudaStream_t s = (cudaStream_t)stream;
     const int N = c->N;
 
-    // The descriptors are written straight into the pinned staging buffer (media | trajs | group trajs).  A batch
+    // The descriptors are written straight into a pinned staging buffer (media | trajs | group trajs).  A batch
     // with a medium per trajectory spent most of the call in a std::map of the (state, medium) groups, which only
     // the rMin shortcut uses (the KSU evolution has no jumps and no shortcut).
     const bool grouped = c->p.use_rmin && c->p.potential == 0;
     const size_t b_md = sizeof(MediumDev) * n_media, b_tr = sizeof(TrajDev) * batch;
     const size_t need = align256(b_md) + align256(b_tr) + (grouped ? align256(b_tr) : 0) + 256;
-    CK(cudaEventSynchronize(c->ev_stage));   // the previous upload has left the staging buffer
-    if (need > c->h_stage_bytes) {
-        if (c->h_stage) cudaFreeHost(c->h_stage);
-        c->h_stage = nullptr;
-        c->h_stage_bytes = 0;
-        CK(cudaMallocHost(&c->h_stage, need));
-        c->h_stage_bytes = need;
+    const cudaError_t up = cudaEventQuery(c->stage[c->stage_at].ev);
+    if (up == cudaErrorNotReady) {
+        cudaGetLastError();
+        c->stage_at ^= 1;
+        CK(cudaEventSynchronize(c->stage[c->stage_at].ev));   // (the upload before the previous one)
+    } else {
+        CK(up);
     }
-    char *h = (char *)c->h_stage;
+    qtraj_ctx::Stage &stage = c->stage[c->stage_at];
+    if (need > stage.bytes) CK(grow_stage(stage, need));
+    char *h = (char *)stage.host;
     MediumDev *md = (MediumDev *)h;
     TrajDev *tr = (TrajDev *)(h + align256(b_md)), *gt = (TrajDev *)(h + align256(b_md) + align256(b_tr));
     std::vector<int> steps(n_media);
@@ -1145,7 +1167,7 @@ qtraj_status qtraj_evolve(qtraj_ctx *c, int batch, const qtraj_medium *media, in
     CK(cudaMemcpyAsync(c->media, md, b_md, cudaMemcpyHostToDevice, s));
     if (b_tr) CK(cudaMemcpyAsync(d_tr, tr, b_tr, cudaMemcpyHostToDevice, s));
     if (b_gt) CK(cudaMemcpyAsync(d_gt, gt, b_gt, cudaMemcpyHostToDevice, s));
-    CK(cudaEventRecord(c->ev_stage, s));
+    CK(cudaEventRecord(stage.ev, s));
     CK(cudaMemsetAsync(d_ctr, 0, 256, s));
 
     c->launches = 0;
@@ -1249,13 +1271,10 @@ qtraj_status reserve_media(qtraj_ctx *c, int n)
     }
     // the pinned staging of an evolve of n trajectories with up to n media and n groups
     const size_t need = align256(sizeof(MediumDev) * n) + 2 * align256(sizeof(TrajDev) * n) + 256;
-    if (need > c->h_stage_bytes) {
+    // (one buffer: a slot's launch has finished before its next one is prepared)
+    if (need > c->stage[c->stage_at].bytes) {
         CK(cudaDeviceSynchronize());
-        if (c->h_stage) CK(cudaFreeHost(c->h_stage));
-        c->h_stage = nullptr;
-        c->h_stage_bytes = 0;
-        CK(cudaMallocHost(&c->h_stage, need));
-        c->h_stage_bytes = need;
+        CK(grow_stage(c->stage[c->stage_at], need));
     }
     return QTRAJ_OK;
 }
