@@ -15,16 +15,18 @@ namespace qt {
 
 struct PlanDims { int R, E, M1, M2; };
 
-// The plans.  FP32 up to N = 4096 and FP64: 16 values a thread where two warps of a trajectory then share an SM
-// quarter and its instruction fetch, 32 above (fewer exchanges).  Small grids run few trajectories at a time more
-// often than thousands, so theirs are the plans of the shortest step: an FP64 instruction takes a warp 64 cycles
-// whatever its lanes do and an SM completes one every 19, so FP64 wants four warps with little each (us a step of 8
-// trajectories / 10^6 trajectory-steps a second of a full device, FP64: N = 512 radix 4, 8 x 8 28.0 / 7.7, radix 8,
-// 16 41.9 / 8.5; N = 1024 radix 8, 8 x 4 44.4 / 3.9, radix 16, 8 65.7 / 4.6.  FP32: N = 128 radix 4, 16 2.2 / 642,
-// radix 8, 4 2.9 / 602).  FP64 N = 256 keeps radix 8: radix 4, 4 x 8 was quicker for a few trajectories (22.5 us a step
-// instead of 34.4) but left final states 5.8e-14 off after 64 steps where the earlier transform left 3.4e-14 (radix 8
-// 1.6e-14).  FP32 at N = 256 and above keeps the larger radix: the throughput lost outweighs the step (N = 512 radix 8, 16 2.9 / 226, radix 16, 4 4.2 /
-// 284), and the share of the spectrum that goes through a running sum, 2/R, sets the rounding noise.
+// The plans.  FP32 up to N = 4096: 16 values a thread where two warps of a trajectory then share an SM quarter and its
+// instruction fetch, 32 above (fewer exchanges).  FP64: 4 to 32 values a thread.  An FP64 instruction takes a warp 64
+// cycles whatever its lanes do and an SM completes one every 19, so a few FP64 trajectories want four warps with little
+// each, and a full device few instructions; the plans up to N = 1024 are those of the shorter step (us a step of 8
+// trajectories / 10^6 trajectory-steps a second of 3000): N = 1024 radix 8, 8 x 4 44.4 / 3.9, radix 16, 8 65.7 / 4.6;
+// FP32 N = 128 radix 4, 16 2.2 / 642, radix 8, 4 2.9 / 602.
+// The share of the spectrum that goes through a running sum, 2/R, sets the rounding noise: FP64 N = 256 and 512 keep radix 8
+// for it.  Radix 4, 4 x 8 at N = 256 left final states 5.8e-14 off after 64 steps where the earlier transform left
+// 3.4e-14 (radix 8 1.6e-14); radix 4, 8 x 8 at N = 512 left 2.5e-14 after 4 steps (earlier transform 0.9e-14; radix 8,
+// 8 x 2 0.6e-14; radix 8, 16 0.4e-14; a step of 8 trajectories 29.5, 37.9 and 41.8 us, 300 steps of 3000 58.0, 61.3 and
+// 58.7 ms).  FP32 at N = 256 and above keeps the larger radix, for the noise and for the throughput (N = 512 radix 8,
+// 16 2.9 / 226, radix 16, 4 4.2 / 284).
 // RAD8: the radix-8 plans of the launch variants 2 and 3 (FP32, N = 2048 and 4096); PLAIN: the plain form's, one
 // middle pass and at most 32 of a sequence's slots (plain_step.cuh).
 enum PlanKind { PLAN_FUSED = 0, PLAN_RAD8 = 1, PLAN_PLAIN = 2 };
@@ -35,7 +37,7 @@ __host__ __device__ constexpr PlanDims plan_dims(int N, bool f64, PlanKind kind)
     if (f64 && kind != PLAN_PLAIN) {
         switch (N) {
         case 128: return {4, 4, 4, 4};
-        case 512: return {4, 4, 8, 8};
+        case 512: return {8, 8, 8, 2};
         case 1024: return {8, 8, 8, 4};
         default: break;
         }

@@ -8,6 +8,27 @@ from test_gpu_parity import check_fp32, check_fp64, fp32_bound, oracle_inputs, q
 pytestmark = pytest.mark.gpu
 
 
+@pytest.mark.parametrize("N,bound", [(256, 4.7e-15), (512, 9.4e-15), (2048, 3.1e-14)])
+def test_fp64_states_of_a_few_steps(q, N, bound):  # noqa: F811
+    """Final states of four steps, no further from 64-bit arithmetic than a transform through one N-point FFT leaves
+    them (bound: its largest error over six seeds of such media).  The plans' running sum over 2/R of the spectrum is
+    what sets the error here: radix 4 at N = 512 left 2.5e-14."""
+    from paper_2107_06147_gb300 import inputs
+    w = inputs.small_parity(N=N, n_traj=24, seed=2)
+    w.grid.L, w.grid.dt = N * (5.0 / 256 if N <= 256 else 5.0 / 512), 0.001
+    w.inits = [inputs.InitSpec("gauss", 0.8, 1, 0, 0), inputs.InitSpec("coulomb", 0.0, 1, 0, 0),
+               inputs.InitSpec("coulomb", 0.0, 2, 0, 0), inputs.InitSpec("gauss", 0.8, 2, 1, 0)]
+    w.init_idx = (np.arange(24) % 4).astype(np.int32)
+    Tf = 0.42 * (0.6 / (0.6 + 3.5 * 0.1973269804 * 0.001)) ** (1 / 3)
+    w.media = [inputs.MediumSpec(0.42, 0.6, Tf, k, g) for k in (4.0, 5.0, 6.0) for g in (-2.0, 0.0)]
+    w.medium_idx = (np.arange(24) // 4).astype(np.int32)
+    w.seeds = np.full(24, 117390, np.uint64)   # (a first threshold of 7e-7: no jump)
+    ref, uref = run_oracle(w, use_rmin=0)
+    obs, u = run_gpu(q, w, q.FP64, use_rmin=0)
+    assert (ref["n_jumps"] == 0).all() and (obs["n_steps_exec"] == 4).all()
+    assert np.linalg.norm(u - uref) <= bound * np.linalg.norm(uref), np.linalg.norm(u - uref) / np.linalg.norm(uref)
+
+
 def test_repeated_evolves_do_not_wait_for_the_first(q):  # noqa: F811
     """Three evolves queued on one stream: the third call prepares and returns while the first one's kernel runs (its
     descriptors may not wait for the second upload, which is queued behind that kernel)."""
