@@ -529,7 +529,7 @@ template <> struct Dyn<double> {
         *m = e;
         return PHASE ? mk(e * c, e * s) : mk(e, 0.0);
     }
-    // exp(z) for the temperature's change over one step, |z| <~ 1e-4: the series to z^3
+    // exp(z) for the temperature's change over one step (factor_regs): the series to z^3
     static __device__ __forceinline__ double near1(double z) { return 1.0 + z * (1.0 + z * (0.5 + z * (1.0 / 6.0))); }
     static __device__ __forceinline__ void f1(double a, double y, double *fr, double *fi, double *e)
     {
@@ -1020,11 +1020,15 @@ template <typename T, int N, int V> struct Pointwise {
     // (the end-of-step norm / dr).  dyn = exp((er + i ei) r^2), er and ei multiplied by T^3; A = (er_a + er_b)
     // dr^2, B = (ei_a + ei_b) dr^2 / pi, D = (er_a - er_b) dr^2, rounded once per step and multiplied with the
     // exact j^2 (N <= 4096; rounded once above), so no rounding that repeats identically every step enters.
-    // exp(2 er_a r^2) = mag exp((er_a - er_b) r^2), the second factor 1 + z with |z| <~ 1e-4 (the temperature's
-    // change over one step): FP32 keeps the first order.
+    // exp(2 er_a r^2) = mag exp((er_a - er_b) r^2), the second factor by its series in z = D j^2 = delta a, with a the
+    // exponent of mag and delta = D / A the relative change of the temperature's factor over one step (1.6e-4 for a
+    // Bjorken medium at 0.6 fm/c and dt = 0.001): FP32 keeps the first order, FP64 the third.  What the series leave
+    // out of mag exp(z) is at most 0.27 delta^2 and 0.2 delta^4 at any a <= 0; the caller keeps |delta| below
+    // series_delta, where that is 1e-6 (the FP32 state is some 1e-6 off) and 3e-12, and takes factor() beyond.
     // The first half-step of a trajectory and the last of its last step are the same with the half-step rows and
     // only one half-step's coefficients (last: the sum is |x_new|^2).
     // PHASE = false: gamma_hat = 0, B = 0 exactly, the phase series is skipped (its value would be 0).
+    static constexpr T series_delta = (T)(1.0 / 512);
     template <bool PHASE>
     static __device__ __forceinline__ void factor_regs(cpx<T> *x, const SC *row, int g, T A, T B, T D, bool last,
                                                        SqAcc<T> &acc, SqAcc<T> &acc2)
@@ -1102,31 +1106,25 @@ template <typename T, int N, int V> struct Pointwise {
 
     // The same in loops over the copy in shared memory, for every mode:
     // mode 0: x <- stat1 dyn_b x (the first half-step of a trajectory)
-    // mode 1: x <- stat2 dyn_a dyn_b x; returns sum exp(2 er_a r^2) |x_old|^2 (end-of-step norm / dr)
+    // mode 1: x <- stat2 dyn_a dyn_b x; returns sum exp(W j^2) |x_old|^2, W = 2 er_a dr^2 (end-of-step norm / dr)
     // mode 2: x <- stat1 dyn_a x; returns sum |x_new|^2
     static __device__ __noinline__ typename NormSum<T>::type factor(cpx<T> *buf, const Tables<T> &tb, int g, int c, int l,
-                                                                    int mode, T A, T B, T D, double *red)
+                                                                    int mode, T A, T B, T W, double *red)
     {
         SqAcc<T> acc;
         const SC *tab = (mode == 1) ? tb.statV2 : tb.statV;
 #pragma unroll 4
         for (int e = 0; e < E; ++e) {
             const T fj = (T)jof(g, e);
-            T f1r, f1i, em1, z;
+            T f1r, f1i, em1;
             if constexpr (sizeof(T) == 4) {
                 const T j2 = fj * fj;
                 Dyn<T>::f1t(A * j2, ((T)3.14159265358979323846 * B) * j2, &f1r, &f1i, &em1);
-                z = D * j2;
             } else {
                 Dyn<T>::f1((A * fj) * fj, (B * fj) * fj, &f1r, &f1i, &em1);
-                z = (D * fj) * fj;
             }
-            const T mag = (T)1 + em1;
             cpx<T> v = buf[e * G + g];
-            if (mode == 1) {
-                if constexpr (sizeof(T) == 4) acc.add_w(v, mag + mag * z);
-                else acc.add_w(v, mag * ((T)1 + z * ((T)1 + z * ((T)0.5 + z * (T)(1.0 / 6.0)))));
-            }
+            if (mode == 1) acc.add_w(v, k_exp((W * fj) * fj));
             v = apply(PR::mul_s(v, stat(tb, tab, c, l, g, e, mode == 1)), f1r, f1i);
             if (mode == 2) acc.add_w(v, (T)1);
             buf[e * G + g] = v;
@@ -1490,8 +1488,9 @@ __global__ void __launch_bounds__(FusedPlan<T, N, V>::G, (FusedBounds<T, N, V>::
             const T cA = erj * Ksum, cB = eij * Tsum, cD = start || last ? (T)0 : erj * (K3a - K3b);
             const int mode = start ? 0 : last ? 2 : 1;
             NS2 n2s;   // norm^2 / dr
-            // (phases beyond 1e5: far2's reduction would lose them)
-            if (KSU || l >= LTAB || !(fabs(cB) * (T)N * (T)N < (T)3e4)) {
+            // (phases beyond 1e5: far2's reduction would lose them; a temperature that changes by more within a step than
+            // the norm's weight allows: steep tabulated media, or dt above 0.01 in a Bjorken medium at 0.6 fm/c)
+            if (KSU || l >= LTAB || !(fabs(cB) * (T)N * (T)N < (T)3e4) || fabs(cD) > PW::series_delta * fabs(cA)) {
                 traj_sync<G>();   // all have read the transform's output
                 PW::to_smem(x, buf, g);
                 in_smem = true;
@@ -1500,7 +1499,7 @@ __global__ void __launch_bounds__(FusedPlan<T, N, V>::G, (FusedBounds<T, N, V>::
                     kb = ksu_at<T>(tb, T3b);
                     n2s = PW::factor_ksu(buf, tb, g, l, mode, ka, kb, red);
                 } else {
-                    n2s = PW::factor(buf, tb, g, c, l, mode, cA, cB, cD, red);
+                    n2s = PW::factor(buf, tb, g, c, l, mode, cA, cB, 2 * erj * K3a, red);
                 }
             } else {
                 SqAcc<T> acc, acc2;

@@ -29,6 +29,46 @@ def test_fp64_states_of_a_few_steps(q, N, bound):  # noqa: F811
     assert np.linalg.norm(u - uref) <= bound * np.linalg.norm(uref), np.linalg.norm(u - uref) / np.linalg.norm(uref)
 
 
+def _pulsed(T, dt, tau0):
+    """A table with the temperatures T at the steps, constant around each step's time."""
+    t = tau0 + np.arange(len(T)) * dt * 0.1973269804
+    d = 0.3 * dt * 0.1973269804
+    tau = np.stack([t - d, t + d], 1).ravel()
+    tau[0] = tau0
+    return tau, np.repeat(T, 2)
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("N", [256, 2048])
+def test_temperature_that_changes_within_a_step(q, N, precision):  # noqa: F811
+    """The end-of-step norm is taken before the merged half-steps of two temperatures are applied; its weight has to
+    hold for any change of T over a step, not only for the 1e-4 of a Bjorken medium: a rise and a fall by 2.5 within
+    the first steps, on states whose exponents reach 5 a step."""
+    import torch
+    import oracle as o
+    n, dt, kappa = 400, 0.02, 150.0
+    tau, T = _pulsed(np.array([0.2, 0.5] + 8 * [0.2] + [0.5, 0.2, 0.2]), dt, 0.6)
+    g = o.Grid(N=N, L=20.0, dt=dt, use_rmin=0)
+    idx = (np.arange(n) % 2).astype(np.int32)
+    seeds = np.arange(n, dtype=np.uint64)
+    states = [("gauss", 2.0, 1, 0, 0), ("gauss", 3.0, 2, 1, 0)]
+    ref, _, uref = o.run_batch(g, [o.init_spec(*s) for s in states], idx,
+                               [o.table_medium(tau, T, Tf=0.15, kappa_hat=kappa, gamma_hat=-1.0)],
+                               np.zeros(n, np.int32), seeds, want_states=True)
+    assert (ref["n_steps_exec"] >= 12).all() and (ref["n_jumps"] > 0).mean() > 0.9
+    e = q.Engine(q.Config(N=N, L=20.0, dt=dt, precision=precision, use_rmin=0, save_states=1))
+    e.set_profiles(tau, T)
+    e.init([q.init_spec(*s) for s in states], n, idx)
+    e.evolve([q.table_medium(0, len(tau), 0.15, kappa, -1.0)], seeds, np.zeros(n, np.int32))
+    obs, u = e.observables(), e.states()
+    torch.cuda.synchronize()
+    e.close()
+    if precision == 0:
+        check_fp64(q, obs, ref, u, uref)
+    else:
+        check_fp32(q, obs, ref, u, uref, min_same=0.98)
+
+
 def test_repeated_evolves_do_not_wait_for_the_first(q):  # noqa: F811
     """Three evolves queued on one stream: the third call prepares and returns while the first one's kernel runs (its
     descriptors may not wait for the second upload, which is queued behind that kernel)."""
