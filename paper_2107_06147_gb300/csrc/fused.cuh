@@ -471,11 +471,11 @@ template <> struct Dyn<float> {
     }
     // the same beyond the series' range, reduced to it by Cody and Waite's two-part constants: exp(a) = 2^n exp(a - n ln 2), and t - 2 pi k quartered
     // and doubled back twice (cos 2x - 1 = -2 sin^2 x, sin 2x = 2 sin x (1 + (cos x - 1))); a < -87 counts as
-    // -87, |t| <= 1e5
+    // -87 (not a NaN, which 0 x inf at r = 0 is and which the norm has to show), |t| <= 1e5
     static __device__ __forceinline__ void far2(float2 a, float2 t, float2 *fr, float2 *fi, float2 *e)
     {
         const float2 magic = rep(12582912.0f);   // 1.5 x 2^23: adding it rounds to the nearest integer
-        a = make_float2(fmaxf(a.x, -87.0f), fmaxf(a.y, -87.0f));
+        a = make_float2(a.x < -87.0f ? -87.0f : a.x, a.y < -87.0f ? -87.0f : a.y);
         const float2 nm = __ffma2_rn(a, rep(1.44269504088896341f), magic);
         const float2 n = __fadd2_rn(nm, rep(-12582912.0f));
         float2 r = __ffma2_rn(n, rep(-0.693147182464599609f), a);

@@ -69,6 +69,44 @@ def test_temperature_that_changes_within_a_step(q, N, precision):  # noqa: F811
         check_fp32(q, obs, ref, u, uref, min_same=0.98)
 
 
+@pytest.mark.parametrize("N", [128, 512, 2048, 8192])
+def test_fp32_exponents_beyond_single_precision(q, N):  # noqa: F811
+    """A wide state on a long grid, kappa_hat 6 and 60: exponents to -11 and -109 and phases to -6 a step at the
+    largest r.  The seed's first threshold (6.9e-7) is below every norm, so nothing jumps."""
+    from paper_2107_06147_gb300 import inputs
+    w = inputs.small_parity(N=N, n_traj=4, seed=1)
+    w.grid.L, w.grid.dt = 200.0, 0.001
+    w.inits = [inputs.InitSpec("gauss", 30.0, 1, 0, 0), inputs.InitSpec("gauss", 60.0, 2, 1, 0)]
+    w.media = [inputs.MediumSpec(0.45, 0.6, 0.4495, 6.0, -3.5), inputs.MediumSpec(0.45, 0.6, 0.4495, 60.0, -3.5)]
+    w.init_idx, w.medium_idx = np.array([0, 1, 0, 1], np.int32), np.array([0, 0, 1, 1], np.int32)
+    w.seeds = np.full(4, 117390, np.uint64)
+    ref, uref = run_oracle(w, use_rmin=0)
+    obs, u = run_gpu(q, w, q.FP32, use_rmin=0)
+    assert (ref["n_jumps"] == 0).all() and (obs["n_jumps"] == 0).all() and (ref["n_steps_exec"] == 11).all()
+    bound = fp32_bound(N, ref["n_steps_exec"])
+    du = np.linalg.norm(u - uref, axis=1) / np.linalg.norm(uref, axis=1)
+    assert (du <= bound).all(), du / bound
+    assert (np.abs(obs["norm2"] / ref["norm2"] - 1) <= 2 * bound).all(), obs["norm2"] / ref["norm2"] - 1
+
+
+@pytest.mark.parametrize("Tf", [0.399, 0.39999])
+@pytest.mark.parametrize("gamma", [0.0, -1.0])
+def test_fp32_exponent_that_overflows_is_reported(q, gamma, Tf):  # noqa: F811
+    """kappa_hat = 1e300 passes the host's checks and its coefficient is infinite in FP32: 0 x inf at r = 0 is not a
+    number and is flagged, in media of one step and more, with jumps capped as well (no renormalisation of a zero
+    state then)."""
+    import torch
+    e = q.Engine(q.Config(N=512, L=5.0, dt=0.001, precision=q.FP32, use_rmin=0, max_jumps=0))
+    e.init([q.init_spec("gauss", 0.3, 1, 0, 0)], 2)
+    e.evolve([q.medium(0.4, 0.6, Tf, 1e300, gamma)], np.arange(2, dtype=np.uint64))
+    o = e.observables(check_finite=False)
+    with pytest.raises(q.QtrajError) as ei:
+        e.observables()
+    torch.cuda.synchronize()
+    e.close()
+    assert ei.value.status == 5 and (o["flags"] & q.F_NONFINITE).all(), o["flags"]
+
+
 def test_repeated_evolves_do_not_wait_for_the_first(q):  # noqa: F811
     """Three evolves queued on one stream: the third call prepares and returns while the first one's kernel runs (its
     descriptors may not wait for the second upload, which is queued behind that kernel)."""
