@@ -41,7 +41,8 @@ typedef enum {
 } qtraj_status;
 
 /* arithmetic of the step.  FP32: the waiting-time comparison is in double-float, the final norm and the overlaps are
- * sums of FP32 products in error-free parts (2^-46 of the terms), reported as FP64 */
+ * sums of FP32 products in error-free parts (within 2^-46 of the sum of the terms' magnitudes), in FP64 where such
+ * products would leave FP32's range, reported as FP64 */
 typedef enum { QTRAJ_FP64 = 0, QTRAJ_FP32 = 1 } qtraj_precision;
 
 /* QTRAJ_FUSED: one persistent kernel; every trajectory stays in shared memory/registers for its

@@ -223,6 +223,10 @@ struct Dot2 {
     __device__ __forceinline__ double x() const { return (double)s.x + (double)c.x; }
     __device__ __forceinline__ double y() const { return (double)s.y + (double)c.y; }
 };
+// Where a norm's sum by Dot2 is taken: the parts of products below 2^-149 are lost and those above 2^128 overflow, N 2^-149
+// in all, which is less than 2^-53 of a sum above 2^-80.  Other sums (states decayed without a jump, and non-finite
+// ones), and states without a step behind them, whose overlaps may cancel to any depth, are taken again in FP64.
+__device__ __forceinline__ bool dot2_holds(double norm) { return norm > 0x1p-80 && norm < 0x1p100; }
 struct Dot1 {   // the FP64 form
     double s = 0.0, t = 0.0;
     __device__ __forceinline__ void add(double f, cpx<double> u) { s = fma(f, u.x, s); t = fma(f, u.y, t); }
@@ -1271,6 +1275,28 @@ template <typename T, int N, int V> struct Pointwise {
         }
     }
 
+    // fin <- the sums of the read-out (norm^2 / dr, overlaps / dr with the nb basis states of l) of an FP32 state in FP64
+    static __device__ __noinline__ void read_out64(const cpx<T> *buf, const Tables<T> &tb, int g, int nb, int l, double *red,
+                                                   double *fin)
+    {
+        double v[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+        const double *phi = tb.eig + (size_t)(l == 0 ? 0 : l == 1 ? 2 : 5) * N;   // 1S 2S . 3S, 1P . 2P, 1D
+#pragma unroll 1
+        for (int e = 0; e < E; ++e) {
+            const int j = jof(g, e);
+            const double sg = odd_half(e) ? -1.0 : 1.0, x = sg * (double)buf[e * G + g].x, y = sg * (double)buf[e * G + g].y;
+            v[0] = fma(x, x, fma(y, y, v[0]));
+#pragma unroll
+            for (int i = 0; i < 3; ++i)
+                if (i < nb) {
+                    const double f = phi[(size_t)(l == 1 ? 2 * i : i == 2 ? 3 : i) * N + j];
+                    v[1 + 2 * i] = fma(f, x, v[1 + 2 * i]);
+                    v[2 + 2 * i] = fma(f, y, v[2 + 2 * i]);
+                }
+        }
+        slot_sums8<G>(v, red, fin);
+    }
+
     // x <- x * r_j * f
     static __device__ void scale_r(cpx<T> *buf, const Tables<T> &tb, int g, double f)
     {
@@ -1614,6 +1640,10 @@ __global__ void __launch_bounds__(FusedPlan<T, N, V>::G, (FusedBounds<T, N, V>::
         else if (nb == 3) observe(std::integral_constant<int, 3>{});
         else if (nb == 2) observe(std::integral_constant<int, 2>{});
         else observe(std::integral_constant<int, 1>{});
+        if constexpr (sizeof(T) == 4) {
+            traj_sync<G>();
+            if (ns == 0 || !dot2_holds(fin[0])) PW::read_out64(buf, tb, g, nb, l, red, fin);
+        }
         if (a.states && !grp) {
             double *st = a.states + (size_t)t * N * 2;
 #pragma unroll 4

@@ -301,6 +301,28 @@ template <int N> struct NftPointwise {
         return static_far<T>(tb.coul[c], tb.M, tb.dt, l, j * tb.dr, full ? 2.0 : 1.0);
     }
 
+    // the read-out's sums in FP64 (Pointwise::read_out64)
+    static __device__ __noinline__ void read_out64(const cpx<T> *buf, const Tables<T> &tb, int g, int nb, int l, double *red,
+                                                   double *fin)
+    {
+        double v[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+        const double *phi = tb.eig + (size_t)(l == 0 ? 0 : l == 1 ? 2 : 5) * N;
+#pragma unroll 1
+        for (int j = 2 * g; j < N; j += (j & 1) ? 2 * G - 1 : 1) {   // the pairs of points g, g + G, ...
+            const cpx<T> u = buf[K::s_pos(j)];
+            const double x = u.x, y = u.y;
+            v[0] = fma(x, x, fma(y, y, v[0]));
+#pragma unroll
+            for (int i = 0; i < 3; ++i)
+                if (i < nb) {
+                    const double f = phi[(size_t)(l == 1 ? 2 * i : i == 2 ? 3 : i) * N + j];
+                    v[1 + 2 * i] = fma(f, x, v[1 + 2 * i]);
+                    v[2 + 2 * i] = fma(f, y, v[2 + 2 * i]);
+                }
+        }
+        slot_sums8<G>(v, red, fin);
+    }
+
     // The potential factor and a norm sum that tells a non-finite state (there are no jumps, so nothing else is
     // done with it and the sum leaves out the weight |K_V|^2, an expf a point):
     // mode 0: x <- stat1 dyn_b x (the first half-step of a trajectory)
@@ -464,6 +486,8 @@ __global__ void __launch_bounds__(NftPlan<N>::G, (NftPlan<N>::MIN_BLOCKS)) ksu32
             }
             double v[8] = {norm.x() + norm.y(), dot[0].x(), dot[0].y(), dot[1].x(), dot[1].y(), dot[2].x(), dot[2].y(), 0};
             slot_sums8<G>(v, red, fin);
+            traj_sync<G>();
+            if (ns == 0 || !dot2_holds(fin[0])) PW::read_out64(buf, tb, g, nb, l, red, fin);
         }
         if (a.states) {
             double *st = a.states + (size_t)t * N * 2;

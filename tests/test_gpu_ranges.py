@@ -8,6 +8,32 @@ from test_gpu_parity import check_fp32, check_fp64, fp32_bound, oracle_inputs, q
 pytestmark = pytest.mark.gpu
 
 
+@pytest.mark.parametrize("potential", [0, 1])
+def test_fp32_read_out_of_decayed_states(q, potential):  # noqa: F811
+    """No-jump evolutions whose norm falls to 1e-26 .. 1e-53, where squares of the FP32 amplitudes underflow: norms
+    and ratios as the FP64 form's, within the FP32 state's error (norm and ratio are quadratic in it)."""
+    import torch
+    if potential:
+        N, L, dt, med = 64, 12.0, 0.05, q.medium(2.0, 25.0, 1.5, 0.0, 0.0)
+    else:
+        N, L, dt, med = 64, 6.0, 0.01, q.medium(0.6, 0.6, 0.3, 100.0, -1.0)
+    res = []
+    for prec in (q.FP64, q.FP32):
+        e = q.Engine(q.Config(N=N, L=L, dt=dt, precision=prec, potential=potential))
+        e.init([q.init_spec("gauss", 0.8, 1, 0, 0), q.init_spec("gauss", 0.8, 2, 1, 0)], 2, np.arange(2))
+        e.evolve([med], np.arange(2, dtype=np.uint64))
+        o = e.observables(check_finite=False)
+        torch.cuda.synchronize()
+        res.append(o if potential else e.nojump_results(2))   # (OQS: the groups' no-jump records)
+        e.close()
+    a, b = res
+    assert (a["norm2"] > 0).all() and a["norm2"].min() < 1e-45 and (a["n_steps_exec"] > 1000).all()
+    bound = 2 * fp32_bound(N, a["n_steps_exec"])
+    assert (np.abs(b["norm2"] / a["norm2"] - 1) <= bound).all(), (a["norm2"], b["norm2"])
+    top = a["surv"].max(1)
+    assert np.isfinite(b["surv"]).all() and (np.abs(b["surv"] - a["surv"]).max(1) <= bound * np.maximum(top, 0 if potential else 1)).all()
+
+
 @pytest.mark.parametrize("N,bound", [(256, 4.7e-15), (512, 9.4e-15), (2048, 3.1e-14)])
 def test_fp64_states_of_a_few_steps(q, N, bound):  # noqa: F811
     """Final states of four steps, no further from 64-bit arithmetic than a transform through one N-point FFT leaves
