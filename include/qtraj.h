@@ -64,8 +64,9 @@ typedef struct {
     int form;        /* qtraj_form */
     int save_states; /* 1: keep every final u(r) (FP64) in the workspace for qtraj_states()     */
     int variant;     /* fused kernel variant (FP32, N in {2048, 4096}; elsewhere the same as 0):
-                        0 = radix 16, 512 resident threads per SM; 1 = radix 16, 640; 2 = radix 8, 768;
-                        3 = radix 8, 1024                                                          */
+                        0 = radix 16, 512 resident threads per SM; 1 = radix 16, 640 (N = 2048; at N =
+                        4096 a CTA has 256 threads, of which 512 and 640 hold two: the same as 0);
+                        2 = radix 8, 768; 3 = radix 8, 1024                                        */
     double t_vacuum; /* >= 0, GeV^-1: vacuum evolution of every initial state before the medium
                         (Table 1: tmed - t0; Sec. 3.5 item 3): round(t_vacuum / dt) Strang steps
                         at T = 0 (Coulomb + centrifugal potential of the state's colour, no

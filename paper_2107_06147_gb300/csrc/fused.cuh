@@ -1389,8 +1389,8 @@ __device__ int fetch_trajectory(const Tables<T> &tb, const LaunchArgs &a)
 constexpr int fused_red = 8;   // sums reduced at once (slot_sums8)
 
 // Occupancy target of a kernel variant: variant 0 asks for 512 resident threads per SM in FP32
-// (<= 128 registers); variant 1 asks for 640 (<= 102 registers, at the price of spills), variants 2 and 3
-// (radix 8) for 768 and 1024.  FP64 holds twice the state and takes what the compiler needs.
+// (<= 128 registers); variant 1 asks for 640 (N = 2048: 5 CTAs of 128 threads, <= 102 registers, at the price of
+// spills; at N = 4096 640 threads hold the same two CTAs of 256), variants 2 and 3 (radix 8) for 768 and 1024.  FP64 holds twice the state and takes what the compiler needs.
 template <typename T, int N, int V> struct FusedBounds {
     static constexpr int G = FusedPlan<T, N, V>::G;
     static constexpr int THREADS = V == 1 ? 640 : V == 2 || V == 6 ? 768 : V == 3 ? 1024 : 512;

@@ -24,9 +24,8 @@ cudaError_t fused_launch_f32_b(int N, const Tables<float> &tb, const LaunchArgs 
                                   : a.trace_every > 0 ? fused_go<float, 2048, 4>(tb, a, sm_count, max_ctas, s, info, query_only)
                                   : fused_go<float, 2048, 0>(tb, a, sm_count, max_ctas, s, info, query_only);
         }
-    case 4096:
+    case 4096:   // (variant 1 is variant 0: FusedBounds)
         switch (variant) {
-        case 1: return fused_go<float, 4096, 1>(tb, a, sm_count, max_ctas, s, info, query_only);
         case 2: return fused_go<float, 4096, 2>(tb, a, sm_count, max_ctas, s, info, query_only);
         case 3: return fused_go<float, 4096, 3>(tb, a, sm_count, max_ctas, s, info, query_only);
         case 6: return fused_go<float, 4096, 6>(tb, a, sm_count, max_ctas, s, info, query_only);
