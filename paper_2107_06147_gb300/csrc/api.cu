@@ -494,18 +494,19 @@ template <typename T> qtraj_status build_tables(qtraj_ctx *c, cudaStream_t s)
             sp[t] = Prec<T>::make_r(std::sin(PI * (double)t / N));
             KT[t] = Prec<T>::make(kt[t].first * 2.0 / N, kt[t].second * 2.0 / N);
         }
-        // last-pass twiddles W^(m g) for m < R, g < G = N/(2R), one compact section [R][G] (N/2 entries)
-        // per radix R = 16, 8, 4: the threads of a warp read consecutive entries
-        std::vector<PC> WL((size_t)3 * (N / 2));
-        for (int sec = 0; sec < 3; ++sec) {
-            const int R = 16 >> sec, G = N / (2 * R);
-            for (int m = 0; m < R; ++m)
-                for (int g = 0; g < G; ++g) WL[(size_t)sec * (N / 2) + (size_t)m * G + g] = W[(size_t)m * g];
-        }
         qtraj_status st = QTRAJ_OK;
         if ((st = upload(&c->W, W)) != QTRAJ_OK || (st = upload(&c->KT, KT)) != QTRAJ_OK ||
-            (st = upload(&c->sinpre, sp)) != QTRAJ_OK || (st = upload(&c->WL, WL)) != QTRAJ_OK)
+            (st = upload(&c->sinpre, sp)) != QTRAJ_OK)
             return st;
+        if (const int R = ksu32_wl_radix(N)) {
+            // last-pass twiddles W^(m g) for m < R, g < G = N/(2R), [R][G]: the threads of a warp read consecutive
+            // entries
+            const int G = N / (2 * R);
+            std::vector<PC> WL((size_t)R * G);
+            for (int m = 0; m < R; ++m)
+                for (int g = 0; g < G; ++g) WL[(size_t)m * G + g] = W[(size_t)m * g];
+            if ((st = upload(&c->WL, WL)) != QTRAJ_OK) return st;
+        }
         return build_set<T>(c, c->fused, nullptr, coul, true, kt, s);
     }
     // a plain context runs the fused kernel only for the vacuum evolution of its initial states
@@ -1568,7 +1569,6 @@ extern "C" qtraj_status qtraj_evolve_static(qtraj_ctx *c, int batch, const qtraj
     ma.n_groups = n_groups;
     ma.gobs = ds->gobs;
     ma.gready = n_groups > 0 ? ds->gready : nullptr;   // (without groups the flags are an earlier call's)
-    FusedInfo fi;
     auto point = [&](auto tb) {
         tb.ic = ds->ic;
         tb.ic_cplx = 0;
@@ -1579,7 +1579,7 @@ extern "C" qtraj_status qtraj_evolve_static(qtraj_ctx *c, int batch, const qtraj
         tb.media = ds->media;
         return tb;
     };
-    if (c->p.precision == QTRAJ_FP32) CK(fused_launch_f32(N, point(tables<float>(c)), ma, c->sm_count, 0, s, &fi, false, c->p.variant));
-    else CK(fused_launch_f64(N, point(tables<double>(c)), ma, c->sm_count, 0, s, &fi, false, c->p.variant));
+    if (c->p.precision == QTRAJ_FP32) CK(fused_launch_f32(N, point(tables<float>(c)), ma, c->sm_count, 0, s, nullptr, false, c->p.variant));
+    else CK(fused_launch_f64(N, point(tables<double>(c)), ma, c->sm_count, 0, s, nullptr, false, c->p.variant));
     return QTRAJ_OK;
 }

@@ -368,7 +368,6 @@ template <typename T> __device__ __noinline__ T table_T3_far(const double *p, in
 // FP64: exp and sincospi; a rounding next to 1 is 1e-16 there and does not matter.
 template <typename T> struct Dyn;
 // the rare points outside the series' ranges, kept out of line so the hot loop stays small
-static __device__ __noinline__ float em1_far(float a) { return expf(a) - 1.0f; }
 static __device__ __noinline__ void dyn_far(float a, float y, float *em1, float *s, float *cm1)
 {
     *em1 = expf(a) - 1.0f;
@@ -383,23 +382,7 @@ template <> struct Dyn<float> {
     {
         f1t(a, 3.14159265358979f * y, fr, fi, e);
     }
-    // exp(a) - 1 alone (the phase-free factor), the same series and range as f1t
-    static __device__ __forceinline__ float em1(float a)
-    {
-        if (a >= -0.5f) {
-            float p = 1.0f / 40320.0f;
-            p = fmaf(p, a, 1.0f / 5040.0f);
-            p = fmaf(p, a, 1.0f / 720.0f);
-            p = fmaf(p, a, 1.0f / 120.0f);
-            p = fmaf(p, a, 1.0f / 24.0f);
-            p = fmaf(p, a, 1.0f / 6.0f);
-            p = fmaf(p, a, 0.5f);
-            p = fmaf(p, a, 1.0f);
-            return a * p;
-        }
-        return em1_far(a);
-    }
-    // the same from the phase t = pi y (the hot loop forms t directly; beyond the series' range y is
+    // f1 from the phase t = pi y (the hot loop forms t directly; beyond the series' range y is
     // recomputed from t)
     static __device__ __forceinline__ void f1t(float a, float t, float *fr, float *fi, float *e)
     {
@@ -436,7 +419,7 @@ template <> struct Dyn<float> {
         *e = em1;
     }
     // both points of a pair at once in packed FP32x2 instructions, the same operations per component
-    // as f1t / em1 (bit-identical), for arguments in the series' range
+    // as f1t (bit-identical), for arguments in the series' range
     static __device__ __forceinline__ float2 rep(float v) { return make_float2(v, v); }
     static __device__ __forceinline__ float2 em1_2(float2 a)
     {

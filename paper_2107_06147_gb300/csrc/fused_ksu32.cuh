@@ -26,7 +26,7 @@ template <int N> struct NftPlan {
     // radix 8 up to N = 2048 (passes 8, 16, 8 at N = 1024 and 8, 16, 2, 8 at 2048: +9% each over
     // radix 16's 16, 4, 16 and 16, 8, 16, whose short middle passes and small CTAs cost more
     // instructions per point), 16 above
-    static constexpr int R = (N <= 32) ? 4 : (N <= 2048) ? 8 : 16;
+    static constexpr int R = ksu32_radix(N);
     static constexpr int G = N / (2 * R);        // threads per trajectory
     static constexpr int NR = N / R;             // stride of a first/last-pass butterfly
     static constexpr int MID = N / (R * R);      // product of the middle radices
@@ -259,10 +259,10 @@ template <int N> struct NftSine {
             cpx<T> v1 = buf[pad(b_of(g, 0) + m * NR)];
             cpx<T> v2 = buf[pad(b_of(g, 1) + m * NR)];
             if (m) {
-                // W^(m g): up to N = 2048 from the radix's compact [m][g] section (a warp reads
+                // W^(m g): up to N = 2048 from the compact [m][g] table (a warp reads
                 // consecutive entries; measured +3% at N = 1024, +6.5% at 2048), above from the
                 // strided W[m g] (the compact table measured 9% slower at N = 4096, 1% at 16384)
-                const C w = N <= 2048 ? PR::ld(&tb.WL[(R == 16 ? 0 : R == 8 ? N / 2 : N) + m * G + g])
+                const C w = ksu32_wl_radix(N) ? PR::ld(&tb.WL[m * G + g])
                                       : PR::ld(&tb.W[m * g]);
                 v1 = cmul(v1, w);
                 if (g != 0) {

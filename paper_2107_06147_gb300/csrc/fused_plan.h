@@ -103,6 +103,11 @@ __host__ __device__ __forceinline__ void plan_entry(int i, bool adjacent, int R,
     e = t * R + (h ? R - 1 - m : m);
 }
 
+// The FP32 KSU kernel's radix (fused_ksu32.cuh), and the radix of its compact last-pass twiddle table, which it reads up
+// to N = 2048 (0: none)
+__host__ __device__ constexpr int ksu32_radix(int N) { return N <= 32 ? 4 : N <= 2048 ? 8 : 16; }
+__host__ __device__ constexpr int ksu32_wl_radix(int N) { return N <= 2048 ? ksu32_radix(N) : 0; }
+
 // host view of a plan
 struct Plan {
     int N, R, E, M, M1, M2, G, S, NS;

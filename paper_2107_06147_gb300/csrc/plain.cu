@@ -8,11 +8,6 @@ namespace {
 
 constexpr int PB = 256; // threads of the per-trajectory kernels
 
-__device__ __forceinline__ bool running(const PlainState &s, const TrajDev &d, int n)
-{
-    return s.active && n < d.n_steps;
-}
-
 // the state's layout (PlainBuffers): grid point of the value at i, and its sign
 struct Order {
     int R, M, G;
@@ -169,7 +164,7 @@ __global__ void __launch_bounds__(PB) plain_jump(Tables<double> tb, LaunchArgs a
     const int b = blockIdx.x;
     const TrajDev d = a.trajs[b];
     PlainState s = st[b];
-    if (!running(s, d, n)) return;
+    if (!plain_running(s, d, n)) return;
     __shared__ double sh[PB / 32];
     cpx<double> *p = psi + (size_t)b * N;
     double n2 = 0.0;

@@ -18,6 +18,11 @@ struct PlainState {
     uint32_t digest;   // jump digest (qtraj_obs.jump_digest)
 };
 
+__device__ __forceinline__ bool plain_running(const PlainState &s, const TrajDev &d, int n)
+{
+    return s.active && n < d.n_steps;
+}
+
 struct PlainBuffers {
     cpx<double> *psi;        // [n_traj][N] states: value e of thread g at e G + g, with the odd extension's sign
     cpx<double> *sa, *sb;    // [n_traj][plain_seq(N)] the exchange arrays of the two transforms

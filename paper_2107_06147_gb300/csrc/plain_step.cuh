@@ -10,11 +10,6 @@
 
 namespace qt {
 
-__device__ __forceinline__ bool plain_running(const PlainState &s, const TrajDev &d, int n)
-{
-    return s.active && n < d.n_steps;
-}
-
 template <int N> struct PlainStep {
     using P = FusedPlan<double, N, 7>;
     using K = Sine<double, N, 7>;

@@ -88,7 +88,6 @@ template <> struct Prec<double> {
     static __device__ __forceinline__ C ld(const C *p) { return ldg(p); }
     static __device__ __forceinline__ Rl re(C w) { return w.x; }
     static __device__ __forceinline__ Rl im(C w) { return w.y; }
-    static __device__ __forceinline__ C from_double(double re, double im) { return {re, im}; }
     // static potential factors (tables of exp(-i V_static dt/2), exp(-i V_static dt)): one double each
     using S = cpx<double>;
     static __host__ __device__ S make_s(double re, double im) { return {re, im}; }
@@ -148,11 +147,6 @@ template <> struct Prec<float> {
     }
     static __device__ __forceinline__ Rl re(C w) { return {w.rh, w.rl}; }
     static __device__ __forceinline__ Rl im(C w) { return {w.ih, w.il}; }
-    static __device__ __forceinline__ C from_double(double re, double im)
-    {
-        const float rh = (float)re, ih = (float)im;
-        return {rh, ih, (float)(re - (double)rh), (float)(im - (double)ih)};
-    }
     // The static potential factors are the one family of constants kept without low parts: the
     // paired FP32/FP64 study measured no loss from rounding them (ensemble errors 1.6e-6 / 1.1e-5 at
     // N = 4096 / 8192 against 2.6e-6 / 4.2e-6 with hi+lo; median norm error 6.7e-7 against 5.3e-7),
@@ -441,7 +435,7 @@ template <typename T> struct Tables {
     using C = typename Prec<T>::C;
     // FP32 KSU kernel, natural order
     const C *W;                        // N twiddles exp(-2 pi i t / N)
-    const C *WL;                       // last-pass twiddles W^(m g): sections [R][N/(2R)] for R = 16, 8, 4
+    const C *WL;                       // last-pass twiddles W^(m g), [R][N/(2R)] (ksu32_wl_radix)
     const C *KT;                       // N kinetic factors exp(-i T_kin(p_k) dt) * 2/N, k = 0..N-1
     const typename Prec<T>::Rl *sinpre; // N values sin(pi j / N)
     // both forms, in the order of the kernels' threads (fused_plan.h)
