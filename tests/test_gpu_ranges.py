@@ -159,3 +159,41 @@ def test_repeated_evolves_do_not_wait_for_the_first(q):  # noqa: F811
     e.close()
     assert running
     assert np.array_equal(a["jump_digest"], b["jump_digest"]) and np.array_equal(a["norm2"], b["norm2"])
+
+
+@pytest.mark.parametrize("N,variant", [(2048, 2), (4096, 3)])
+def test_vacuum_evolution_under_the_radix_8_variants(q, N, variant):  # noqa: F811
+    import oracle as o
+    from paper_2107_06147_gb300 import inputs
+    w = inputs.small_parity(N=N, n_traj=4, seed=35)
+    for m in w.media:
+        m.Tf = 0.99 * m.T0
+    g, inits, media = oracle_inputs(w)
+    g.t_vac, g.use_rmin = 0.05, 0
+    ref, _, uref = o.run_batch(g, inits, w.init_idx, media, w.medium_idx, w.seeds, want_states=True)
+    obs, u = run_gpu(q, w, q.FP32, t_vacuum=0.05, variant=variant, use_rmin=0)
+    check_fp32(q, obs, ref, u, uref, min_same=0.75)
+
+
+@pytest.mark.parametrize("N", [16, 128, 512, 2048, 4096, 8192])
+def test_ksu_fp64_plans(q, N):  # noqa: F811
+    """The FP64 KSU kernel on the plans that test_gpu_ksu leaves out, 1e-10 as there."""
+    import oracle as o
+    from oracle import eigen
+    import torch
+    g = o.Grid(N=N, L=12.0, dt=0.001, potential=1, use_rmin=0)
+    e = q.Engine(q.Config(N=N, L=12.0, dt=0.001, precision=q.FP64, potential=1, save_states=1))
+    states, T = [("gauss", 0.3, 1, 0, 0), ("gauss", 0.5, 2, 1, 0)], (0.4, 0.6, 0.396)
+    g.basis = eigen.numerical_basis(g) if N <= 512 else e.basis()   # (the dense eigensolver of larger grids takes minutes)
+    idx = np.arange(2, dtype=np.int32)
+    ref, _, uref = o.run_batch(g, [o.init_spec(*s) for s in states], idx, [o.medium(*T, 0.0, 0.0)], np.zeros(2, np.int32),
+                               np.arange(2, dtype=np.uint64), want_states=True)
+    e.init([q.init_spec(*s) for s in states], 2, idx)
+    e.evolve([q.medium(*T, 0.0, 0.0)], np.arange(2, dtype=np.uint64), np.zeros(2, np.int32))
+    obs, u = e.observables(), e.states()
+    torch.cuda.synchronize()
+    e.close()
+    assert (ref["n_steps_exec"] > 10).all() and np.array_equal(obs["n_steps_exec"], ref["n_steps_exec"])
+    assert (np.linalg.norm(u - uref, axis=1) <= 1e-10 * np.linalg.norm(uref, axis=1)).all()
+    assert (np.abs(obs["norm2"] / ref["norm2"] - 1) <= 1e-10).all()
+    assert (np.abs(obs["surv"] - ref["surv"]).max(1) <= 1e-10 * np.maximum(1, ref["surv"].max(1))).all()
