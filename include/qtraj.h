@@ -204,8 +204,8 @@ typedef struct {
  * rows (the evolve clears d_counts[0 .. n_traced) first).  Both are caller device buffers that must
  * stay valid while those evolves run.  A trajectory resolved without evolving (rMin shortcut,
  * r_max) writes no row.  Fused form only (EINVAL for the plain form); while it is on, evolves run a
- * traced copy of the fused kernel (variant 0's plan), which at each recorded step of a traced
- * trajectory makes one more pass over the state per quantity. */
+ * traced copy of the fused kernel (on the plan of the context's variant), which at each recorded step
+ * of a traced trajectory makes one more pass over the state per quantity. */
 qtraj_status qtraj_set_trace(qtraj_ctx *ctx, int every, int n_traced, int max_records, qtraj_trace_rec *d_records,
                              int *d_counts);
 

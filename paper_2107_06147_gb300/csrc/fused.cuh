@@ -97,11 +97,11 @@ __device__ __forceinline__ DF df_add(DF a, DF b)
 template <typename T> struct SqAcc;
 template <> struct SqAcc<float> {
     DF v{0.f, 0.f};
-    // v += w |a|^2 in plain FP32: a thread sums its ~N/G terms of one parity (16 at N = 4096), a
-    // relative error of ~sqrt(16) x 6e-8 = 2.4e-7, random from step to step; the sums of the threads
-    // are then combined in double-float.  The norm feeds only the waiting-time comparison and the
-    // jump's renormalisation, and the FP32 state's own norm error is ~1e-6 per hundred steps, so a
-    // compensated per-thread sum (as an earlier revision had) buys nothing the comparison can see.
+    // v += w |a|^2 in plain FP32: a thread sums its E values in two chains (8 terms each at N = 4096), a
+    // relative error of ~sqrt(8) x 6e-8 = 1.7e-7, random from step to step; the sums of the chains and
+    // threads are then combined in double-float.  The norm feeds only the waiting-time comparison and the
+    // jump's renormalisation, and the FP32 state's own norm is 0.4 .. 1.4e-6 off after 64 .. 300 steps, so
+    // a compensated per-thread sum (as an earlier revision had) buys nothing the comparison can see.
     __device__ __forceinline__ void add_w(cpx<float> a, float w) { v.hi = fmaf(w, fmaf(a.x, a.x, a.y * a.y), v.hi); }
     __device__ __forceinline__ void shfl_add(unsigned mask, int off, int w)
     {
@@ -924,10 +924,11 @@ template <typename T, int N, int V> struct Sine {
 };
 
 // ------------------------------------------------------------------------------------------------
-// pointwise work.  The common step's factor and norm act on the registers (factor_regs).  Everything
-// rarer -- the first and last half-steps, jumps, caps, summary rows, rows beyond the static table, the KSU
-// factor and the read-out -- works on a copy of the registers in shared memory, element e of thread g at
-// e G + g, in loops over e: a thread only touches its own elements, and the step's code stays short.
+// pointwise work.  The step's factor and norm act on the registers (factor_regs), the first and last half-steps
+// of a trajectory too.  Everything rarer -- jumps, caps, summary rows, rows beyond the static table, phases beyond
+// 1e5, temperatures that change too much within a step, the FP64 KSU factor and the read-out -- works on a copy of
+// the registers in shared memory, element e of thread g at e G + g, in loops over e: a thread only touches its own
+// elements, and the step's code stays short.
 // Values carry the odd extension's sign (fused_plan.h).
 // ------------------------------------------------------------------------------------------------
 template <typename T, int N, int V> struct Pointwise {
@@ -965,9 +966,10 @@ template <typename T, int N, int V> struct Pointwise {
         for (int e = 0; e < E; ++e) x[e] = buf[e * G + g];
     }
 
-    // The dynamic factor exp(a) exp(i pi y) is close to 1 and changes little from step to step; it is applied
+    // The dynamic factor exp(a) exp(i pi y) is close to 1 and changes little from step to step; FP32 applies it
     // as w + w f1 with f1 its deviation from 1, evaluated so that the rounding is relative to f1, not to 1 (a
-    // rounding of a value next to 1 would repeat identically every step and add up).
+    // rounding of a value next to 1 would repeat identically every step and add up).  In FP64 a rounding next to 1 does
+    // not matter: factor() shares this form, factor_regs multiplies by the factor itself.
     static __device__ __forceinline__ cpx<T> apply(cpx<T> w, T f1r, T f1i)
     {
         if constexpr (sizeof(T) == 4) return mk(fmaf(w.x, f1r, fmaf(-w.y, f1i, w.x)), fmaf(w.y, f1r, fmaf(w.x, f1i, w.y)));

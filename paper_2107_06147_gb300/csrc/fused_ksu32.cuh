@@ -1,10 +1,11 @@
 // fused_ksu32.cuh -- the FP32 kernel of the isotropic KSU potential (App. E; no jumps): one CTA evolves one
 // trajectory, its wave function in shared memory for its whole life, as fused.cuh's kernel does, with the
 // sine transform taken through one N-point FFT with sine pre- and post-processing and a compensated prefix
-// sum.  fused.cuh's transform is faster and more accurate, but the KSU survival ratios are referred to the
-// overlaps of the initial state with the Cornell basis, and where one of these nearly vanishes the ratio
-// magnifies the two transforms' FP32 difference past 2e-5 of the records (25% of Gaussian widths in 0.7 ..
-// 0.9 GeV^-1 on N = 4096, 16 steps): results stay those of this transform.
+// sum.  fused.cuh's transform is faster and more accurate.  It is not taken here yet because it would move results:
+// the KSU survival ratios are referred to the overlaps of the initial state with the Cornell basis, and where one
+// of these nearly vanishes the ratio magnifies the two transforms' FP32 difference, to more than 2e-5 of a batch's ratios
+// (relative 2-norm) for 25% of Gaussian widths in 0.7 .. 0.9 GeV^-1 on N = 4096, 16 steps, while states and
+// overlaps differ by no more than this transform's own error there, 1e-5.
 //
 // The DST-I of the N-point complex vector f (f_0 = f_N = 0) is computed with one N-point complex FFT:
 //   y_j = sin(pi j/N)(f_j + f_{N-j}) + (f_j - f_{N-j})/2,   Y = FFT_N(y),

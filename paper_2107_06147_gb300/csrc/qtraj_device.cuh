@@ -66,11 +66,11 @@ __device__ __forceinline__ cpx<double> ldg(const cpx<double> *p)
     return {v.x, v.y};
 }
 // ------------------------------------------------------------------------------------------------
-// constant multipliers.  In FP32 every constant of the step (twiddles, in-register DFT constants,
-// sine pre-factors, kinetic and potential phase tables) is carried as an unevaluated sum hi + lo of
-// two floats: the rounding of a constant is the same in every step and would otherwise accumulate
-// coherently over 10^4 steps, while the rounding of data is random and grows only as a square root.
-// In FP64 a constant is one double.
+// constant multipliers.  The rounding of a constant is the same in every step and accumulates coherently over
+// 10^4 steps, while the rounding of data is random and grows only as a square root.  So the FP32 constants of the
+// transforms and the kinetic factors carry more than 24 bits: complex ones as directions (Prec<float>::D, 2^-35), real
+// ones, and all of the FP32 KSU kernel's, as unevaluated sums hi + lo of two floats (2^-48).  The static potential
+// rows are single floats.  In FP64 a constant is one double.
 // ------------------------------------------------------------------------------------------------
 template <typename T> struct Prec;
 template <> struct Prec<double> {
